@@ -125,6 +125,11 @@ def algorithmic_bytes_per_iteration(n, n_x, n_u, n_v, prec):
 
 STAGES = {1: ["apg_iter"], 2: ["fwd_scan", "prox_node", "scan_s", "node_mv_gt", "scan_r", "node_mv_dh"],
           3: ["fwd_scan", "prox_node", "apg_iter_gt", "node_mv_dh"], 4: ["fwd_scan", "prox_node", "apg_iter_bwd"]}
+SWEEP_STAGES = ["tree_sweep", "lambda_apply"]  # the two-launch form of schedule 4 (sparse [Bbar; L])
+
+
+def stages_of(schedule, stage_ms):
+    return SWEEP_STAGES if schedule == 4 and len(stage_ms) == 2 else STAGES[schedule]
 
 
 def stage_bytes(stage, n, n_x, n_u, n_v, prec, shared):
@@ -141,6 +146,13 @@ def stage_bytes(stage, n, n_x, n_u, n_v, prec, shared):
         return n * ((0 if shared else n_k * n_v * ms) + (n_k + n_x + 2 * n_v) * vs)
     if stage == "node_mv_dh":
         return n * ((0 if shared else (n_k * n_v + n_v * n_v) * ms) + (n_v + n_k) * vs)
+    if stage == "tree_sweep":
+        # delta (n_v), e and u_hat (n_k), steps, reciprocals and mu in; u, x (n_k) and r (n_v) out;
+        # beta in; the dual state of two iterates in and one out (8 bytes an entry)
+        return n * ((3 * n_v + 2 * n_k + 2 * (n_u + 2) + 1) * vs + 3 * 8 * (2 * n_x + n_u))
+    if stage == "lambda_apply":
+        # one half of the symmetric Lambda of every node; r in, delta out
+        return n * ((0 if shared else n_v * (n_v + 1) // 2 * ms) + 2 * n_v * vs)
     if stage == "apg_iter_bwd":
         # the whole backward sweep with each pack read once: [Bbar; L] and Lambda per node;
         # w (n_k) and beta (n_v) in, h (n_k) out, s and r published (n_x + n_v)
@@ -157,6 +169,8 @@ def stage_flops(stage, n, n_x, n_u, n_v):
         return n * 2 * (n_k * n_v + n_v * n_v)
     if stage == "apg_iter_bwd":
         return n * 2 * (2 * n_k * n_v + n_v * n_v)
+    if stage == "lambda_apply":
+        return n * 2 * n_v * n_v
     return None
 
 
@@ -410,7 +424,7 @@ def kernel_roofline(S, P, prec, inp, stream, fp64_peak, iters=200):
     host = {k: v.cpu().numpy() for k, v in inp.items()}
     stage_ms = S.smpc.smpc_profile_solve(S.fac, host["p"], host["q"], host["dhat"], host["alpha2"], eps=P["eps"],
                                          iters=iters)
-    names = STAGES[S.schedule]
+    names = stages_of(S.schedule, stage_ms)
     hbm, src = peaks()
     if S.schedule == 1:
         kern, k_ms, k_bytes = "apg_iter", stage_ms[0], nbytes

@@ -122,7 +122,10 @@ typedef struct smpc_factor_opts {
    * pass up to r, and the node-parallel Lambda / [Bbar; L] launch; 4 = node-parallel forward
    * sweep and prox, then the whole backward sweep as one chain pass (every pack read once
    * per iteration); 0 = time all of them on this GPU when the factor is built and keep the
-   * fastest.  Results agree to rounding. */
+   * fastest.  Where [Bbar; L] is sparse (at most 4096 entries in the reduced basis, A = I,
+   * float64 or float32) 0 also times a two-launch form of 4 - a tree pass with the sparse
+   * products inside, and Lambda r of every node - which is reported as 4.  Results agree to
+   * rounding. */
   int32_t schedule;
   /* SMPC_BF16 with shared_packs = 1: the Lambda and [Bbar; L] products of the delta
    * iterations (and, on the node-parallel schedule 2, their [Bbar; L]' products) run on the
@@ -217,7 +220,9 @@ int smpc_tree_info_get(const smpc_tree* tree, smpc_tree_info* info);
 void smpc_tree_destroy(smpc_tree* tree);
 
 /* Offline factor step (App. A and App. B; Alg. 2 lines 1-2), in float64 on the
- * host: L = orthonormal basis of null(E), B_bar = B L, R_hat = W_u L,
+ * host: L = basis of null(E) (orthonormal; in float64 and float32 factors the reduced one
+ * [-E1^{-1} E2; I] where its entries stay within 4, since it keeps a network's incidence
+ * structure; u, x and y do not depend on the basis), B_bar = B L, R_hat = W_u L,
  * R_bar = L' R_hat, Cholesky of R_bar, Lambda = -R_bar^{-1}; then per-node packs
  * [B_bar; L] (n_x + n_u) x n_v and Lambda / (2 p_n) (n_v x n_v, Alg. 1's
  * node-indexed factor matrices) in the requested precision on the device, the
@@ -345,7 +350,8 @@ void smpc_shard_destroy(smpc_shard* shard);
  * [Bbar; L]' mat-vec, subtree scan of r, Lambda and [Bbar; L] mat-vecs) and 4 for schedule 3
  * (forward sweep; prox and dual update; s, [Bbar; L]' mat-vecs and r along the chains; Lambda
  * and [Bbar; L] mat-vecs) and 3 for schedule 4 (forward sweep; prox and dual update; the
- * whole backward sweep along the chains).  SMPC_BF16 anchor iterations are not timed.  Leaves
+ * whole backward sweep along the chains; n = 2 for its two-launch form: tree pass; Lambda r).
+ * SMPC_BF16 anchor iterations are not timed.  Leaves
  * the factor's duals as that solve ends.  Returns n, or minus an smpc_status. */
 int smpc_profile_solve(smpc_factor_t* fac, const smpc_step_data* data, int32_t iters, double* stage_ms,
                        int32_t max_stages);

@@ -78,7 +78,8 @@ bool finite_if_host(const double* p, size_t n) { return !host_readable(p) || fin
 
 void free_tree_dev(smpc::DevTree& d) {
   void* ptrs[] = {d.parent, d.stage, d.child_begin, d.child_count, d.chain_off, d.chain_node, d.chain_parent,
-                  d.top_nodes, d.top_expect, d.path_off, d.path_node, d.tree_of, d.row, d.seg, d.prob, d.pbar};
+                  d.top_nodes, d.top_expect, d.path_off, d.path_node, d.tree_of, d.row, d.seg, d.prob, d.pbar,
+                  d.top_src_off, d.top_src};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   d = smpc::DevTree();
@@ -222,6 +223,38 @@ int build_tree(int32_t n, const int32_t* parent, const double* prob, smpc_tree& 
     }
   }
   t.path_off[n] = (int)t.path_node.size();
+  // Per top node t the chain heads below it, then the top nodes below it and itself, each with
+  // the number of top nodes from t down to its parent (a top node: itself included), which is
+  // how often its xi counts in t's sums of s.  No lists (SCHED_SWEEP does not run) beyond
+  // kMaxTopSrc entries, which only deep trees that branch at every stage reach.
+  constexpr size_t kMaxTopSrc = size_t(1) << 24;
+  {
+    std::vector<int> index(n, -1);
+    for (size_t i = 0; i < t.top_nodes.size(); ++i) index[t.top_nodes[i]] = (int)i;
+    std::vector<size_t> cnt(2 * t.top_nodes.size() + 1, 0);
+    auto visit = [&](auto&& f) {  // f(list, node, weight)
+      for (size_t c = 0; c + 1 < t.chain_off.size(); ++c) {
+        const int h = t.chain_node[t.chain_off[c]];
+        for (int k = parent[h]; k >= 0; k = parent[k]) f(2 * index[k], h, t.stage[h] - t.stage[k]);
+      }
+      for (int m : t.top_nodes)
+        for (int k = m; k >= 0; k = parent[k]) f(2 * index[k] + 1, m, t.stage[m] - t.stage[k] + 1);
+    };
+    size_t total = 0;
+    visit([&](int list, int, int) { ++cnt[list + 1], ++total; });
+    t.top_src_off.clear();
+    t.top_src.clear();
+    if (total <= kMaxTopSrc) {
+      for (size_t i = 1; i < cnt.size(); ++i) cnt[i] += cnt[i - 1];
+      t.top_src_off.assign(cnt.begin(), cnt.end());
+      t.top_src.resize(2 * total);
+      visit([&](int list, int m, int w) {
+        const size_t q = cnt[list]++;
+        t.top_src[2 * q] = m;
+        t.top_src[2 * q + 1] = w;
+      });
+    }
+  }
   const int n_seg = (int)(t.top_nodes.size() + t.chain_parent.size());
   t.seg.assign((size_t)n_seg * smpc::kSegInts, 0);
   for (int b = 0; b < n_seg; ++b) {
@@ -256,6 +289,8 @@ int upload_tree(smpc_tree& t) {
   TRY(dev_upload(&d.tree_of, t.tree_of.data(), t.n));
   TRY(dev_upload(&d.row, t.row.data(), t.n));
   TRY(dev_upload(&d.seg, t.seg.data(), t.seg.size()));
+  TRY(dev_upload(&d.top_src_off, t.top_src_off.data(), t.top_src_off.size()));
+  TRY(dev_upload(&d.top_src, t.top_src.data(), t.top_src.size()));
   TRY(dev_upload(&d.prob, t.prob.data(), t.n));
   TRY(dev_upload(&d.pbar, t.pbar.data(), t.n));
   return SMPC_OK;
@@ -264,6 +299,19 @@ int upload_tree(smpc_tree& t) {
 }  // namespace
 
 // smpc_factor_t is defined in smpc_internal.h
+
+namespace smpc {
+void set_sweep_args(const smpc_factor_t* f, IterArgs& a) {
+  const smpc_tree* t = f->tree;
+  a.sp = t->top_src_off.empty() ? nullptr : f->sp;
+  a.sp_nnz = f->sp_nnz;
+  a.depth = t->N;
+  a.lam = f->lam;
+  a.lam_stride = f->shared_packs ? 0 : lam_pack_entries(f->n_v);
+  a.top_src_off = t->dev.top_src_off;
+  a.top_src = t->dev.top_src;
+}
+}  // namespace smpc
 
 namespace {
 
@@ -329,6 +377,7 @@ IterArgs make_args(const smpc_factor_t* f) {
   a.R = f->R;
   a.res_tree = f->res_tree;  // NULL for a single tree
   a.tree_done = f->tree_done;
+  set_sweep_args(f, a);
   return a;
 }
 
@@ -501,9 +550,9 @@ int choose_schedule(smpc_factor_t* f, int requested) {
     a.wa = f->wa;
   }
   const int mode_extra = anchored ? MODE_DELTA : 0;
-  bool fits[kSchedules + 1] = {};
+  bool fits[SCHED_SWEEP + 1] = {};
   int n_fit = 0, only = SCHED_CHAIN;
-  for (int s = 1; s <= kSchedules; ++s) {
+  for (int s = 1; s <= SCHED_SWEEP; ++s) {
     fits[s] = iter_config(f->prec, a, f->num_sms, s).stages > 0;
     if (fits[s]) {
       ++n_fit;
@@ -528,7 +577,7 @@ int choose_schedule(smpc_factor_t* f, int requested) {
   CK(cudaEventCreate(&e1));
   float best = -1;
   constexpr int kWarm = 2, kTimed = 6;
-  for (int s = 1; s <= kSchedules; ++s) {
+  for (int s = 1; s <= SCHED_SWEEP; ++s) {
     if (!fits[s]) continue;
     const LaunchCfg cfg = iter_config(f->prec, a, f->num_sms, s);
     int rc = SMPC_OK;
@@ -880,7 +929,9 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   f->n_u = n_u;
   f->n_d = n_d;
   f->n_e = n_e;
-  int rc = host_factor(*net, cost->W_u, f->hf);
+  // A bfloat16 factor keeps the orthonormal basis: its entries are rounded to 8 bits, and the
+  // orthonormal one has no large entries to round.
+  int rc = host_factor(*net, cost->W_u, f->hf, f->prec != SMPC_BF16);
   if (rc != SMPC_OK) return fail(rc);
   const int n_v = f->hf.n_v;
   f->n_v = n_v;
@@ -943,6 +994,20 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
     const size_t hb = sizeof(float) * (size_t)n * n_k;
     if ((rc = f->alloc(&f->ha, hb)) || (rc = f->alloc(&f->wa, hb))) return fail(rc);
     if (cudaMemset(f->ha, 0, hb) != cudaSuccess || cudaMemset(f->wa, 0, hb) != cudaSuccess) return fail(SMPC_ECUDA);
+  }
+  // ---- the two-launch form of schedule 4: only a factor that may choose its schedule
+  const size_t lam_bytes = (size_t)np * lam_pack_entries(n_v) * f->vs;
+  if (o.schedule == 0 && f->prec != SMPC_BF16 && !general_A && !tree->top_src_off.empty()) {
+    for (double v : K) f->sp_nnz += v != 0.0;
+    if (f->sp_nnz <= kSparseMax) {
+      const std::vector<unsigned char> image = sparse_image(f->prec, n_k, n_v, K.data());
+      if ((rc = f->alloc(&f->sp, image.size()))) return fail(rc);
+      if (cudaMemcpy(f->sp, image.data(), image.size(), cudaMemcpyHostToDevice) != cudaSuccess) return fail(SMPC_ECUDA);
+      // without room for it the other schedules run as before
+      if (f->alloc(&f->lam, lam_bytes) == SMPC_OK &&
+          (rc = launch_lam_pack(f->prec, np, n_v, f->Lam64, pprob, f->lam, nullptr)))
+        return fail(rc);
+    }
   }
   // ---- vectors
   const size_t vs = f->vs;
@@ -1094,6 +1159,10 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   }
   if ((rc = choose_schedule(f, o.schedule))) return fail(rc);
   if ((rc = tune_tc(f, o.tc_width))) return fail(rc);
+  if (f->lam && f->schedule != SCHED_SWEEP) {  // not chosen: its matrices go
+    f->release(f->lam, lam_bytes);
+    f->lam = nullptr;
+  }
   *out = f;
   return SMPC_OK;
 }
@@ -1111,9 +1180,10 @@ int smpc_factor_schedule(const smpc_factor_t* f, double* ms_per_iter) {
     ms_per_iter[0] = f->tuned_ms[SCHED_CHAIN];
     ms_per_iter[1] = f->tuned_ms[SCHED_NODE];
     ms_per_iter[2] = f->tuned_ms[SCHED_HYBRID];
-    ms_per_iter[3] = f->tuned_ms[SCHED_FUSED];
+    const float sw = f->tuned_ms[SCHED_SWEEP];  // its two-launch form, where that was timed and is faster
+    ms_per_iter[3] = sw > 0 && sw < f->tuned_ms[SCHED_FUSED] ? sw : f->tuned_ms[SCHED_FUSED];
   }
-  return f->schedule;
+  return f->schedule == SCHED_SWEEP ? (int)SCHED_FUSED : f->schedule;
 }
 
 int smpc_factor_tc_width(const smpc_factor_t* f, double* ms_per_width) {

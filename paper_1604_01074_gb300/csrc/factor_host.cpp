@@ -95,9 +95,63 @@ void householder_q(std::vector<double> M, int rows, int cols, std::vector<double
   }
 }
 
+// A basis of null(E) in reduced form: with E column-permuted to [E1 E2], E1 square, the rows
+// of the basis are those of -E1^{-1} E2 for E1's columns and unit rows for the others.  For an
+// incidence matrix it is sparse (a junction's balance solved for one of its actuators), and so
+// is B L.  Gauss-Jordan elimination with complete pivoting, ties towards the column with the
+// fewest entries.  False (L untouched) when an entry of -E1^{-1} E2 exceeds 4: the basis could
+// then be worse conditioned than the orthonormal one by more than rounding forgives.
+bool reduced_null_basis(const double* E, int n_e, int n_u, std::vector<double>& L) {
+  std::vector<double> M(E, E + (size_t)n_e * n_u);
+  std::vector<int> piv(n_e, -1), used(n_u, 0), count(n_u, 0);
+  for (int i = 0; i < n_e; ++i)
+    for (int j = 0; j < n_u; ++j) count[j] += E[(size_t)i * n_u + j] != 0.0;
+  for (int step = 0; step < n_e; ++step) {
+    int pi = -1, pj = -1;
+    double best = 0;
+    for (int i = 0; i < n_e; ++i)
+      if (piv[i] < 0)
+        for (int j = 0; j < n_u; ++j) {
+          const double v = std::fabs(M[(size_t)i * n_u + j]);
+          if (used[j] || v == 0) continue;
+          if (v > best * (1 + 1e-9) || (v > best * (1 - 1e-9) && count[j] < count[pj])) {
+            best = std::fmax(best, v);
+            pi = i;
+            pj = j;
+          }
+        }
+    if (pi < 0) return false;
+    piv[pi] = pj;
+    used[pj] = 1;
+    const double d = 1.0 / M[(size_t)pi * n_u + pj];
+    for (int j = 0; j < n_u; ++j) M[(size_t)pi * n_u + j] *= d;
+    M[(size_t)pi * n_u + pj] = 1.0;
+    for (int i = 0; i < n_e; ++i) {
+      const double f = M[(size_t)i * n_u + pj];
+      if (i == pi || f == 0) continue;
+      for (int j = 0; j < n_u; ++j) M[(size_t)i * n_u + j] -= f * M[(size_t)pi * n_u + j];
+      M[(size_t)i * n_u + pj] = 0.0;
+    }
+  }
+  const int n_v = n_u - n_e;
+  std::vector<double> B((size_t)n_u * n_v, 0.0);
+  for (int j = 0, k = 0; j < n_u; ++j) {
+    if (used[j]) continue;
+    B[(size_t)j * n_v + k] = 1.0;
+    for (int i = 0; i < n_e; ++i) {
+      const double v = M[(size_t)i * n_u + j];
+      if (!(std::fabs(v) <= 4.0)) return false;
+      if (std::fabs(v) > 1e-15) B[(size_t)piv[i] * n_v + k] = -v;  // cancellations leave some 1e-16
+    }
+    ++k;
+  }
+  L = B;
+  return true;
+}
+
 }  // namespace
 
-int host_factor(const smpc_network& net, const double* W_u, HostFactor& f) {
+int host_factor(const smpc_network& net, const double* W_u, HostFactor& f, bool reduced_basis) {
   const int n_x = net.n_x, n_u = net.n_u, n_d = net.n_d, n_e = net.n_e;
   f.n_x = n_x;
   f.n_u = n_u;
@@ -127,6 +181,7 @@ int host_factor(const smpc_network& net, const double* W_u, HostFactor& f) {
     f.L.assign((size_t)n_u * f.n_v, 0.0);
     for (int i = 0; i < n_u; ++i)
       for (int j = 0; j < f.n_v; ++j) f.L[i * f.n_v + j] = Q[i * n_u + n_e + j];
+    if (reduced_basis) reduced_null_basis(net.E, n_e, n_u, f.L);
     // Pu = -E' (E E')^{-1} Ed  (minimum-norm particular solution of E u + Ed d = 0)
     std::vector<double> EEt((size_t)n_e * n_e);
     for (int i = 0; i < n_e; ++i)

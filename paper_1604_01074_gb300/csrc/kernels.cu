@@ -26,8 +26,11 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
+#include <cstring>
 #include <type_traits>
+#include <vector>
 
 #include "smpc_internal.h"
 
@@ -3203,6 +3206,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) node_gt_tc(const __grid_constan
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(64));
 }
 
+#include "sweep.cuh"
+
 int optin_smem() {
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
@@ -3217,6 +3222,17 @@ LaunchCfg config_t(const IterArgs& a, int num_sms, int S_max, int schedule, int 
   c.schedule = schedule;
   c.block = kThreads;
   const bool fits_threads = a.n_k <= kThreads && a.n_v <= kThreads;  // one thread per entry
+  if (schedule == SCHED_SWEEP) {  // sparse [Bbar; L] and packed Lambda of the vector type, A = I
+    c.stages = 0;
+    if constexpr (std::is_same<VT, MT>::value) {
+      c.smem = sweep_smem_bytes<VT>(a.sp_nnz, a.depth, a.n_x, a.n_u, a.n_v);
+      c.grid = a.n_chains + a.n_top;
+      c.smem_lam = lambda_smem_bytes<VT>(a.n_k, a.n_v);
+      c.grid_lam = a.n_top + (a.n - a.n_top + kWarps - 1) / kWarps;
+      if (a.lam && a.sp && fits_threads && !a.A && c.smem + 512 <= (size_t)optin) c.stages = 1;
+    }
+    return c;
+  }
   if (schedule == SCHED_CHAIN) {
     int S = S_max;
     while (S > 1 && iter_smem_bytes<MT>(S, a.n_x, a.n_u, a.n_v) > (size_t)optin) --S;
@@ -3313,6 +3329,14 @@ void launch_dep(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaSt
   cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// tree_sweep for the network's tanks and inputs per lane (n_x + n_u <= 256)
+template <typename VT>
+auto sweep_kernel(const IterArgs& a) {
+  if (a.n_x <= 32 && a.n_u <= 64) return tree_sweep<VT, 1, 2>;
+  if (a.n_x <= 64 && a.n_u <= 128) return tree_sweep<VT, 2, 4>;
+  return tree_sweep<VT, 8, 8>;
+}
+
 template <typename VT, typename MT>
 int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream_t s) {
   // once per process and instantiation; thread-safe (solves may run on several threads).
@@ -3335,6 +3359,12 @@ int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream
     if constexpr (std::is_same<MT, __nv_bfloat16>::value) {
       allow(node_mv_tc<VT>);
       allow(node_gt_tc<VT>);
+    } else {
+      allow(tree_sweep<VT, 1, 2>);
+      allow(tree_sweep<VT, 2, 4>);
+      allow(tree_sweep<VT, 8, 8>);
+      allow(lambda_apply<VT, 4>);
+      allow(lambda_apply<VT, 8>);
     }
     cudaGetLastError();  // a refused attribute surfaces at the launch, not here
     return true;
@@ -3350,6 +3380,18 @@ int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream
     launch_dep(apg_iter<VT, MT>, c.grid, c.block, c.smem, s, dep, a, c.stages, nu, mode);
     mark();
     return check_launch("apg_iter");
+  }
+  if constexpr (std::is_same<VT, MT>::value) {
+    if (c.schedule == SCHED_SWEEP) {
+      launch_dep(sweep_kernel<VT>(a), c.grid, kThreads, c.smem, s, dep, a, nu, mode);
+      mark();
+      if (mode & MODE_BWD) {
+        launch_dep(lam_bs(a.n_v) == 4 ? lambda_apply<VT, 4> : lambda_apply<VT, 8>, c.grid_lam, kThreads, c.smem_lam, s,
+                   dep, a, nu, mode);
+        mark();
+      }
+      return check_launch("tree sweep");
+    }
   }
   if ((mode & MODE_PROX) && nu >= 1) {
     launch_dep(fwd_scan<VT, MT>, c.grid_fwd, c.block, c.smem_fwd, s, dep, a, nu, mode);
@@ -3467,6 +3509,48 @@ int launch_pack(int prec, int n, int n_k, int n_v, const double* K, const double
       pack_kernel<float, __nv_bfloat16><<<grid, 256, 0, s>>>(n, n_k, n_v, K, Lam, prob, (__nv_bfloat16*)packs, stride);
   }
   return check_launch("pack_kernel");
+}
+
+long long lam_pack_entries(int n_v) { return lam_entries(n_v); }
+int launch_lam_pack(int prec, int n, int n_v, const double* Lam, const double* prob, void* out, void* stream) {
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const int grid = n < 4096 ? n : 4096;
+  if (prec == SMPC_FP64)
+    lam_pack_kernel<double><<<grid, 256, 0, s>>>(n, n_v, Lam, prob, (double*)out);
+  else
+    lam_pack_kernel<float><<<grid, 256, 0, s>>>(n, n_v, Lam, prob, (float*)out);
+  return check_launch("lam_pack_kernel");
+}
+namespace {
+template <typename VT>
+std::vector<unsigned char> sparse_t(int n_k, int n_v, const double* K) {
+  std::vector<SpEnt<VT>> ent;
+  std::vector<int> idx;
+  for (int tr = 0; tr < 2; ++tr) {  // the rows of K, then the rows of K'
+    const int R = tr ? n_v : n_k, C = tr ? n_k : n_v;
+    auto at = [&](int i, int j) { return tr ? K[(size_t)j * n_v + i] : K[(size_t)i * n_v + j]; };
+    std::vector<int> count(R, 0), id(R), ptr(1, 0);
+    for (int i = 0; i < R; ++i) {
+      id[i] = i;
+      for (int j = 0; j < C; ++j) count[i] += at(i, j) != 0.0;
+    }
+    std::stable_sort(id.begin(), id.end(), [&](int x, int y) { return count[x] > count[y]; });
+    for (int i : id) {
+      for (int j = 0; j < C; ++j)
+        if (at(i, j) != 0.0) ent.push_back(SpEnt<VT>{(VT)at(i, j), j});
+      ptr.push_back(ptr.back() + count[i]);
+    }
+    idx.insert(idx.end(), ptr.begin(), ptr.end());
+    idx.insert(idx.end(), id.begin(), id.end());
+  }
+  std::vector<unsigned char> out(sp_bytes<VT>((int)ent.size() / 2, n_k, n_v), 0);
+  std::memcpy(out.data(), ent.data(), ent.size() * sizeof(SpEnt<VT>));
+  std::memcpy(out.data() + ent.size() * sizeof(SpEnt<VT>), idx.data(), idx.size() * sizeof(int));
+  return out;
+}
+}  // namespace
+std::vector<unsigned char> sparse_image(int prec, int n_k, int n_v, const double* K) {
+  return prec == SMPC_FP64 ? sparse_t<double>(n_k, n_v, K) : sparse_t<float>(n_k, n_v, K);
 }
 
 int launch_cost_update(int prec, const CostArgs& a, void* stream) {

@@ -248,6 +248,7 @@ extern "C" int smpc_solve_static(smpc_factor_t* f, const smpc_step_data* data, c
   a.R = f->R;
   a.res_tree = nullptr;
   a.tree_done = f->tree_done;
+  set_sweep_args(f, a);
   IterPlan plan;
   STRY(plan_iters(f, a, *opts, &plan));
 

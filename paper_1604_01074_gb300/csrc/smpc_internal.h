@@ -21,7 +21,7 @@ void set_error(const char* fmt, ...);
 // Host FP64 dense linear algebra for the factor step (App. A, App. B).
 struct HostFactor {
   int n_x = 0, n_u = 0, n_d = 0, n_e = 0, n_v = 0;
-  std::vector<double> L;      // n_u x n_v, orthonormal basis of null(E)
+  std::vector<double> L;      // n_u x n_v, basis of null(E): orthonormal or reduced
   std::vector<double> Bbar;   // n_x x n_v
   std::vector<double> Rhat;   // n_u x n_v
   std::vector<double> Rbar;   // n_v x n_v
@@ -32,7 +32,8 @@ struct HostFactor {
   std::vector<double> diagL;  // n_u, diag(L Rbar^{-1} L')
 };
 // Returns SMPC_OK or SMPC_EINVAL (rank-deficient E, W_u not positive definite).
-int host_factor(const smpc_network& net, const double* W_u, HostFactor& out);
+// reduced_basis: L in reduced form where that basis is well conditioned (factor_host.cpp).
+int host_factor(const smpc_network& net, const double* W_u, HostFactor& out, bool reduced_basis);
 
 // ---------------------------------------------------------------------------
 // Tree structure after validation (host copy + device mirrors).
@@ -57,6 +58,8 @@ struct DevTree {
   int* tree_of = nullptr;       // per node: its tree (the index of its root)
   int* row = nullptr;           // per node: its row of the stage-indexed step data
   int* seg = nullptr;           // kSegInts per forward-sweep segment (top nodes, then chains)
+  int* top_src_off = nullptr;   // per top node: its chain heads and top nodes below (SCHED_SWEEP)
+  int* top_src = nullptr;       // {node, weight}
   double* prob = nullptr;
   double* pbar = nullptr;       // p_n + sum of children's p (App. A)
 };
@@ -74,6 +77,7 @@ struct smpc_tree {
   std::vector<int> top_nodes, is_top, top_expect;
   std::vector<int> path_off, path_node;
   std::vector<int> seg;  // forward-sweep segment descriptors (kSegInts each)
+  std::vector<int> top_src_off, top_src;
   smpc::DevTree dev;
 };
 
@@ -148,6 +152,15 @@ struct IterArgs {
   // (its chains and the replicated top nodes), or NULL for all n nodes.
   const int* node_list;
   int n_list;
+  // SCHED_SWEEP: the sparse image of [Bbar; L] (sparse_image), Lambda / (2 p_n) of every node
+  // as symmetric blocks (or one unscaled Lambda, lam_stride 0, with pscale), the largest tree
+  // depth, and per top node its sources {node, weight}: chain heads, then top nodes.
+  const void* sp;
+  int sp_nnz, depth;
+  const void* lam;
+  long long lam_stride;
+  const int* top_src_off;        // 2 n_top + 1
+  const int* top_src;
 };
 
 enum KernelMode : int {
@@ -171,6 +184,12 @@ enum Schedule : int {
   SCHED_FUSED = 4    // node-parallel forward sweep and prox, then the whole backward sweep as one chain pass
 };
 constexpr int kSchedules = 4;
+// The form of schedule 4 that a factor may choose by timing where [Bbar; L] is sparse: one
+// tree pass and one Lambda launch per iteration (sweep.cuh).  Reported as schedule 4.
+constexpr int SCHED_SWEEP = 5;
+// Entries of [Bbar; L] up to which it counts as sparse: its image is read into shared memory
+// by every CTA of the tree pass (64 KB at this size in float32).
+constexpr int kSparseMax = 4096;
 
 struct LaunchCfg {
   int schedule = SCHED_CHAIN;
@@ -194,6 +213,8 @@ struct LaunchCfg {
   // hybrid schedule: the backward sweep up to r runs as the chain kernel in MODE_GT
   int grid_chain = 1, stages_chain = 0;
   size_t smem_chain = 0;
+  int grid_lam = 1;         // SCHED_SWEEP: the Lambda launch (the tree pass: grid, smem)
+  size_t smem_lam = 0;
   // profiling: when set, an event is recorded before the first and after every kernel
   // of a launch_iter call (kernels_per_call + 1 events)
   cudaEvent_t* events = nullptr;
@@ -201,6 +222,7 @@ struct LaunchCfg {
 // kernels one launch_iter call enqueues
 inline int kernels_per_call(const LaunchCfg& c, int mode) {
   if (c.schedule == SCHED_CHAIN) return 1;
+  if (c.schedule == SCHED_SWEEP) return 1 + ((mode & MODE_BWD) ? 1 : 0);
   const int bwd = c.schedule == SCHED_HYBRID ? 2 : c.schedule == SCHED_FUSED ? 1 : 4;
   return 1 + ((mode & MODE_PROX) ? 1 : 0) + ((mode & MODE_BWD) ? bwd : 0);
 }
@@ -212,6 +234,11 @@ LaunchCfg iter_config(int prec, const IterArgs& a, int num_sms, int schedule = S
 int launch_iter(int prec, const IterArgs& a, const LaunchCfg& cfg, int nu, int mode, void* stream);
 int launch_pack(int prec, int n, int n_k, int n_v, const double* K, const double* Lam, const double* prob,
                 void* packs, long long pack_stride, void* stream);
+// SCHED_SWEEP: entries of one node's packed Lambda, the packing of n matrices (prob NULL: one,
+// unscaled), and the host image of the sparse [Bbar; L] (n_k x n_v, float64) in the vector type
+long long lam_pack_entries(int n_v);
+int launch_lam_pack(int prec, int n, int n_v, const double* Lam, const double* prob, void* out, void* stream);
+std::vector<unsigned char> sparse_image(int prec, int n_k, int n_v, const double* K);
 struct CostArgs {
   int n, N, n_x, n_u, n_d, n_v;  // N: rows of stage-indexed data (sum of the trees' horizons)
   const int* parent;
@@ -291,6 +318,8 @@ int solve_end(smpc_factor_t* f, IterPlan& plan, const IterArgs& a, int launched,
 // does not fit the shared-memory pipeline.
 int plan_iters(const smpc_factor_t* f, const IterArgs& a, const smpc_solve_opts& opts, IterPlan* plan);
 int launch_planned(IterPlan& plan, int nu, int mode, void* stream);
+// The SCHED_SWEEP fields of a.
+void set_sweep_args(const smpc_factor_t* f, IterArgs& a);
 // Copies the final dual of the factor's last solve (vector type) to dst; synchronous.
 int copy_final_y(smpc_factor_t* f, void* dst);
 }  // namespace smpc
@@ -342,7 +371,9 @@ struct smpc_factor_t {
   int last_launches = 0;
   int num_sms = 0;
   int schedule = smpc::SCHED_CHAIN;  // iteration schedule in use
-  float tuned_ms[5] = {0, 0, 0, 0, 0};  // per schedule: ms per iteration measured when the factor chose
+  void *sp = nullptr, *lam = nullptr;  // SCHED_SWEEP: sparse [Bbar; L], packed Lambda
+  int sp_nnz = 0;
+  float tuned_ms[6] = {0, 0, 0, 0, 0, 0};  // per schedule: ms per iteration measured when the factor chose
   int tc_width = 0;                   // bfloat16 shared packs: nodes per tensor-core GEMM (0: none)
   float tc_ms[3] = {0, 0, 0};         // ms per delta iteration measured for widths 16, 32, 64
   smpc::Profile* profile = nullptr;  // set while smpc_profile_solve runs
@@ -365,6 +396,15 @@ struct smpc_factor_t {
     graphs.clear();
   }
 
+  void release(void* p, size_t bytes) {
+    for (size_t i = 0; i < allocs.size(); ++i)
+      if (allocs[i] == p) {
+        cudaFree(p);
+        allocs.erase(allocs.begin() + (long)i);
+        device_bytes -= bytes;
+        return;
+      }
+  }
   template <typename T>
   int alloc(T** p, size_t bytes) {
     *p = nullptr;
