@@ -79,7 +79,7 @@ bool finite_if_host(const double* p, size_t n) { return !host_readable(p) || fin
 void free_tree_dev(smpc::DevTree& d) {
   void* ptrs[] = {d.parent, d.stage, d.child_begin, d.child_count, d.chain_off, d.chain_node, d.chain_parent,
                   d.top_nodes, d.top_expect, d.path_off, d.path_node, d.tree_of, d.row, d.seg, d.prob, d.pbar,
-                  d.top_src_off, d.top_src};
+                  d.top_src_off, d.top_src, d.chain_kids};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   d = smpc::DevTree();
@@ -223,36 +223,33 @@ int build_tree(int32_t n, const int32_t* parent, const double* prob, smpc_tree& 
     }
   }
   t.path_off[n] = (int)t.path_node.size();
-  // Per top node t the chain heads below it, then the top nodes below it and itself, each with
-  // the number of top nodes from t down to its parent (a top node: itself included), which is
-  // how often its xi counts in t's sums of s.  No lists (SCHED_SWEEP does not run) beyond
-  // kMaxTopSrc entries, which only deep trees that branch at every stage reach.
+  t.chain_kids.assign(n, 0);
+  for (int p : t.chain_parent)
+    if (p >= 0) ++t.chain_kids[p];
+  // Per top node t the top nodes below it and itself, each with the number of top nodes from t
+  // down to it, which is how often its xi counts in the sums of s over t's top nodes.  No lists
+  // (SCHED_SWEEP does not run) beyond kMaxTopSrc entries, which only deep trees that branch at
+  // every stage reach.
   constexpr size_t kMaxTopSrc = size_t(1) << 24;
   {
     std::vector<int> index(n, -1);
     for (size_t i = 0; i < t.top_nodes.size(); ++i) index[t.top_nodes[i]] = (int)i;
-    std::vector<size_t> cnt(2 * t.top_nodes.size() + 1, 0);
-    auto visit = [&](auto&& f) {  // f(list, node, weight)
-      for (size_t c = 0; c + 1 < t.chain_off.size(); ++c) {
-        const int h = t.chain_node[t.chain_off[c]];
-        for (int k = parent[h]; k >= 0; k = parent[k]) f(2 * index[k], h, t.stage[h] - t.stage[k]);
-      }
-      for (int m : t.top_nodes)
-        for (int k = m; k >= 0; k = parent[k]) f(2 * index[k] + 1, m, t.stage[m] - t.stage[k] + 1);
-    };
+    std::vector<size_t> cnt(t.top_nodes.size() + 1, 0);
     size_t total = 0;
-    visit([&](int list, int, int) { ++cnt[list + 1], ++total; });
+    for (int m : t.top_nodes)
+      for (int k = m; k >= 0; k = parent[k]) ++cnt[index[k] + 1], ++total;
     t.top_src_off.clear();
     t.top_src.clear();
     if (total <= kMaxTopSrc) {
       for (size_t i = 1; i < cnt.size(); ++i) cnt[i] += cnt[i - 1];
       t.top_src_off.assign(cnt.begin(), cnt.end());
       t.top_src.resize(2 * total);
-      visit([&](int list, int m, int w) {
-        const size_t q = cnt[list]++;
-        t.top_src[2 * q] = m;
-        t.top_src[2 * q + 1] = w;
-      });
+      for (int m : t.top_nodes)
+        for (int k = m; k >= 0; k = parent[k]) {
+          const size_t q = cnt[index[k]]++;
+          t.top_src[2 * q] = m;
+          t.top_src[2 * q + 1] = t.stage[m] - t.stage[k] + 1;
+        }
     }
   }
   const int n_seg = (int)(t.top_nodes.size() + t.chain_parent.size());
@@ -291,6 +288,7 @@ int upload_tree(smpc_tree& t) {
   TRY(dev_upload(&d.seg, t.seg.data(), t.seg.size()));
   TRY(dev_upload(&d.top_src_off, t.top_src_off.data(), t.top_src_off.size()));
   TRY(dev_upload(&d.top_src, t.top_src.data(), t.top_src.size()));
+  TRY(dev_upload(&d.chain_kids, t.chain_kids.data(), t.chain_kids.size()));
   TRY(dev_upload(&d.prob, t.prob.data(), t.n));
   TRY(dev_upload(&d.pbar, t.pbar.data(), t.n));
   return SMPC_OK;
@@ -306,10 +304,12 @@ void set_sweep_args(const smpc_factor_t* f, IterArgs& a) {
   a.sp = t->top_src_off.empty() ? nullptr : f->sp;
   a.sp_nnz = f->sp_nnz;
   a.depth = t->N;
+  a.max_len = t->max_chain_len;
   a.lam = f->lam;
   a.lam_stride = f->shared_packs ? 0 : lam_pack_entries(f->n_v);
   a.top_src_off = t->dev.top_src_off;
   a.top_src = t->dev.top_src;
+  a.chain_kids = t->dev.chain_kids;
 }
 }  // namespace smpc
 

@@ -3227,8 +3227,23 @@ LaunchCfg config_t(const IterArgs& a, int num_sms, int S_max, int schedule, int 
     if constexpr (std::is_same<VT, MT>::value) {
       c.smem = sweep_smem_bytes<VT>(a.sp_nnz, a.depth, a.n_x, a.n_u, a.n_v);
       c.grid = a.n_chains + a.n_top;
-      c.smem_lam = lambda_smem_bytes<VT>(a.n_k, a.n_v);
-      c.grid_lam = a.n_top + (a.n - a.n_top + kWarps - 1) / kWarps;
+      const int tasks = a.max_len * (1 + (a.n_u + 63) / 64);  // of a chain's prox, one warp each
+      c.sweep_warps = a.n_x > 64 ? 16
+                      : a.n_chains > 2 * num_sms || tasks <= 8 ? 8
+                      : a.n_chains <= num_sms && tasks >= 48 && sizeof(VT) == 4 ? 32 : 16;
+      // Lambda: matrix slots for four chain warps where two CTAs fit an SM, else as many as fit
+      const int n_c = a.n - a.n_top;
+      const int ctas = sizeof(VT) == 4 && lam_bs(a.n_v) == 4 ? 2 : 1;  // CTAs an SM, by registers
+      const size_t room = (size_t)optin / ctas - (ctas == 2 ? 8192 : 24576);
+      // float64: the pipe, not the copies, sets the time, and eight warps reading in place keep
+      // it busier than the four that slots of 42 KB leave
+      c.lam_slots = a.lam_stride == 0 ? 1 : sizeof(VT) == 8 ? 0 : 4;
+      while (c.lam_slots > 1 && lambda_smem_bytes<VT>(a.n_v, c.lam_slots) > room) --c.lam_slots;
+      if (lambda_smem_bytes<VT>(a.n_v, c.lam_slots) > room) c.lam_slots = 0;
+      c.smem_lam = lambda_smem_bytes<VT>(a.n_v, c.lam_slots);
+      c.lam_warps = a.lam_stride == 0 || sizeof(VT) == 8 ? 8 : 4;  // chain warps a CTA
+      const int cw = c.lam_slots == 0 || a.lam_stride == 0 ? c.lam_warps : c.lam_slots;
+      c.grid_lam = std::min(std::max((n_c + cw - 1) / cw, a.n_top), ctas * num_sms);
       if (a.lam && a.sp && fits_threads && !a.A && c.smem + 512 <= (size_t)optin) c.stages = 1;
     }
     return c;
@@ -3329,12 +3344,14 @@ void launch_dep(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaSt
   cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// tree_sweep for the network's tanks and inputs per lane (n_x + n_u <= 256)
+// tree_sweep for the network's tanks per lane and the tree's chains per SM
 template <typename VT>
-auto sweep_kernel(const IterArgs& a) {
-  if (a.n_x <= 32 && a.n_u <= 64) return tree_sweep<VT, 1, 2>;
-  if (a.n_x <= 64 && a.n_u <= 128) return tree_sweep<VT, 2, 4>;
-  return tree_sweep<VT, 8, 8>;
+auto sweep_kernel(const IterArgs& a, int warps) {
+  if constexpr (sizeof(VT) == 4) {
+    if (warps == 32) return a.n_x <= 32 ? tree_sweep<VT, 1, 32> : tree_sweep<VT, 2, 32>;
+  }
+  if (warps == 8) return a.n_x <= 32 ? tree_sweep<VT, 1, 8> : tree_sweep<VT, 2, 8>;
+  return a.n_x <= 32 ? tree_sweep<VT, 1, 16> : a.n_x <= 64 ? tree_sweep<VT, 2, 16> : tree_sweep<VT, 8, 16>;
 }
 
 template <typename VT, typename MT>
@@ -3360,11 +3377,18 @@ int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream
       allow(node_mv_tc<VT>);
       allow(node_gt_tc<VT>);
     } else {
-      allow(tree_sweep<VT, 1, 2>);
-      allow(tree_sweep<VT, 2, 4>);
-      allow(tree_sweep<VT, 8, 8>);
-      allow(lambda_apply<VT, 4>);
-      allow(lambda_apply<VT, 8>);
+      IterArgs t{};
+      for (int n_x : {32, 64, 65})
+        for (int warps : {8, 16, 32}) {
+          t.n_x = n_x;
+          if (n_x <= 64 || warps == 16) allow(sweep_kernel<VT>(t, warps));
+        }
+      if constexpr (sizeof(VT) == 4) {
+        allow(lambda_apply<VT, 4, 4>);
+        allow(lambda_apply<VT, 8, 4>);
+      }
+      allow(lambda_apply<VT, 4, 8>);
+      allow(lambda_apply<VT, 8, 8>);
     }
     cudaGetLastError();  // a refused attribute surfaces at the launch, not here
     return true;
@@ -3383,11 +3407,16 @@ int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream
   }
   if constexpr (std::is_same<VT, MT>::value) {
     if (c.schedule == SCHED_SWEEP) {
-      launch_dep(sweep_kernel<VT>(a), c.grid, kThreads, c.smem, s, dep, a, nu, mode);
+      // nu = 0 waits for everything before it, so that later launches may read the solve's
+      // affine data before their programmatic wait
+      launch_dep(sweep_kernel<VT>(a, c.sweep_warps), c.grid, 32 * c.sweep_warps, c.smem, s, dep && nu > 0, a, nu, mode);
       mark();
       if (mode & MODE_BWD) {
-        launch_dep(lam_bs(a.n_v) == 4 ? lambda_apply<VT, 4> : lambda_apply<VT, 8>, c.grid_lam, kThreads, c.smem_lam, s,
-                   dep, a, nu, mode);
+        const bool wide = lam_bs(a.n_v) == 8;
+        auto kern = wide ? lambda_apply<VT, 8, 8> : lambda_apply<VT, 4, 8>;
+        if constexpr (sizeof(VT) == 4)
+          if (c.lam_warps == 4) kern = wide ? lambda_apply<VT, 8, 4> : lambda_apply<VT, 4, 4>;
+        launch_dep(kern, c.grid_lam, (c.lam_warps + kWarps) * 32, c.smem_lam, s, dep, a, c.lam_slots, nu, mode);
         mark();
       }
       return check_launch("tree sweep");

@@ -58,8 +58,9 @@ struct DevTree {
   int* tree_of = nullptr;       // per node: its tree (the index of its root)
   int* row = nullptr;           // per node: its row of the stage-indexed step data
   int* seg = nullptr;           // kSegInts per forward-sweep segment (top nodes, then chains)
-  int* top_src_off = nullptr;   // per top node: its chain heads and top nodes below (SCHED_SWEEP)
+  int* top_src_off = nullptr;   // per top node: the top nodes below and itself (SCHED_SWEEP)
   int* top_src = nullptr;       // {node, weight}
+  int* chain_kids = nullptr;    // per node: chains among its children
   double* prob = nullptr;
   double* pbar = nullptr;       // p_n + sum of children's p (App. A)
 };
@@ -77,7 +78,7 @@ struct smpc_tree {
   std::vector<int> top_nodes, is_top, top_expect;
   std::vector<int> path_off, path_node;
   std::vector<int> seg;  // forward-sweep segment descriptors (kSegInts each)
-  std::vector<int> top_src_off, top_src;
+  std::vector<int> top_src_off, top_src, chain_kids;
   smpc::DevTree dev;
 };
 
@@ -154,13 +155,14 @@ struct IterArgs {
   int n_list;
   // SCHED_SWEEP: the sparse image of [Bbar; L] (sparse_image), Lambda / (2 p_n) of every node
   // as symmetric blocks (or one unscaled Lambda, lam_stride 0, with pscale), the largest tree
-  // depth, and per top node its sources {node, weight}: chain heads, then top nodes.
+  // depth and chain length, and per top node its sources {node, weight}: the top nodes below and itself.
   const void* sp;
-  int sp_nnz, depth;
+  int sp_nnz, depth, max_len;
   const void* lam;
   long long lam_stride;
-  const int* top_src_off;        // 2 n_top + 1
+  const int* top_src_off;        // n_top + 1
   const int* top_src;
+  const int* chain_kids;         // per node: chains among its children
 };
 
 enum KernelMode : int {
@@ -213,7 +215,7 @@ struct LaunchCfg {
   // hybrid schedule: the backward sweep up to r runs as the chain kernel in MODE_GT
   int grid_chain = 1, stages_chain = 0;
   size_t smem_chain = 0;
-  int grid_lam = 1;         // SCHED_SWEEP: the Lambda launch (the tree pass: grid, smem)
+  int sweep_warps = 16, grid_lam = 1, lam_slots = 0, lam_warps = 8;  // SCHED_SWEEP: the Lambda launch (the tree pass: grid, smem)
   size_t smem_lam = 0;
   // profiling: when set, an event is recorded before the first and after every kernel
   // of a launch_iter call (kernels_per_call + 1 events)

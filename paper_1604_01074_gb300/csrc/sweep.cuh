@@ -8,15 +8,21 @@
 //   tree_sweep    one CTA per chain or top node: v = path sums of delta, [Bbar; L] v, x and u,
 //                 prox and dual update, w of the next iteration, then along the chain s, g =
 //                 [Bbar; L]' [s; psi] and r bottom-up.
-//   lambda_apply  delta_n = Lambda_n r_n, one warp per chain node; one CTA per top node, which
-//                 first forms its r from the chain heads and top nodes below it.  A top node's
-//                 s and r are weighted sums over them (a head's xi counts once for every top
-//                 node between the two), so no top node waits for another one.
+//   lambda_apply  delta_n = Lambda_n r_n, one warp per chain node; eight warps per top node,
+//                 which first add up its r.  With S_m = xi_m + the s of m's chains and R_m =
+//                 beta_m + the r of m's chains (m a top node),
+//                   r_t = sum over the top nodes m below t, and t itself, of
+//                         R_m + L' psi_m + c Bbar' S_m,
+//                 c the number of top nodes from t down to m.  The last of m's chains and m
+//                 itself forms the two terms in tree_sweep, so no top node waits for another.
 // Per iteration on GB300, one pack per node (the launches of schedules 2 to 4 before): 2081
-// nodes 39.5 us in float32 (104), 162 us in float64 (381); 21 111 nodes 191 us (577); one pack
-// for all of 21 111 nodes 157 us (396).
+// nodes 27.2 us in float32 (104), 116 us in float64 (381); 21 111 nodes 145 us (577), the tree
+// pass 71 and Lambda 75; one pack for all of 21 111 nodes 107 us (396).  The tree pass is bound
+// by issue slots (some 1900 warp instructions a node, half of them the prox in float32 pairs),
+// Lambda by HBM (439 MB at 5.9 TB/s) and in float64 by the pipe (2 lanes a cycle and SM).
 // Vectors between the launches: h holds delta (n x n_v), rpub r of the chain nodes, spub s of
-// the chain heads, wbuf w of the top nodes.
+// the chain heads; a top node m's row of rpub holds R_m + L' psi_m, the first n_v entries of
+// its row of wbuf (w, until the last arrival) Bbar' S_m.
 
 // ---------------------------------------------------------------- sparse [Bbar; L]
 // One entry: 8 bytes (float32) or 16 (float64).  Rows of K = [Bbar; L] and of K' are sorted
@@ -35,13 +41,13 @@ __host__ __device__ inline int sp_bytes(int nnz, int n_k, int n_v) {
 // put(r, e, (A x_r)_e + pre(r, e)) for rows r0 <= r < r1 of X (row stride xs) and all rows e
 // of the sparse matrix.  A warp takes 32 rows e and four vectors r at a time, so each entry
 // is read once for four products.  X has three readable rows behind r1.
-template <typename VT, typename P, typename F>
+template <int NW, typename VT, typename P, typename F>
 __device__ __forceinline__ void sparse_rows(const SpEnt<VT>* ent, const int* ptr, const int* id, int rows, const VT* X,
                                             int xs, int r0, int r1, P&& pre, F&& put) {
   constexpr int NB = 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int rw = (rows + 31) / 32, ng = (r1 - r0 + NB - 1) / NB;
-  for (int task = warp; task < rw * ng; task += kWarps) {
+  for (int task = warp; task < rw * ng; task += NW) {
     const int g = task / rw, k = (task - g * rw) * 32 + lane;
     if (k >= rows) continue;
     const int e = id[k], rb = r0 + g * NB;
@@ -70,31 +76,83 @@ __device__ __forceinline__ double ld_state(const double* p) { return *p; }
 __device__ __forceinline__ void st_state(DS* p, DS v) { *reinterpret_cast<float2*>(p) = make_float2(v.hi, v.lo); }
 __device__ __forceinline__ void st_state(double* p, double v) { *p = v; }
 
+// acc += w v, the product taken exactly
+__device__ __forceinline__ void st_fma_acc(DS& acc, float w, float v) { acc = st_axpy(acc, w, v); }
+__device__ __forceinline__ void st_fma_acc(double& acc, double w, double v) { acc = fma(w, v, acc); }
+
 template <typename VT>
 __host__ __device__ inline size_t sweep_smem_bytes(int nnz, int depth, int n_x, int n_u, int n_v) {
   const int n_k = n_x + n_u;
   size_t b = sp_bytes<VT>(nnz, n_k, n_v);
-  b += (size_t)(3 * n_x + 2 * n_u + (depth + 3) * (n_v + n_k)) * sizeof(VT);
+  b += (size_t)(3 * n_x + 2 * n_u + (depth + 3) * (n_v + n_k)) * sizeof(VT);  // depth + 3 >= 4 rows: the last arrival's too
   return round_up(b + (size_t)depth * sizeof(int), 16);
 }
 
-// Prox, dual update and w of node m on one warp (App. C; the arithmetic of
-// Kern::warp_prox_staged).  z holds x and u on entry and w on return.  All of the node's
-// loads are issued before the first use: lane l owns the tanks l + 32 k and the inputs
-// l + 32 k, NT and NU of them at most.
-template <typename VT, int NT, int NU>
-__device__ __forceinline__ void sweep_prox(const IterArgs& a, int m, VT* z, const VT* bnd, int nu, VT& rmax, VT& hmax,
-                                           VT& tmax) {
+// Running maxima of absolute values as bit patterns, which order like the values; an
+// infinity or NaN is above every finite one and stays visible in the maximum.  In float64 this
+// also keeps comparisons and maxima off the float64 pipe (2 lanes a cycle and SM).
+template <typename VT>
+struct MaxAbs;
+template <>
+struct MaxAbs<float> {
+  unsigned b = 0;
+  __device__ void add(float v) { b = max(b, __float_as_uint(v) & 0x7fffffffu); }
+  __device__ bool bad() const { return b >= 0x7f800000u; }
+  __device__ float value() const { return __uint_as_float(b); }
+};
+template <>
+struct MaxAbs<double> {
+  unsigned long long b = 0;
+  __device__ void add(double v) { b = max(b, (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull); }
+  __device__ bool bad() const { return b >= 0x7ff0000000000000ull; }
+  __device__ double value() const { return __longlong_as_double((long long)b); }
+};
+
+// Extrapolation and signs of the tree pass: in float64 the extrapolation is one fused
+// multiply-add on the difference, and signs are read from the bits.  In float32 the difference
+// and the product stay unnormalised pairs (their low parts are still below an ulp of the high
+// ones), which saves six of st_extrap's 28 operations; only the sum is renormalised.
+__device__ __forceinline__ DS sw_extrap(DS y1, DS y2, float c) {
+  const DS d = two_sum(y1.hi, -y2.hi);
+  const float dl = __fadd_rn(d.lo, __fsub_rn(y1.lo, y2.lo));
+  const float p = __fmul_rn(d.hi, c);
+  const float pe = __fmaf_rn(dl, c, __fmaf_rn(d.hi, c, -p));
+  const DS t = two_sum(y1.hi, p);
+  return fast_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(y1.lo, pe)));
+}
+// a - b rounded to the vector type
+__device__ __forceinline__ float sw_diff(DS a, DS b) {
+  return __fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo));
+}
+__device__ __forceinline__ double sw_diff(double a, double b) { return a - b; }
+__device__ __forceinline__ double sw_extrap(double y1, double y2, double c) { return fma(c, y1 - y2, y1); }
+__device__ __forceinline__ bool sw_neg(DS x) { return x.hi < 0.f; }
+__device__ __forceinline__ bool sw_neg(double x) { return __double_as_longlong(x) < 0; }
+__device__ __forceinline__ bool sw_pos(DS x) { return x.hi > 0.f; }
+__device__ __forceinline__ bool sw_pos(double x) { return __double_as_longlong(x) > 0; }
+template <typename ST>
+__device__ __forceinline__ ST sw_box(ST qh, ST ql) {
+  return sw_pos(qh) ? qh : (sw_neg(ql) ? ql : st_from<ST>(0.0));
+}
+
+// Prox, dual update and w of node m (App. C; the arithmetic of Kern::warp_prox_staged) in two
+// independent pieces, so that a node's work spreads over several warps: its tanks (both
+// distance blocks, whose norms couple them) on one warp, 32 NT at most, and its inputs, 64 per
+// warp.  z holds x and u on entry and w on return.  All loads are issued before the first use.
+template <typename VT>
+struct SweepOut {
+  MaxAbs<VT> r, h, t;  // residual maxima: |x - t|, |x|, |t| of the prox
+};
+template <typename VT, int NT>
+__device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, const VT* bnd, int it, VT c, VT cn,
+                                            SweepOut<VT>& o) {
   using ST = typename St<VT>::T;
-  const int lane = threadIdx.x & 31, n_x = a.n_x, n_u = a.n_u, nd = 2 * n_x + n_u, it = nu - 1;
-  const VT *xs = bnd, *xhi = xs + n_x, *xlo = xhi + n_x, *uhi = xlo + n_x, *ulo = uhi + n_u;
+  const int lane = threadIdx.x & 31, n_x = a.n_x, nd = 2 * n_x + a.n_u;
+  const VT *xs = bnd, *xhi = xs + n_x, *xlo = xhi + n_x;
   const ST* y1 = reinterpret_cast<const ST*>((it & 1) ? a.ybuf1 : a.ybuf0) + (long long)m * nd;
   ST* y2 = reinterpret_cast<ST*>((it & 1) ? a.ybuf0 : a.ybuf1) + (long long)m * nd;
-  const VT* step_p = reinterpret_cast<const VT*>(a.step_p) + (long long)m * n_u;
-  const VT* inv_p = reinterpret_cast<const VT*>(a.inv_p) + (long long)m * n_u;
   const ST zero = st_from<ST>(0.0);
-  ST v1[NT], ws[NT], w1[NT], wz[NT], p1[NU], p2[NU];
-  VT lp[NU], ip[NU];
+  ST v1[NT], ws[NT], w1[NT], wz[NT];
 #pragma unroll
   for (int k = 0; k < NT; ++k) {
     const int e = lane + 32 * k;
@@ -106,25 +164,10 @@ __device__ __forceinline__ void sweep_prox(const IterArgs& a, int m, VT* z, cons
       wz[k] = ld_state(y2 + n_x + e);
     }
   }
-#pragma unroll
-  for (int k = 0; k < NU; ++k) {
-    const int i = lane + 32 * k;
-    p1[k] = p2[k] = zero;
-    lp[k] = ip[k] = 1;
-    if (i < n_u) {
-      p1[k] = ld_state(y1 + 2 * n_x + i);
-      p2[k] = ld_state(y2 + 2 * n_x + i);
-      lp[k] = step_p[i];
-      ip[k] = inv_p[i];
-    }
-  }
-  const VT c = (VT)a.cvec[it], cn = (VT)a.cvec[it + 1];
   const VT ls = reinterpret_cast<const VT*>(a.step_s)[m], lz = reinterpret_cast<const VT*>(a.step_z)[m];
   const VT is = reinterpret_cast<const VT*>(a.inv_s)[m], iz = reinterpret_cast<const VT*>(a.inv_z)[m];
   const VT mus = reinterpret_cast<const VT*>(a.mu_s)[m], muz = (VT)a.gamma_d;
-  const VT th = a.xbar && it > 0 ? (VT)a.theta[it] : (VT)1;  // ergodic average (theta_0 = 1)
   VT* xo = reinterpret_cast<VT*>(a.xout) + (long long)m * n_x;
-  VT* uo = reinterpret_cast<VT*>(a.uout) + (long long)m * n_u;
   // block norms ||lambda r|| of the two distance blocks
   VT ps = 0, pz = 0;
   ST qs[NT], qz[NT];
@@ -134,147 +177,222 @@ __device__ __forceinline__ void sweep_prox(const IterArgs& a, int m, VT* z, cons
     qs[k] = qz[k] = zero;
     if (e < n_x) {
       const VT x = z[e];
-      ws[k] = st_extrap(v1[k], ws[k], c);
-      wz[k] = st_extrap(w1[k], wz[k], c);
+      ws[k] = sw_extrap(v1[k], ws[k], c);
+      wz[k] = sw_extrap(w1[k], wz[k], c);
       const ST q = st_axpy(ws[k], ls, x - xs[e]);
-      qs[k] = st_neg(q) ? q : zero;  // C = {x >= x_s}
-      qz[k] = box_lr(st_axpy(wz[k], lz, x - xhi[e]), st_axpy(wz[k], lz, x - xlo[e]));
+      qs[k] = sw_neg(q) ? q : zero;  // C = {x >= x_s}
+      qz[k] = sw_box(st_axpy(wz[k], lz, x - xhi[e]), st_axpy(wz[k], lz, x - xlo[e]));
       const VT rs = st_val(qs[k]), rz = st_val(qz[k]);
       ps += rs * rs;
       pz += rz * rz;
     }
   }
-  // the input blocks do not need the norms: they fill the reduction's latency
-  VT rm = 0, hm = 0, tm = 0;
-  bool bad = false;
+  // lanes 0 .. 15 add up and finish the s block, the others the z block: kappa = min(1, mu /
+  // ||lambda r||), where a block within mu needs no root and division (in float64 as much work
+  // as the rest of a node)
+  const bool lo = lane < 16;
+  VT sq = lo ? ps : pz;
+  sq += __shfl_xor_sync(0xffffffffu, lo ? pz : ps, 16);
 #pragma unroll
-  for (int k = 0; k < NU; ++k) {
-    const int i = lane + 32 * k;
-    if (i < n_u) {
-      const VT u = z[n_x + i];
-      const ST wp = st_extrap(p1[k], p2[k], c);
-      const ST ypn = box_lr(st_axpy(wp, lp[k], u - uhi[i]), st_axpy(wp, lp[k], u - ulo[i]));
-      const VT ep = st_val(st_sub(ypn, wp)) * ip[k];
-      st_state(y2 + 2 * n_x + i, ypn);
-      uo[i] = u;
-      z[n_x + i] = st_extrap_val(ypn, p1[k], cn);
-      if (a.ubar) {
-        VT* b = reinterpret_cast<VT*>(a.ubar) + (long long)m * n_u + i;
-        *b = it == 0 ? u : (VT)(((VT)1 - th) * *b + th * u);
-      }
-      rm = fmax(rm, fabs(ep));
-      hm = fmax(hm, fabs(u));
-      tm = fmax(tm, fabs(u - ep));
-      bad |= !isfinite(st_val(ypn)) || !isfinite(u);
-    }
+  for (int d = 8; d > 0; d >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, d);
+  const VT mu = lo ? mus : muz;
+  VT kap = 1;
+  if (!(sq <= mu * mu)) {
+    const VT dist = sqrt(sq);
+    kap = dist > mu ? mu / dist : (VT)1;
   }
-  ps = warp_sum(ps);
-  pz = warp_sum(pz);
-  const VT ds = sqrt(ps), dz = sqrt(pz);
-  const VT ks = ds > mus ? mus / ds : (VT)1, kz = dz > muz ? muz / dz : (VT)1;
+  const VT ks = __shfl_sync(0xffffffffu, kap, 0), kz = __shfl_sync(0xffffffffu, kap, 16);
 #pragma unroll
   for (int k = 0; k < NT; ++k) {
     const int e = lane + 32 * k;
     if (e < n_x) {
       const VT x = z[e];
       const ST ysn = st_scale(qs[k], ks), yzn = st_scale(qz[k], kz);
-      const VT es = st_val(st_sub(ysn, ws[k])) * is, ez = st_val(st_sub(yzn, wz[k])) * iz;
+      const VT es = sw_diff(ysn, ws[k]) * is, ez = sw_diff(yzn, wz[k]) * iz;
       st_state(y2 + e, ysn);
       st_state(y2 + n_x + e, yzn);
       xo[e] = x;
       z[e] = st_extrap_val(ysn, v1[k], cn) + st_extrap_val(yzn, w1[k], cn);
-      if (a.xbar) {
+      if (a.xbar) {  // ergodic average (theta_0 = 1: the previous contents are not read then)
         VT* b = reinterpret_cast<VT*>(a.xbar) + (long long)m * n_x + e;
+        const VT th = (VT)a.theta[it];
         *b = it == 0 ? x : (VT)(((VT)1 - th) * *b + th * x);
       }
-      rm = fmax(rm, fmax(fabs(es), fabs(ez)));
-      hm = fmax(hm, fabs(x));
-      tm = fmax(tm, fmax(fabs(x - es), fabs(x - ez)));
-      // the prox maps a non-finite v to 0, so the primal iterate is checked as well
-      bad |= !isfinite(st_val(ysn)) || !isfinite(st_val(yzn)) || !isfinite(x);
+      o.r.add(es);  // a non-finite y shows in its residual
+      o.r.add(ez);
+      o.h.add(x);  // the prox maps a non-finite v to 0, so the primal iterate counts as well
+      o.t.add(x - es);
+      o.t.add(x - ez);
     }
   }
-  if (bad) a.flags[1] = SMPC_EDIVERGED;
-  rmax = fmax(rmax, rm);
-  hmax = fmax(hmax, hm);
-  tmax = fmax(tmax, tm);
+}
+template <typename VT>
+__device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, VT* z, const VT* bnd, int it, VT c, VT cn,
+                                             SweepOut<VT>& o) {
+  using ST = typename St<VT>::T;
+  constexpr int NU = 2;
+  const int lane = threadIdx.x & 31, n_x = a.n_x, n_u = a.n_u, nd = 2 * n_x + n_u;
+  const VT *uhi = bnd + 3 * n_x, *ulo = uhi + n_u;
+  const ST* y1 = reinterpret_cast<const ST*>((it & 1) ? a.ybuf1 : a.ybuf0) + (long long)m * nd + 2 * n_x;
+  ST* y2 = reinterpret_cast<ST*>((it & 1) ? a.ybuf0 : a.ybuf1) + (long long)m * nd + 2 * n_x;
+  const long long mu = (long long)m * n_u;
+  const ST zero = st_from<ST>(0.0);
+  ST p1[NU], p2[NU];
+  VT lp[NU], ip[NU];
+#pragma unroll
+  for (int k = 0; k < NU; ++k) {
+    const int i = i0 + lane + 32 * k;
+    p1[k] = p2[k] = zero;
+    lp[k] = ip[k] = 1;
+    if (i < n_u) {
+      p1[k] = ld_state(y1 + i);
+      p2[k] = ld_state(y2 + i);
+      lp[k] = reinterpret_cast<const VT*>(a.step_p)[mu + i];
+      ip[k] = reinterpret_cast<const VT*>(a.inv_p)[mu + i];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < NU; ++k) {
+    const int i = i0 + lane + 32 * k;
+    if (i < n_u) {
+      const VT u = z[n_x + i];
+      const ST wp = sw_extrap(p1[k], p2[k], c);
+      const ST ypn = sw_box(st_axpy(wp, lp[k], u - uhi[i]), st_axpy(wp, lp[k], u - ulo[i]));
+      const VT ep = sw_diff(ypn, wp) * ip[k];
+      st_state(y2 + i, ypn);
+      reinterpret_cast<VT*>(a.uout)[mu + i] = u;
+      z[n_x + i] = st_extrap_val(ypn, p1[k], cn);
+      if (a.ubar) {
+        VT* b = reinterpret_cast<VT*>(a.ubar) + mu + i;
+        const VT th = (VT)a.theta[it];
+        *b = it == 0 ? u : (VT)(((VT)1 - th) * *b + th * u);
+      }
+      o.r.add(ep);
+      o.h.add(u);
+      o.t.add(u - ep);
+    }
+  }
 }
 
-template <typename VT, int NT, int NU>
-__global__ void __launch_bounds__(kThreads, NT == 8 ? 1 : sizeof(VT) == 4 ? 3 : 2)
+// In-place running sums of column `col` over rows r0, r0 + dr, ... (n of them); put(r, v) sees
+// each sum.  Eight rows are read ahead of their sums.
+template <typename VT, typename F>
+__device__ __forceinline__ void run_sums(VT* X, int xs, int col, int r0, int dr, int n, VT v, F&& put) {
+  constexpr int B = 8;
+  for (int q0 = 0; q0 < n; q0 += B) {
+    VT t[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) t[b] = q0 + b < n ? X[(r0 + (q0 + b) * dr) * xs + col] : (VT)0;
+#pragma unroll
+    for (int b = 0; b < B; ++b)
+      if (q0 + b < n) {
+        v += t[b];
+        put(r0 + (q0 + b) * dr, v);
+      }
+  }
+}
+
+// NW warps a CTA at 64 registers a thread (float64: 128).  Most phases of a segment wait on
+// memory or shared memory with few warps busy, so trees with several chains an SM run four
+// small CTAs there, side by side in different phases; trees with at most a chain an SM have
+// nothing to overlap and spread each chain over as many warps as an SM takes.
+template <typename VT, int NT, int NW>
+__global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 : 16) / NW)
     tree_sweep(const __grid_constant__ IterArgs a, int nu, int mode) {
   using ST = typename St<VT>::T;
+  constexpr int kSweepThreads = 32 * NW;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int flag[2];
-  __shared__ VT red[3 * kWarps];
+  __shared__ VT red[3 * NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_x = a.n_x, n_u = a.n_u, n_k = a.n_k, n_v = a.n_v, nnz = a.sp_nnz;
-  // ---- constants of the factor and the tree, read while the previous launch drains
+  const bool prox = (mode & MODE_PROX) != 0 && nu >= 1;
+  // ---- read while the previous launch drains: constants of the factor and the tree, and the
+  // solve's affine data, complete before its first launch (nu = 0), which starts without
+  // programmatic overlap
   const int blob = sp_bytes<VT>(nnz, n_k, n_v);
-  for (int q = tid; q < blob / 16; q += kThreads)
-    reinterpret_cast<uint4*>(smem_raw)[q] = reinterpret_cast<const uint4*>(a.sp)[q];
   const SpEnt<VT>* ek = reinterpret_cast<const SpEnt<VT>*>(smem_raw);
   const SpEnt<VT>* et = ek + nnz;
   const int* rptr = reinterpret_cast<const int*>(et + nnz);
   const int *rid = rptr + n_k + 1, *cptr = rid + n_k, *cid = cptr + n_v + 1;
   VT* bnd = reinterpret_cast<VT*>(smem_raw + blob);
-  VT* V = bnd + 3 * n_x + 2 * n_u;  // delta, then v, then g and r: a row of n_v per node
-  VT* Z = V + (a.depth + 3) * n_v;  // [Bbar; L] v, then x and u, then w and s: a row of n_k per node
+  VT* V = bnd + 3 * n_x + 2 * n_u;  // delta, then v, then beta, g and r: a row of n_v per node
+  VT* Z = V + (a.depth + 3) * n_v;  // e and u_hat, then x and u, then w and s: a row of n_k per node
   int* sid = reinterpret_cast<int*>(Z + (a.depth + 3) * n_k);
-  for (int q = tid; q < 3 * n_x + 2 * n_u; q += kThreads) {
-    const void* src = q < n_x ? a.x_s : q < 2 * n_x ? a.x_max : q < 3 * n_x ? a.x_min : q < 3 * n_x + n_u ? a.u_max : a.u_min;
-    const int i = q < 3 * n_x ? q % n_x : (q - 3 * n_x) % n_u;
-    bnd[q] = reinterpret_cast<const VT*>(src)[i];
-  }
   // chains first (the long tasks), then the top nodes
   const int b = (int)blockIdx.x < a.n_chains ? a.n_top + blockIdx.x : blockIdx.x - a.n_chains;
   const int4 d0 = *reinterpret_cast<const int4*>(a.seg + (long long)kSegInts * b);
   const int4 d1 = *reinterpret_cast<const int4*>(a.seg + (long long)kSegInts * b + 4);
   const int pl = d0.z, len = d1.y, tree = d0.w;
-  const int L = pl + len;                   // the path (root .. parent), then the segment's own nodes
-  const int own = len == 0 ? pl - 1 : pl;   // first own row (a top node ends its path)
-  for (int r = tid; r < L; r += kThreads) sid[r] = r < pl ? a.path_node[d0.y + r] : a.chain_node[d1.x + r - pl];
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (early_exit(a, nu, mode, flag, true)) return;  // its barrier publishes the above
-  const bool prox = (mode & MODE_PROX) != 0 && nu >= 1;
-  if (!tree_active(a, tree, nu)) return;  // a forest's tree that stopped keeps its iterates
-  VT rmax = 0, hmax = 0, tmax = 0;
+  const int L = pl + len;                  // the path (root .. parent), then the segment's own nodes
+  const int own = len == 0 ? pl - 1 : pl;  // first own row (a top node ends its path)
+  for (int r = tid; r < L; r += kSweepThreads) sid[r] = r < pl ? a.path_node[d0.y + r] : a.chain_node[d1.x + r - pl];
+  for (int q = tid; q < blob / 16; q += kSweepThreads)
+    reinterpret_cast<uint4*>(smem_raw)[q] = reinterpret_cast<const uint4*>(a.sp)[q];
+  for (int q = tid; q < 3 * n_x + 2 * n_u; q += kSweepThreads) {
+    const void* src = q < n_x ? a.x_s : q < 2 * n_x ? a.x_max : q < 3 * n_x ? a.x_min : q < 3 * n_x + n_u ? a.u_max : a.u_min;
+    const int i = q < 3 * n_x ? q % n_x : (q - 3 * n_x) % n_u;
+    bnd[q] = reinterpret_cast<const VT*>(src)[i];
+  }
+  const VT c = (VT)a.cvec[prox ? nu - 1 : nu], cn = prox ? (VT)a.cvec[nu] : (VT)0;
+  __syncthreads();
   if (prox) {
-    const VT* delta = reinterpret_cast<const VT*>(a.h);
-    for (int r = warp; r < L; r += kWarps) {
-      const VT* src = delta + (long long)sid[r] * n_v;
-      for (int j = lane; j < n_v; j += 32) V[r * n_v + j] = src[j];
-    }
-    __syncthreads();
-    if (tid < n_v) {  // v along the path
-      VT v = 0;
-#pragma unroll 8
-      for (int r = 0; r < L; ++r) V[r * n_v + tid] = v += V[r * n_v + tid];
-    }
-    __syncthreads();
     const VT* E = reinterpret_cast<const VT*>(a.e);
     const VT* UH = reinterpret_cast<const VT*>(a.uhat);
-    sparse_rows<VT>(
-        ek, rptr, rid, n_k, V, n_v, 0, L,
-        [&](int r, int e) -> VT {
-          const long long m = sid[r];
-          return e < n_x ? E[m * n_x + e] : r >= own ? UH[m * n_u + e - n_x] : (VT)0;
-        },
+    for (int r = warp; r < L; r += NW) {
+      const long long m = sid[r];
+      for (int e = lane; e < n_x; e += 32) cp_async_elem(Z + r * n_k + e, E + m * n_x + e);
+      if (r >= own)
+        for (int i = lane; i < n_u; i += 32) cp_async_elem(Z + r * n_k + n_x + i, UH + m * n_u + i);
+    }
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (prox) {
+    const VT* delta = reinterpret_cast<const VT*>(a.h);
+    for (int r = warp; r < L; r += NW)
+      for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * n_v + j, delta + (long long)sid[r] * n_v + j);
+  }
+  const bool stop = early_exit(a, nu, mode, flag, true) || !tree_active(a, tree, nu);
+  cp_async_wait_all();
+  // the solve stopped, or this tree of a forest did (it keeps its iterates)
+  if (stop) return;
+  SweepOut<VT> o;
+  if (prox) {
+    __syncthreads();
+    if (tid < n_v)  // v along the path
+      run_sums(V, n_v, tid, 0, 1, L, (VT)0, [&](int r, VT v) { V[r * n_v + tid] = v; });
+    __syncthreads();
+    // x increments (Bbar v + e) and u; of path nodes only the tanks are used
+    sparse_rows<NW, VT>(
+        ek, rptr, rid, n_k, V, n_v, 0, L, [&](int r, int e) -> VT { return Z[r * n_k + e]; },
         [&](int r, int e, VT v) { Z[r * n_k + e] = v; });
     __syncthreads();
-    if (tid < n_x) {  // x_n = x_parent + Bbar v_n + e_n
-      VT x = reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid];
-#pragma unroll 8
-      for (int r = 0; r < L; ++r) Z[r * n_k + tid] = x += Z[r * n_k + tid];
-    }
+    if (tid < n_x)  // x_n = x_parent + Bbar v_n + e_n
+      run_sums(Z, n_k, tid, 0, 1, L, reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid],
+               [&](int r, VT v) { Z[r * n_k + tid] = v; });
     __syncthreads();
-    for (int r = own + warp; r < L; r += kWarps)
-      sweep_prox<VT, NT, NU>(a, sid[r], Z + r * n_k, bnd, nu, rmax, hmax, tmax);
+  }
+  if (len > 0 && (mode & MODE_BWD)) {  // beta, used after the prox
+    const VT* beta = reinterpret_cast<const VT*>(a.beta);
+    for (int r = own + warp; r < L; r += NW)
+      for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * n_v + j, beta + (long long)sid[r] * n_v + j);
+  }
+  if (prox) {
+    const int rows = L - own, ni = (n_u + 63) / 64;
+    for (int task = warp; task < rows * (1 + ni); task += NW) {
+      if (task < rows) {
+        const int r = own + task;
+        sweep_tanks<VT, NT>(a, sid[r], Z + r * n_k, bnd, nu - 1, c, cn, o);
+      } else {
+        const int q = (task - rows) / ni, r = own + q;
+        sweep_inputs<VT>(a, sid[r], 64 * (task - rows - q * ni), Z + r * n_k, bnd, nu - 1, c, cn, o);
+      }
+    }
+    if (o.r.bad() || o.h.bad()) a.flags[1] = SMPC_EDIVERGED;
   } else {  // w^nu without a prox: the first iteration
-    const VT c = (VT)a.cvec[nu];
     const int nd = 2 * n_x + n_u;
-    for (int r = own + warp; r < L; r += kWarps) {
+    for (int r = own + warp; r < L; r += NW) {
       const ST* ya = reinterpret_cast<const ST*>((nu & 1) ? a.ybuf1 : a.ybuf0) + (long long)sid[r] * nd;
       const ST* yb = reinterpret_cast<const ST*>((nu & 1) ? a.ybuf0 : a.ybuf1) + (long long)sid[r] * nd;
       for (int e = lane; e < n_k; e += 32) {
@@ -287,49 +405,93 @@ __global__ void __launch_bounds__(kThreads, NT == 8 ? 1 : sizeof(VT) == 4 ? 3 : 
     }
   }
   if (prox) {  // residual maxima (Sec. IV-E)
-    rmax = warp_max(rmax);
-    hmax = warp_max(hmax);
-    tmax = warp_max(tmax);
+    const VT rw = warp_max(o.r.value()), hw = warp_max(o.h.value()), tw = warp_max(o.t.value());
     if (lane == 0) {
-      red[warp] = rmax;
-      red[kWarps + warp] = hmax;
-      red[2 * kWarps + warp] = tmax;
+      red[warp] = rw;
+      red[NW + warp] = hw;
+      red[2 * NW + warp] = tw;
     }
   }
+  cp_async_wait_all();
   __syncthreads();
-  if (prox && tid < 3) {
+  if (prox && tid >= kSweepThreads - 3) {
+    const int k = kSweepThreads - 1 - tid;
     VT v = 0;
-    for (int w = 0; w < kWarps; ++w) v = fmax(v, red[tid * kWarps + w]);
-    atomic_max_nonneg(a.res + 3ll * (nu - 1) + tid, (double)v);
-    if (a.res_tree) atomic_max_nonneg(a.res_tree + 3ll * ((long long)(nu - 1) * a.R + tree) + tid, (double)v);
+    for (int w = 0; w < NW; ++w) v = fmax(v, red[k * NW + w]);
+    atomic_max_nonneg(a.res + 3ll * (nu - 1) + k, (double)v);
+    if (a.res_tree) atomic_max_nonneg(a.res_tree + 3ll * ((long long)(nu - 1) * a.R + tree) + k, (double)v);
   }
   if (!(mode & MODE_BWD)) return;
-  if (len == 0) {  // a top node: its w, for lambda_apply
+  if (len == 0) {  // a top node: its w
     VT* w = reinterpret_cast<VT*>(a.wbuf) + (long long)sid[own] * n_k;
-    for (int e = tid; e < n_k; e += kThreads) w[e] = Z[own * n_k + e];
-    return;
-  }
-  if (tid < n_x) {  // s along the chain, bottom-up
-    VT s = 0;
-#pragma unroll 8
-    for (int r = L - 1; r >= own; --r) Z[r * n_k + tid] = s += Z[r * n_k + tid];
-    reinterpret_cast<VT*>(a.spub)[(long long)sid[own] * n_x + tid] = s;
-  }
-  __syncthreads();
-  const VT* beta = reinterpret_cast<const VT*>(a.beta);
-  sparse_rows<VT>(
-      et, cptr, cid, n_v, Z, n_k, own, L, [&](int r, int j) -> VT { return beta[(long long)sid[r] * n_v + j]; },
-      [&](int r, int j, VT v) { V[r * n_v + j] = v; });
-  __syncthreads();
-  if (tid < n_v) {  // r along the chain
-    VT* R = reinterpret_cast<VT*>(a.rpub);
-    VT s = 0;
-#pragma unroll 8
-    for (int r = L - 1; r >= own; --r) {
-      s += V[r * n_v + tid];
-      R[(long long)sid[r] * n_v + tid] = s;
+    for (int e = tid; e < n_k; e += kSweepThreads) w[e] = Z[own * n_k + e];
+  } else {
+    if (tid < n_x) {  // s along the chain, bottom-up
+      VT s = 0;
+      run_sums(Z, n_k, tid, L - 1, -1, len, (VT)0, [&](int r, VT v) { Z[r * n_k + tid] = s = v; });
+      reinterpret_cast<VT*>(a.spub)[(long long)sid[own] * n_x + tid] = s;
+    }
+    __syncthreads();
+    sparse_rows<NW, VT>(
+        et, cptr, cid, n_v, Z, n_k, own, L, [&](int r, int j) -> VT { return V[r * n_v + j]; },
+        [&](int r, int j, VT v) { V[r * n_v + j] = v; });
+    __syncthreads();
+    if (tid < n_v) {  // r along the chain
+      VT* R = reinterpret_cast<VT*>(a.rpub);
+      run_sums(V, n_v, tid, L - 1, -1, len, (VT)0, [&](int r, VT v) { R[(long long)sid[r] * n_v + tid] = v; });
     }
   }
+  // the last of a top node and its chains adds up their xi and s, beta and r
+  const int t = d0.x;
+  if (t < 0) return;
+  __syncthreads();  // this CTA's outputs, then one fence, before its arrival
+  if (tid == 0) {
+    fence_acq_rel_gpu();
+    const int last = atomicAdd(&a.counters[t], 1) == a.chain_kids[t];
+    if (last) {
+      a.counters[t] = 0;
+      fence_acq_rel_gpu();
+    }
+    flag[1] = last;
+  }
+  __syncthreads();
+  if (!flag[1]) return;
+  const int c0 = a.child_begin[t], cc = a.child_count[t];
+  const VT* sp = reinterpret_cast<const VT*>(a.spub);
+  VT* rp = reinterpret_cast<VT*>(a.rpub);
+  VT* wt = reinterpret_cast<VT*>(a.wbuf) + (long long)t * n_k;
+  VT *S0 = Z, *R0 = Z + 2 * n_k;  // row 0: [S; 0], row 1: [0; psi], then R
+  for (int q = tid; q < n_x + n_k; q += kSweepThreads) {
+    if (q < n_x) {
+      S0[n_k + q] = 0;
+    } else {
+      const int e = q - n_x;
+      if (e < n_x) continue;
+      S0[e] = 0;
+      S0[n_k + e] = ldcg(wt + e);
+    }
+  }
+  for (int q = tid; q < n_x + n_v; q += kSweepThreads) {
+    const bool tank = q < n_x;
+    const VT* in = tank ? sp : rp;
+    const int cols = tank ? n_x : n_v, e = tank ? q : q - n_x;
+    ST sum = st_from<ST>(0.0);
+    st_fma_acc(sum, (VT)1, tank ? ldcg(wt + e) : reinterpret_cast<const VT*>(a.beta)[(long long)t * n_v + e]);
+    constexpr int C = 8;
+    for (int i = 0; i < cc; i += C) {  // children in index order, C loads in flight
+      VT v[C];
+#pragma unroll
+      for (int k = 0; k < C; ++k)
+        v[k] = i + k < cc && a.top_expect[c0 + i + k] == 0 ? ldcg(in + (long long)(c0 + i + k) * cols + e) : (VT)0;
+#pragma unroll
+      for (int k = 0; k < C; ++k) st_fma_acc(sum, (VT)1, v[k]);
+    }
+    (tank ? S0 : R0)[e] = st_val(sum);
+  }
+  __syncthreads();  // also: w has been read
+  sparse_rows<NW, VT>(
+      et, cptr, cid, n_v, Z, n_k, 0, 2, [&](int r, int j) -> VT { return r == 1 ? R0[j] : (VT)0; },
+      [&](int r, int j, VT v) { (r == 1 ? rp + (long long)t * n_v : wt)[j] = v; });
 }
 
 // ---------------------------------------------------------------- delta = Lambda r
@@ -365,181 +527,286 @@ __global__ void lam_pack_kernel(int n, int n_v, const double* Lam, const double*
   }
 }
 
-// Steps [k0, k1) of one matrix on a warp: acc += the part of Lambda r in row block `lane`.
-// rs: r, zero-padded to G BS entries, 16-byte aligned.
+// Steps [k0, k1) of one matrix (in shared or global memory) on a warp: acc += the part of
+// Lambda r in row block `lane`.  rs: r, zero-padded to G BS entries, 16-byte aligned.
+// Entries in pairs: two float32 in one register pair and one fused multiply-add instruction
+// (f32x2), or one float64.
+__device__ __forceinline__ unsigned long long f2(float x, float y) {
+  return (unsigned long long)__float_as_uint(x) | ((unsigned long long)__float_as_uint(y) << 32);
+}
+struct PairF {
+  using T = unsigned long long;
+  static constexpr int N = 2;
+  __device__ static T fma(T a, T b, T c) {
+    T d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+  }
+  __device__ static T dup(float x) { return f2(x, x); }
+  __device__ static T zero() { return 0; }
+  __device__ static float sum(T a) { return __uint_as_float((unsigned)a) + __uint_as_float((unsigned)(a >> 32)); }
+  __device__ static float at(T a, int k) { return __uint_as_float((unsigned)(k ? a >> 32 : a)); }
+  __device__ static void ld(const float* p, T (&o)[2]) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+    o[0] = t.x;
+    o[1] = t.y;
+  }
+};
+struct PairD {
+  using T = double;
+  static constexpr int N = 1;
+  __device__ static T fma(T a, T b, T c) { return ::fma(a, b, c); }
+  __device__ static T dup(double x) { return x; }
+  __device__ static T zero() { return 0; }
+  __device__ static double sum(T a) { return a; }
+  __device__ static double at(T a, int) { return a; }
+  __device__ static void ld(const double* p, T (&o)[2]) {
+    const double2 t = *reinterpret_cast<const double2*>(p);
+    o[0] = t.x;
+    o[1] = t.y;
+  }
+};
 template <typename VT, int BS>
-__device__ __forceinline__ void lam_steps(const VT* lam, int G, const VT* rs, int k0, int k1, VT (&acc)[BS]) {
-  constexpr int CE = 16 / (int)sizeof(VT), NC = BS * BS / CE;
-  constexpr int U = BS == 8 ? 1 : sizeof(VT) == 4 ? 4 : 2;  // steps whose loads are in flight together
+__device__ __forceinline__ void lam_steps(const VT* lam, int G, const VT* rs, int k0, int k1, VT (&out)[BS]) {
+  using P = typename std::conditional<sizeof(VT) == 4, PairF, PairD>::type;
+  using T = typename P::T;
+  constexpr int CE = 16 / (int)sizeof(VT);  // entries of a chunk: two pairs
+  constexpr int NC = BS * BS / CE, RC = BS / CE > 0 ? BS / CE : 1, NP = BS / P::N;
   const int lane = threadIdx.x & 31;
   const int I = lane < G ? lane : 0;  // idle lanes repeat lane 0's loads; nothing of theirs is used
-  VT ri[BS], tr[BS];
+  T ri[BS], acc[BS], tr[NP];
 #pragma unroll
   for (int r = 0; r < BS; ++r) {
-    ri[r] = rs[BS * I + r];
-    tr[r] = 0;
+    ri[r] = P::dup(rs[BS * I + r]);
+    acc[r] = P::zero();
   }
+#pragma unroll
+  for (int q = 0; q < NP; ++q) tr[q] = P::zero();
   const int from = I + 1 < G ? I + 1 : 0;
-  for (int kb = k0; kb < k1; kb += U) {
-    VT A[U][BS * BS];
+  const VT* blk = lam + ((long long)k0 * NC * G + I) * CE;
+  int J = I + k0 < G ? I + k0 : I + k0 - G;
+#pragma unroll 2
+  for (int k = k0; k < k1; ++k) {
+    T A[NC][2], rj[RC][2];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int k = min(kb + u, k1 - 1);
+    for (int c = 0; c < NC; ++c) P::ld(blk + (long long)c * G * CE, A[c]);
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        VT t[CE];
-        ld16(lam + ((long long)(k * NC + c) * G + I) * CE, t);
+    for (int c = 0; c < RC; ++c) P::ld(rs + BS * J + c * CE, rj[c]);
+    blk += (long long)NC * G * CE;
+    if (++J == G) J = 0;
+    if (k > 0) {  // the diagonal blocks are symmetric themselves
 #pragma unroll
-        for (int q = 0; q < CE; ++q) A[u][c * CE + q] = t[q];
-      }
+      for (int q = 0; q < NP; ++q) tr[q] = __shfl_sync(0xffffffffu, tr[q], from);
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) tr[(c % RC) * 2 + h] = P::fma(A[c][h], ri[c / RC], tr[(c % RC) * 2 + h]);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int k = kb + u;
-      if (k >= k1) break;
-      int J = I + k;
-      if (J >= G) J -= G;
-      const VT* rj = rs + BS * J;
+    for (int c = 0; c < NC; ++c)
 #pragma unroll
-      for (int q = 0; q < BS; ++q) tr[q] = __shfl_sync(0xffffffffu, tr[q], from);
-#pragma unroll
-      for (int r = 0; r < BS; ++r)
-#pragma unroll
-        for (int q = 0; q < BS; ++q) {
-          acc[r] += A[u][r * BS + q] * rj[q];
-          if (k > 0) tr[q] += A[u][r * BS + q] * ri[r];
-        }
-    }
+      for (int h = 0; h < 2; ++h) acc[c / RC] = P::fma(A[c][h], rj[c % RC][h], acc[c / RC]);
   }
   int back = (I - (k1 - 1)) % G;  // row block I's travelling sums are on lane I - (k1 - 1)
   if (back < 0) back += G;
 #pragma unroll
-  for (int q = 0; q < BS; ++q) acc[q] += __shfl_sync(0xffffffffu, tr[q], back);
+  for (int q = 0; q < NP; ++q) tr[q] = __shfl_sync(0xffffffffu, tr[q], back);
+#pragma unroll
+  for (int r = 0; r < BS; ++r) out[r] = P::sum(acc[r]) + P::at(tr[r / P::N], r % P::N);
 }
 
-// acc += w v, the product taken exactly
-__device__ __forceinline__ void st_fma_acc(DS& acc, float w, float v) { acc = st_axpy(acc, w, v); }
-__device__ __forceinline__ void st_fma_acc(double& acc, double w, double v) { acc = fma(w, v, acc); }
+constexpr int kTopList = 128;  // <= 256
+__device__ __forceinline__ void bar_top() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
-template <typename VT, int BS>
-__global__ void __launch_bounds__(kThreads) lambda_apply(const __grid_constant__ IterArgs a, int nu, int mode) {
+// Warps 0 .. LW - 1 of a CTA take chain nodes, warps LW .. LW + 7 the top nodes, side by side.
+// A chain warp owns one slot of shared memory, filled by a bulk copy of its next node's
+// matrix: the first copy is issued before the previous launch has drained (the matrices are
+// constants), the following ones as soon as the slot has been read, and with eight warps on an
+// SM (two CTAs) seven copies are in flight while one is used.  One matrix shared by all nodes
+// is copied once per CTA.  slots = 0: a matrix larger than shared memory is read in place.
+template <typename VT>
+__host__ __device__ inline size_t lambda_smem_bytes(int n_v, int slots) {
+  return (size_t)round_up((size_t)slots * lam_entries(n_v) * sizeof(VT), 128) + (size_t)kWarps * 32 * kStateSize +
+         (size_t)kWarps * 32 * lam_bs(n_v) * sizeof(VT);
+}
+
+template <typename VT, int BS, int LW>
+__global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 : 1)
+    lambda_apply(const __grid_constant__ IterArgs a, int slots, int nu, int mode) {
   using ST = typename St<VT>::T;
-  grid_dep_sync();
-  __shared__ int flag[2];
-  __shared__ __align__(16) VT rs[kWarps][32 * BS];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  if (early_exit(a, nu, mode, flag, false)) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n_x = a.n_x, n_k = a.n_k, n_v = a.n_v;
+  __shared__ int flag[2];
+  __shared__ __align__(16) VT rs[LW + 1][32 * BS];
+  __shared__ uint64_t bar[LW];
+  __shared__ int2 list[kTopList];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n_x = a.n_x, n_k = a.n_k, n_v = a.n_v, n_c = a.n - a.n_top;
   const int G = (n_v + BS - 1) / BS, steps = G / 2 + 1;
+  const long long per = lam_entries(n_v);
   const VT* lam = reinterpret_cast<const VT*>(a.lam);
   VT* delta = reinterpret_cast<VT*>(a.h);
-  if ((int)blockIdx.x >= a.n_top) {  // a warp per chain node
-    const int q = ((int)blockIdx.x - a.n_top) * kWarps + warp;
-    if (q >= a.n - a.n_top) return;
-    const long long m = a.chain_node[q];
-    const VT* r = reinterpret_cast<const VT*>(a.rpub) + m * n_v;
-    for (int j = lane; j < 32 * BS; j += 32) rs[warp][j] = j < n_v ? r[j] : (VT)0;
-    __syncwarp();
-    VT acc[BS] = {};
-    lam_steps<VT, BS>(lam + m * a.lam_stride, G, rs[warp], 0, steps, acc);
-    const VT sc = a.pscale ? reinterpret_cast<const VT*>(a.pscale)[m] : (VT)1;
-    if (lane < G) {
-#pragma unroll
-      for (int c = 0; c < BS; ++c)
-        if (BS * lane + c < n_v) delta[m * n_v + BS * lane + c] = acc[c] * sc;
-    }
+  const bool one = a.lam_stride == 0;  // one matrix for all nodes
+  const int cw = one || slots == 0 ? LW : slots;  // chain warps at work
+  VT* slot = reinterpret_cast<VT*>(smem_raw) + (one ? 0 : (long long)warp * per);
+  int q = (int)blockIdx.x * cw + warp;
+  const int dq = (int)gridDim.x * cw;
+  const bool chains = warp < cw && q < n_c;
+  auto fetch = [&](int m) {  // lane 0: node m's matrix into this warp's slot
+    mbar_expect_tx(&bar[warp], (uint32_t)(per * sizeof(VT)));
+    bulk_g2s(slot, lam + m * a.lam_stride, (uint32_t)(per * sizeof(VT)), &bar[warp]);
+  };
+  if (slots > 0 && warp < cw && lane == 0) {
+    mbar_init(&bar[warp], 1);
+    fence_barrier_init();
+    fence_proxy_async();
+    if (one ? warp == 0 : chains) fetch(one ? 0 : a.chain_node[q]);
+  }
+  const bool mine = one ? warp == 0 : chains;  // a copy of this warp's is under way
+  // the top warps: the first top node's sources into shared memory, its matrix towards the L2
+  const int tid = (int)threadIdx.x - LW * 32;
+  ST* part = reinterpret_cast<ST*>(smem_raw + round_up((size_t)slots * per * sizeof(VT), 128));  // ng n_v <= 256 sums
+  VT* lsum = reinterpret_cast<VT*>(part + kWarps * 32);  // the warps' parts of delta
+  const int2* src = reinterpret_cast<const int2*>(a.top_src);
+  int s0 = 0, s1 = 0, m_top = 0;
+  if (warp >= LW && (int)blockIdx.x < a.n_top) {
+    m_top = a.top_nodes[blockIdx.x];
+    s0 = a.top_src_off[blockIdx.x];
+    s1 = a.top_src_off[blockIdx.x + 1];
+    if (tid < min(kTopList, s1 - s0)) list[tid] = src[s0 + tid];
+    const char* lm = reinterpret_cast<const char*>(lam + m_top * a.lam_stride);
+    for (long long o = 128ll * tid; o < per * (long long)sizeof(VT); o += 128ll * 256)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(lm + o));
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (early_exit(a, nu, mode, flag, false)) {
+    if (slots > 0 && mine) mbar_wait(&bar[warp], 0);  // the copy lands (bounded) before the CTA leaves
     return;
   }
-  // a top node: [S; P | R] = the weighted sums of s (weights: top nodes between), psi and r
-  // (or beta) over the heads and top nodes below; then r = R + [Bbar; L]' [S; P].  These are
-  // sums of hundreds of terms that nearly cancel, and they move every scenario below: float32
-  // ones run in the state type (two float32), else the duals of the top nodes drift.
-  const int W = n_k + n_v;
-  ST* part = reinterpret_cast<ST*>(smem_raw);  // kWarps x W, in the state type (see above)
-  const long long m = a.top_nodes[blockIdx.x];
-  const VT* sp = reinterpret_cast<const VT*>(a.spub);
+  if (warp < LW) {
+    if (one && slots > 0 && warp != 0 && !chains) return;
+    uint32_t phase = 0;
+    // ids are read two nodes ahead and r one node ahead of their use
+    constexpr int RL = BS;  // 32 RL >= n_v
+    const bool any = warp < cw && q < n_c;
+    int m = any ? a.chain_node[q] : 0, m1 = any && q + dq < n_c ? a.chain_node[q + dq] : -1;
+    VT rn[RL], sc = 1;
+    auto read_r = [&](long long node) {
+#pragma unroll
+      for (int k = 0; k < RL; ++k) {
+        const int j = lane + 32 * k;
+        rn[k] = j < n_v ? reinterpret_cast<const VT*>(a.rpub)[node * n_v + j] : (VT)0;
+      }
+      if (a.pscale) sc = reinterpret_cast<const VT*>(a.pscale)[node];
+    };
+    if (any) read_r(m);
+    for (; q < n_c && warp < cw; q += dq) {
+      const int m2 = q + 2 * dq < n_c ? a.chain_node[q + 2 * dq] : -1;
+      const VT scale = sc;
+#pragma unroll
+      for (int k = 0; k < RL; ++k) rs[warp][lane + 32 * k] = rn[k];
+      if (m1 >= 0) read_r(m1);
+      if (slots > 0) {
+        const bool ok = mbar_wait(one ? &bar[0] : &bar[warp], one ? 0 : phase);
+        if (!__all_sync(0xffffffffu, ok)) {
+          if (lane == 0) a.flags[1] = SMPC_ETIMEOUT;
+          mbar_wait(one ? &bar[0] : &bar[warp], one ? 0 : phase);  // bounded: let the copy land
+          return;
+        }
+        phase ^= 1;
+      }
+      __syncwarp();
+      VT acc[BS] = {};
+      lam_steps<VT, BS>(slots > 0 ? slot : lam + m * a.lam_stride, G, rs[warp], 0, steps, acc);
+      __syncwarp();  // the slot and r have been read
+      if (slots > 0 && !one && lane == 0 && m1 >= 0) {
+        fence_proxy_async();
+        fetch(m1);
+      }
+      if (lane < G) {
+#pragma unroll
+        for (int c = 0; c < BS; ++c)
+          if (BS * lane + c < n_v) delta[(long long)m * n_v + BS * lane + c] = acc[c] * scale;
+      }
+      m = m1;
+      m1 = m2;
+    }
+    if (one && slots > 0 && warp == 0) mbar_wait(&bar[0], 0);  // bounded: also where it had no node
+    return;
+  }
+  // a top node: r = the sum of its sources' two terms.  These are sums of many terms that
+  // nearly cancel, and they move every scenario below: float32 ones run in the state type (two
+  // float32), else the duals of the top nodes drift (plain sums over the chains: errors 3 to 8
+  // times those of sums along the tree).
+  const int tw = warp - LW;
+  VT* rt = rs[LW];
   const VT* rp = reinterpret_cast<const VT*>(a.rpub);
   const VT* wb = reinterpret_cast<const VT*>(a.wbuf);
-  const VT* beta = reinterpret_cast<const VT*>(a.beta);
-  const int h0 = a.top_src_off[2 * blockIdx.x], t0 = a.top_src_off[2 * blockIdx.x + 1],
-            t1 = a.top_src_off[2 * blockIdx.x + 2];
-  // a warp takes every kWarps-th source with all its columns in flight
-  constexpr int NC = 8;  // 32 NC >= n_k, n_v
-  const int2* src = reinterpret_cast<const int2*>(a.top_src);
-  ST y[NC], g[NC];  // [S; P] and R, columns lane + 32 k
-#pragma unroll
-  for (int k = 0; k < NC; ++k) y[k] = g[k] = st_from<ST>(0.0);
-#pragma unroll 4
-  for (int q = h0 + warp; q < t0; q += kWarps) {
-    const int2 s = src[q];
-#pragma unroll
-    for (int k = 0; k < NC; ++k) {
-      const int e = lane + 32 * k;
-      if (e < n_x) st_fma_acc(y[k], (VT)s.y, sp[(long long)s.x * n_x + e]);
-      if (e < n_v) st_fma_acc(g[k], (VT)1, rp[(long long)s.x * n_v + e]);
+  for (int t = blockIdx.x; t < a.n_top; t += gridDim.x) {
+    const bool first = t == (int)blockIdx.x;
+    if (!first) {
+      m_top = a.top_nodes[t];
+      s0 = a.top_src_off[t];
+      s1 = a.top_src_off[t + 1];
     }
-  }
-#pragma unroll 2
-  for (int q = t0 + warp; q < t1; q += kWarps) {
-    const int2 s = src[q];
+    const long long m = m_top;
+    // with 2 ng <= 8 warps a group of threads takes one column of every ng-th source, eight
+    // sources (sixteen loads) in flight; the ids go through shared memory, kTopList at a time
+    const int gw = (n_v + 31) / 32, ng = kWarps / gw, grp = tid / (32 * gw), j = tid - grp * 32 * gw;
+    const bool on = grp < ng && j < n_v;
+    ST sum = st_from<ST>(0.0);
+    for (int i0 = s0; i0 < s1; i0 += kTopList) {
+      const int cnt = min(kTopList, s1 - i0);
+      if (!first || i0 > s0) {
+        bar_top();  // the previous list has been used
+        if (tid < cnt) list[tid] = src[i0 + tid];
+        bar_top();
+      }
+      constexpr int B = 8;
+      if (on)
+        for (int i = grp; i < cnt; i += B * ng) {
+          VT v[B], w[B];
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
-      const int e = lane + 32 * k;
-      if (e < n_k) st_fma_acc(y[k], e < n_x ? (VT)s.y : (VT)1, wb[(long long)s.x * n_k + e]);
-      if (e < n_v) st_fma_acc(g[k], (VT)1, beta[(long long)s.x * n_v + e]);
+          for (int k = 0; k < B; ++k) {  // behind the end: the last source again, not added
+            const long long id = list[min(i + k * ng, cnt - 1)].x;
+            v[k] = rp[id * n_v + j];
+            w[k] = wb[id * n_k + j];
+          }
+#pragma unroll
+          for (int k = 0; k < B; ++k)
+            if (i + k * ng < cnt) {
+              st_fma_acc(sum, (VT)1, v[k]);
+              st_fma_acc(sum, (VT)list[i + k * ng].y, w[k]);
+            }
+        }
     }
-  }
-#pragma unroll
-  for (int k = 0; k < NC; ++k) {
-    const int e = lane + 32 * k;
-    if (e < n_k) part[warp * W + e] = y[k];
-    if (e < n_v) part[warp * W + n_k + e] = g[k];
-  }
-  __syncthreads();
-  for (int e = tid; e < W; e += kThreads) {
-    ST v = part[e];
-#pragma unroll
-    for (int w = 1; w < kWarps; ++w) v = st_add(v, part[w * W + e]);
-    part[e] = v;  // entry e of every warp's row is read and written by this thread only
-  }
-  __syncthreads();
-  const int nnz = a.sp_nnz;
-  const SpEnt<VT>* et = reinterpret_cast<const SpEnt<VT>*>(a.sp) + nnz;
-  const int* rptr = reinterpret_cast<const int*>(et + nnz);
-  const int *cptr = rptr + 2 * n_k + 1, *cid = cptr + n_v + 1;
-  for (int j = tid; j < 32 * BS; j += kThreads) {
-    if (j < n_v) {
-      const int col = cid[j];
-      ST v = part[n_k + col];
-      for (int q = cptr[j]; q < cptr[j + 1]; ++q) v = st_add(v, st_scale(part[et[q].c], et[q].v));
-      rs[0][col] = st_val(v);
-    } else {
-      rs[0][j] = 0;
+    if (on) part[grp * n_v + j] = sum;
+    bar_top();
+    if (tid < 32 * BS) {
+      ST v = st_from<ST>(0.0);
+      if (tid < n_v) {
+        v = part[tid];
+        for (int g = 1; g < ng; ++g) v = st_add(v, part[g * n_v + tid]);
+      }
+      rt[tid] = st_val(v);
     }
-  }
-  __syncthreads();
-  // the steps shared by the warps, their sums added in order
-  const int k0 = steps * warp / kWarps, k1 = steps * (warp + 1) / kWarps;
-  VT acc[BS] = {};
-  if (k0 < k1) lam_steps<VT, BS>(lam + m * a.lam_stride, G, rs[0], k0, k1, acc);
-  __syncthreads();  // part is free
-  VT* lsum = reinterpret_cast<VT*>(smem_raw);
-  if (lane < G) {
+    bar_top();
+    // the steps shared by the warps, their sums added in order
+    const int k0 = steps * tw / kWarps, k1 = steps * (tw + 1) / kWarps;
+    VT acc[BS] = {};
+    if (k0 < k1) lam_steps<VT, BS>(lam + m * a.lam_stride, G, rt, k0, k1, acc);
+    if (lane < G) {
 #pragma unroll
-    for (int c = 0; c < BS; ++c) lsum[warp * (32 * BS) + BS * lane + c] = acc[c];
-  }
-  __syncthreads();
-  const VT sc = a.pscale ? reinterpret_cast<const VT*>(a.pscale)[m] : (VT)1;
-  for (int j = tid; j < n_v; j += kThreads) {
-    VT v = 0;
+      for (int c = 0; c < BS; ++c) lsum[tw * (32 * BS) + BS * lane + c] = acc[c];
+    }
+    bar_top();
+    const VT sc = a.pscale ? reinterpret_cast<const VT*>(a.pscale)[m] : (VT)1;
+    for (int j = tid; j < n_v; j += 256) {
+      VT v = 0;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) v += lsum[w * (32 * BS) + j];
-    delta[m * n_v + j] = v * sc;
+      for (int w = 0; w < kWarps; ++w) v += lsum[w * (32 * BS) + j];
+      delta[m * n_v + j] = v * sc;
+    }
+    // part is rewritten behind the next top node's first barrier, lsum behind later ones
   }
-}
-template <typename VT>
-__host__ __device__ inline size_t lambda_smem_bytes(int n_k, int n_v) {
-  const int W = n_k + n_v, R = 32 * lam_bs(n_v);
-  return (size_t)kWarps * (W > R ? W : R) * kStateSize;
 }
