@@ -968,9 +968,40 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
     return SMPC_OK;
   };
   if ((rc = up64(&f->K64, K.data(), K.size())) || (rc = up64(&f->Lam64, f->hf.Lam.data(), f->hf.Lam.size())) ||
-      (rc = up64(&f->Pu, f->hf.Pu.data(), f->hf.Pu.size())) || (rc = up64(&f->Pe, f->hf.Pe.data(), f->hf.Pe.size())) ||
       (rc = up64(&f->Rhat, f->hf.Rhat.data(), f->hf.Rhat.size())) || (rc = up64(&f->L, f->hf.L.data(), f->hf.L.size())) ||
       (rc = up64(&f->alpha1, cost->alpha1, n_u)))
+    return fail(rc);
+  auto up_csr = [&](CsrRows* out, int rows, int cols, auto&& at) -> int {
+    std::vector<int> ptr(1, 0), col;
+    std::vector<double> val;
+    for (int i = 0; i < rows; ++i) {
+      for (int j = 0; j < cols; ++j)
+        if (at(i, j) != 0.0) {
+          col.push_back(j);
+          val.push_back(at(i, j));
+        }
+      ptr.push_back((int)col.size());
+    }
+    int *dp = nullptr, *dc = nullptr;
+    double* dv = nullptr;
+    TRY(f->alloc(&dp, ptr.size() * sizeof(int)));
+    TRY(f->alloc(&dc, col.size() * sizeof(int)));
+    TRY(up64(&dv, val.data(), val.size()));
+    CK(cudaMemcpy(dp, ptr.data(), ptr.size() * sizeof(int), cudaMemcpyHostToDevice));
+    if (!col.empty()) CK(cudaMemcpy(dc, col.data(), col.size() * sizeof(int), cudaMemcpyHostToDevice));
+    out->ptr = dp;
+    out->col = dc;
+    out->val = dv;
+    return SMPC_OK;
+  };
+  size_t rhat_nnz = 0;
+  for (double v : f->hf.Rhat) rhat_nnz += v != 0.0;
+  if ((rc = up_csr(&f->pue, n_u + n_x, n_d, [&](int i, int j) {
+         return i < n_u ? f->hf.Pu[(size_t)i * n_d + j] : f->hf.Pe[(size_t)(i - n_u) * n_d + j];
+       })) ||
+      // a dense Rhat (the orthonormal basis, coupled input weights) is read by coalesced columns
+      (4 * rhat_nnz <= f->hf.Rhat.size() &&
+       (rc = up_csr(&f->rhat_t, n_v, n_u, [&](int i, int j) { return f->hf.Rhat[(size_t)j * n_v + i]; }))))
     return fail(rc);
   // ---- packs: one per node, or one shared pack (Lambda unscaled) and the node scales
   f->shared_packs = o.shared_packs != 0;
@@ -1273,8 +1304,8 @@ int solve_begin(smpc_factor_t* f, const smpc_step_data* data, const smpc_solve_o
   c.child_count = f->tree->dev.child_count;
   c.prob = f->tree->dev.prob;
   c.pbar = f->tree->dev.pbar;
-  c.Pu = f->Pu;
-  c.Pe = f->Pe;
+  c.pue = f->pue;
+  c.rhat_t = f->rhat_t;
   c.Rhat = f->Rhat;
   c.L = f->L;
   c.alpha1 = f->alpha1;

@@ -2509,19 +2509,31 @@ __global__ void cost_alpha_kernel(CostArgs a) {
     }
 }
 
+// Rows of a matrix by their nonzero entries, in the order of a dense row (the sums round the
+// same way).  A network couples few inputs and demands: Pu and Pe of the 63-tank network have
+// 260 of 15 576 entries, and W_u L is about as sparse in the reduced basis; the float64 pipe
+// (2 lanes a cycle and SM) set the time of the dense rows.
+__device__ __forceinline__ double csr_row(const CsrRows& m, int row, const double* x) {
+  double s = 0;
+  for (int q = m.ptr[row]; q < m.ptr[row + 1]; ++q) s += m.val[q] * x[m.col[q]];
+  return s;
+}
+
 template <typename VT>
 __global__ void cost_uhat_kernel(CostArgs a) {
   // d_n = dhat_j + eps_n ; u_hat_n = Pu d_n ; e_n = Pe d_n
   extern __shared__ double dsh[];
   for (int m = blockIdx.x; m < a.n; m += gridDim.x) {
     const int j = a.stage[m];
-    for (int i = threadIdx.x; i < a.n_d; i += blockDim.x)
-      dsh[i] = a.dhat[(long long)j * a.n_d + i] + a.eps[(long long)m * a.n_d + i];
-    __syncthreads();
+    bool bad = false;  // a non-finite disturbance makes every entry NaN, also those it does not reach
+    for (int i = threadIdx.x; i < a.n_d; i += blockDim.x) {
+      const double d = a.dhat[(long long)j * a.n_d + i] + a.eps[(long long)m * a.n_d + i];
+      bad |= (__double2hiint(d) & 0x7ff00000) == 0x7ff00000;
+      dsh[i] = d;
+    }
+    bad = __syncthreads_or(bad);
     for (int i = threadIdx.x; i < a.n_u + a.n_x; i += blockDim.x) {
-      const double* row = (i < a.n_u) ? a.Pu + (long long)i * a.n_d : a.Pe + (long long)(i - a.n_u) * a.n_d;
-      double s = 0;
-      for (int k = 0; k < a.n_d; ++k) s += row[k] * dsh[k];
+      const double s = bad ? __longlong_as_double(0x7ff8000000000000ll) : csr_row(a.pue, i, dsh);
       if (i < a.n_u) {
         a.uhat64[(long long)m * a.n_u + i] = s;
         reinterpret_cast<VT*>(a.uhat)[(long long)m * a.n_u + i] = (VT)s;
@@ -2541,17 +2553,22 @@ __global__ void cost_beta_kernel(CostArgs a) {
     const double pm = a.prob[m];
     const int par = a.parent[m];
     const int cb = a.child_begin[m], cc = a.child_count[m];
+    bool bad = false;
     for (int i = threadIdx.x; i < a.n_u; i += blockDim.x) {
       double D = a.pbar[m] * a.uhat64[(long long)m * a.n_u + i];
       D -= pm * (par >= 0 ? a.uhat64[(long long)par * a.n_u + i] : a.q[(long long)a.tree_of[m] * a.n_u + i]);
       for (int c = cb; c < cb + cc; ++c) D -= a.prob[c] * a.uhat64[(long long)c * a.n_u + i];
+      bad |= (__double2hiint(D) & 0x7ff00000) == 0x7ff00000;
       Dsh[i] = D;
     }
-    __syncthreads();
+    bad = __syncthreads_or(bad);
     const int j = a.stage[m];
     for (int k = threadIdx.x; k < a.n_v; k += blockDim.x) {
       double s = 0;
-      for (int i = 0; i < a.n_u; ++i) s += a.Rhat[(long long)i * a.n_v + k] * Dsh[i];
+      if (a.rhat_t.ptr)
+        s = bad ? __longlong_as_double(0x7ff8000000000000ll) : csr_row(a.rhat_t, k, Dsh);
+      else
+        for (int i = 0; i < a.n_u; ++i) s += a.Rhat[(long long)i * a.n_v + k] * Dsh[i];
       reinterpret_cast<VT*>(a.beta)[(long long)m * a.n_v + k] = (VT)(pm * a.abar[(long long)j * a.n_v + k] + 2.0 * s);
     }
     __syncthreads();

@@ -285,8 +285,8 @@ extern "C" int smpc_solve_static(smpc_factor_t* f, const smpc_step_data* data, c
   c.child_count = f->tree->dev.child_count;
   c.prob = f->tree->dev.prob;
   c.pbar = f->tree->dev.pbar;
-  c.Pu = f->Pu;
-  c.Pe = f->Pe;
+  c.pue = f->pue;
+  c.rhat_t = f->rhat_t;
   c.Rhat = f->Rhat;
   c.L = f->L;
   c.alpha1 = f->alpha1;

@@ -241,6 +241,11 @@ int launch_pack(int prec, int n, int n_k, int n_v, const double* K, const double
 long long lam_pack_entries(int n_v);
 int launch_lam_pack(int prec, int n, int n_v, const double* Lam, const double* prob, void* out, void* stream);
 std::vector<unsigned char> sparse_image(int prec, int n_k, int n_v, const double* K);
+struct CsrRows {  // rows of a matrix by their nonzero entries (device arrays)
+  const int* ptr = nullptr;
+  const int* col = nullptr;
+  const double* val = nullptr;
+};
 struct CostArgs {
   int n, N, n_x, n_u, n_d, n_v;  // N: rows of stage-indexed data (sum of the trees' horizons)
   const int* parent;
@@ -250,8 +255,8 @@ struct CostArgs {
   const int* child_count;
   const double* prob;
   const double* pbar;
-  const double* Pu;       // n_u x n_d
-  const double* Pe;       // n_x x n_d
+  CsrRows pue;            // Pu (n_u x n_d) over Pe (n_x x n_d)
+  CsrRows rhat_t;         // Rhat' (n_v x n_u) where it is sparse (ptr NULL: Rhat below)
   const double* Rhat;     // n_u x n_v
   const double* L;        // n_u x n_v
   const double* alpha1;   // n_u
@@ -346,7 +351,8 @@ struct smpc_factor_t {
   void* packs32 = nullptr;    // SMPC_BF16 only: float32 packs (anchor and polish launches)
   long long pack_stride32 = 0;
   void *ha = nullptr, *wa = nullptr;  // SMPC_BF16 only: anchor h and w, n x n_k each
-  double *K64 = nullptr, *Lam64 = nullptr, *Pu = nullptr, *Pe = nullptr, *Rhat = nullptr, *L = nullptr;
+  double *K64 = nullptr, *Lam64 = nullptr, *Rhat = nullptr, *L = nullptr;
+  smpc::CsrRows pue, rhat_t;  // cost update: [Pu; Pe], and Rhat' where it is sparse
   double *alpha1 = nullptr, *uhat64 = nullptr, *abar = nullptr;
   double *d_p = nullptr, *d_q = nullptr, *d_dhat = nullptr, *d_eps = nullptr, *d_alpha2 = nullptr;
   void *ybuf0 = nullptr, *ybuf1 = nullptr, *wbuf = nullptr, *h = nullptr, *uhat = nullptr, *e = nullptr, *beta = nullptr;
