@@ -129,7 +129,7 @@ SWEEP_STAGES = ["tree_sweep", "lambda_apply"]  # the two-launch form of schedule
 
 
 def stages_of(schedule, stage_ms):
-    return SWEEP_STAGES if schedule == 4 and len(stage_ms) == 2 else STAGES[schedule]
+    return SWEEP_STAGES if len(stage_ms) == 2 else STAGES[schedule]
 
 
 def stage_bytes(stage, n, n_x, n_u, n_v, prec, shared):

@@ -122,9 +122,10 @@ typedef struct smpc_factor_opts {
    * pass up to r, and the node-parallel Lambda / [Bbar; L] launch; 4 = node-parallel forward
    * sweep and prox, then the whole backward sweep as one chain pass (every pack read once
    * per iteration); 0 = time all of them on this GPU when the factor is built and keep the
-   * fastest.  Where [Bbar; L] is sparse (at most 4096 entries in the reduced basis, A = I,
+   * fastest.  Where [Bbar; L] is sparse (at most 4096 entries in the reduced basis,
    * float64 or float32) 0 also times a two-launch form of 4 - a tree pass with the sparse
-   * products inside, and Lambda r of every node - which is reported as 4.  Results agree to
+   * products inside, and Lambda r of every node - which is reported as 4 (with a general A,
+   * as 2).  Results agree to
    * rounding. */
   int32_t schedule;
   /* SMPC_BF16 with shared_packs = 1: the Lambda and [Bbar; L] products of the delta
@@ -350,7 +351,7 @@ void smpc_shard_destroy(smpc_shard* shard);
  * [Bbar; L]' mat-vec, subtree scan of r, Lambda and [Bbar; L] mat-vecs) and 4 for schedule 3
  * (forward sweep; prox and dual update; s, [Bbar; L]' mat-vecs and r along the chains; Lambda
  * and [Bbar; L] mat-vecs) and 3 for schedule 4 (forward sweep; prox and dual update; the
- * whole backward sweep along the chains; n = 2 for its two-launch form: tree pass; Lambda r).
+ * whole backward sweep along the chains; n = 2 for the two-launch form: tree pass; Lambda r).
  * SMPC_BF16 anchor iterations are not timed.  Leaves
  * the factor's duals as that solve ends.  Returns n, or minus an smpc_status. */
 int smpc_profile_solve(smpc_factor_t* fac, const smpc_step_data* data, int32_t iters, double* stage_ms,

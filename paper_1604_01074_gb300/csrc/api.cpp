@@ -1026,9 +1026,9 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
     if ((rc = f->alloc(&f->ha, hb)) || (rc = f->alloc(&f->wa, hb))) return fail(rc);
     if (cudaMemset(f->ha, 0, hb) != cudaSuccess || cudaMemset(f->wa, 0, hb) != cudaSuccess) return fail(SMPC_ECUDA);
   }
-  // ---- the two-launch form of schedule 4: only a factor that may choose its schedule
+  // ---- the two-launch form of schedule 4 (with a general A: of schedule 2): only a factor that may choose its schedule
   const size_t lam_bytes = (size_t)np * lam_pack_entries(n_v) * f->vs;
-  if (o.schedule == 0 && f->prec != SMPC_BF16 && !general_A && !tree->top_src_off.empty()) {
+  if (o.schedule == 0 && f->prec != SMPC_BF16 && !tree->top_src_off.empty()) {
     for (double v : K) f->sp_nnz += v != 0.0;
     if (f->sp_nnz <= kSparseMax) {
       const std::vector<unsigned char> image = sparse_image(f->prec, n_k, n_v, K.data());
@@ -1211,10 +1211,12 @@ int smpc_factor_schedule(const smpc_factor_t* f, double* ms_per_iter) {
     ms_per_iter[0] = f->tuned_ms[SCHED_CHAIN];
     ms_per_iter[1] = f->tuned_ms[SCHED_NODE];
     ms_per_iter[2] = f->tuned_ms[SCHED_HYBRID];
-    const float sw = f->tuned_ms[SCHED_SWEEP];  // its two-launch form, where that was timed and is faster
-    ms_per_iter[3] = sw > 0 && sw < f->tuned_ms[SCHED_FUSED] ? sw : f->tuned_ms[SCHED_FUSED];
+    ms_per_iter[3] = f->tuned_ms[SCHED_FUSED];
+    const float sw = f->tuned_ms[SCHED_SWEEP];  // the two-launch form, where that was timed and is faster
+    double& as = ms_per_iter[(f->A ? SCHED_NODE : SCHED_FUSED) - 1];
+    if (sw > 0 && sw < as) as = sw;
   }
-  return f->schedule == SCHED_SWEEP ? (int)SCHED_FUSED : f->schedule;
+  return f->schedule == SCHED_SWEEP ? (int)(f->A ? SCHED_NODE : SCHED_FUSED) : f->schedule;
 }
 
 int smpc_factor_tc_width(const smpc_factor_t* f, double* ms_per_width) {

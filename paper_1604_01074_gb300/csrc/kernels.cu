@@ -3239,17 +3239,17 @@ LaunchCfg config_t(const IterArgs& a, int num_sms, int S_max, int schedule, int 
   c.schedule = schedule;
   c.block = kThreads;
   const bool fits_threads = a.n_k <= kThreads && a.n_v <= kThreads;  // one thread per entry
-  if (schedule == SCHED_SWEEP) {  // sparse [Bbar; L] and packed Lambda of the vector type, A = I
+  if (schedule == SCHED_SWEEP) {  // sparse [Bbar; L] and packed Lambda of the vector type
     c.stages = 0;
     if constexpr (std::is_same<VT, MT>::value) {
-      c.smem = sweep_smem_bytes<VT>(a.sp_nnz, a.depth, a.n_x, a.n_u, a.n_v);
+      c.smem = sweep_smem_bytes<VT>(a.sp_nnz, a.depth, a.n_x, a.n_u, a.n_v, a.A != nullptr);
       c.grid = a.n_chains + a.n_top;
       const int tasks = a.max_len * (1 + (a.n_u + 63) / 64);  // of a chain's prox, one warp each
       c.sweep_warps = a.n_x > 64 ? 16
                       : a.n_chains > 2 * num_sms || tasks <= 8 ? 8
                       : a.n_chains <= num_sms && tasks >= 48 && sizeof(VT) == 4 ? 32 : 16;
       // Lambda: matrix slots for four chain warps where two CTAs fit an SM, else as many as fit
-      const int n_c = a.n - a.n_top;
+      const int n_c = a.A ? a.n : a.n - a.n_top;
       const int ctas = sizeof(VT) == 4 && lam_bs(a.n_v) == 4 ? 2 : 1;  // CTAs an SM, by registers
       const size_t room = (size_t)optin / ctas - (ctas == 2 ? 8192 : 24576);
       // float64: the pipe, not the copies, sets the time, and eight warps reading in place keep
@@ -3260,8 +3260,8 @@ LaunchCfg config_t(const IterArgs& a, int num_sms, int S_max, int schedule, int 
       c.smem_lam = lambda_smem_bytes<VT>(a.n_v, c.lam_slots);
       c.lam_warps = a.lam_stride == 0 || sizeof(VT) == 8 ? 8 : 4;  // chain warps a CTA
       const int cw = c.lam_slots == 0 || a.lam_stride == 0 ? c.lam_warps : c.lam_slots;
-      c.grid_lam = std::min(std::max((n_c + cw - 1) / cw, a.n_top), ctas * num_sms);
-      if (a.lam && a.sp && fits_threads && !a.A && c.smem + 512 <= (size_t)optin) c.stages = 1;
+      c.grid_lam = std::min(std::max((n_c + cw - 1) / cw, a.A ? 1 : a.n_top), ctas * num_sms);
+      if (a.lam && a.sp && fits_threads && c.smem + 512 <= (size_t)optin) c.stages = 1;
     }
     return c;
   }

@@ -187,7 +187,8 @@ enum Schedule : int {
 };
 constexpr int kSchedules = 4;
 // The form of schedule 4 that a factor may choose by timing where [Bbar; L] is sparse: one
-// tree pass and one Lambda launch per iteration (sweep.cuh).  Reported as schedule 4.
+// tree pass and one Lambda launch per iteration (sweep.cuh).  Reported as schedule 4, with a
+// general A as schedule 2, the one that carries it.
 constexpr int SCHED_SWEEP = 5;
 // Entries of [Bbar; L] up to which it counts as sparse: its image is read into shared memory
 // by every CTA of the tree pass (64 KB at this size in float32).

@@ -15,6 +15,9 @@
 //                         R_m + L' psi_m + c Bbar' S_m,
 //                 c the number of top nodes from t down to m.  The last of m's chains and m
 //                 itself forms the two terms in tree_sweep, so no top node waits for another.
+// A general A: x and s along a chain take one product with A per node (A in shared memory, a
+// block barrier each), and s and r of the top nodes climb in tree_sweep.  1531 nodes of a
+// 50-tank network: 45 us an iteration, against 128 us of the six launches of schedule 2.
 // Per iteration on GB300, one pack per node (the launches of schedules 2 to 4 before): 2081
 // nodes 27.2 us in float32 (104), 116 us in float64 (381); 21 111 nodes 145 us (577), the tree
 // pass 71 and Lambda 75; one pack for all of 21 111 nodes 107 us (396).  The tree pass is bound
@@ -81,10 +84,11 @@ __device__ __forceinline__ void st_fma_acc(DS& acc, float w, float v) { acc = st
 __device__ __forceinline__ void st_fma_acc(double& acc, double w, double v) { acc = fma(w, v, acc); }
 
 template <typename VT>
-__host__ __device__ inline size_t sweep_smem_bytes(int nnz, int depth, int n_x, int n_u, int n_v) {
+__host__ __device__ inline size_t sweep_smem_bytes(int nnz, int depth, int n_x, int n_u, int n_v, bool general_A) {
   const int n_k = n_x + n_u;
   size_t b = sp_bytes<VT>(nnz, n_k, n_v);
   b += (size_t)(3 * n_x + 2 * n_u + (depth + 3) * (n_v + n_k)) * sizeof(VT);  // depth + 3 >= 4 rows: the last arrival's too
+  if (general_A) b += (size_t)n_x * n_x * sizeof(VT);
   return round_up(b + (size_t)depth * sizeof(int), 16);
 }
 
@@ -292,6 +296,21 @@ __device__ __forceinline__ void run_sums(VT* X, int xs, int col, int r0, int dr,
   }
 }
 
+// out[e] += (A x)_e (trans: (A' x)_e) for e < n, A in shared memory: eight lanes a row.
+template <int NW, typename VT>
+__device__ __forceinline__ void add_Ax(const VT* A, int n, bool trans, const VT* x, VT* out) {
+  const int lane = threadIdx.x & 31, part = lane & 7;
+  for (int e0 = (threadIdx.x >> 5) * 4; e0 < n; e0 += NW * 4) {
+    const int e = e0 + (lane >> 3);
+    VT v = 0;
+    if (e < n)
+      for (int j = part; j < n; j += 8) v += (trans ? A[j * n + e] : A[e * n + j]) * x[j];
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    if (part == 0 && e < n) out[e] += v;
+  }
+}
+
 // NW warps a CTA at 64 registers a thread (float64: 128).  Most phases of a segment wait on
 // memory or shared memory with few warps busy, so trees with several chains an SM run four
 // small CTAs there, side by side in different phases; trees with at most a chain an SM have
@@ -319,7 +338,10 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
   VT* bnd = reinterpret_cast<VT*>(smem_raw + blob);
   VT* V = bnd + 3 * n_x + 2 * n_u;  // delta, then v, then beta, g and r: a row of n_v per node
   VT* Z = V + (a.depth + 3) * n_v;  // e and u_hat, then x and u, then w and s: a row of n_k per node
-  int* sid = reinterpret_cast<int*>(Z + (a.depth + 3) * n_k);
+  VT* As = Z + (a.depth + 3) * n_k;  // a general state matrix
+  int* sid = reinterpret_cast<int*>(As + (a.A ? n_x * n_x : 0));
+  if (a.A)
+    for (int q = tid; q < n_x * n_x; q += kSweepThreads) As[q] = reinterpret_cast<const VT*>(a.A)[q];
   // chains first (the long tasks), then the top nodes
   const int b = (int)blockIdx.x < a.n_chains ? a.n_top + blockIdx.x : blockIdx.x - a.n_chains;
   const int4 d0 = *reinterpret_cast<const int4*>(a.seg + (long long)kSegInts * b);
@@ -368,7 +390,13 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
         ek, rptr, rid, n_k, V, n_v, 0, L, [&](int r, int e) -> VT { return Z[r * n_k + e]; },
         [&](int r, int e, VT v) { Z[r * n_k + e] = v; });
     __syncthreads();
-    if (tid < n_x)  // x_n = x_parent + Bbar v_n + e_n
+    if (a.A) {  // x_n = A x_parent + Bbar v_n + e_n (App. B), a barrier a node
+      if (tid < n_x) Z[L * n_k + tid] = reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid];
+      for (int r = 0; r < L; ++r) {
+        __syncthreads();
+        add_Ax<NW>(As, n_x, false, Z + (r > 0 ? r - 1 : L) * n_k, Z + r * n_k);
+      }
+    } else if (tid < n_x)  // x_n = x_parent + Bbar v_n + e_n
       run_sums(Z, n_k, tid, 0, 1, L, reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid],
                [&](int r, VT v) { Z[r * n_k + tid] = v; });
     __syncthreads();
@@ -426,7 +454,13 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
     VT* w = reinterpret_cast<VT*>(a.wbuf) + (long long)sid[own] * n_k;
     for (int e = tid; e < n_k; e += kSweepThreads) w[e] = Z[own * n_k + e];
   } else {
-    if (tid < n_x) {  // s along the chain, bottom-up
+    if (a.A) {  // s_n = xi_n + A' s_child
+      for (int r = L - 2; r >= own; --r) {
+        add_Ax<NW>(As, n_x, true, Z + (r + 1) * n_k, Z + r * n_k);
+        __syncthreads();
+      }
+      if (tid < n_x) reinterpret_cast<VT*>(a.spub)[(long long)sid[own] * n_x + tid] = Z[own * n_k + tid];
+    } else if (tid < n_x) {  // s along the chain, bottom-up
       VT s = 0;
       run_sums(Z, n_k, tid, L - 1, -1, len, (VT)0, [&](int r, VT v) { Z[r * n_k + tid] = s = v; });
       reinterpret_cast<VT*>(a.spub)[(long long)sid[own] * n_x + tid] = s;
@@ -441,57 +475,68 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
       run_sums(V, n_v, tid, L - 1, -1, len, (VT)0, [&](int r, VT v) { R[(long long)sid[r] * n_v + tid] = v; });
     }
   }
-  // the last of a top node and its chains adds up their xi and s, beta and r
-  const int t = d0.x;
-  if (t < 0) return;
-  __syncthreads();  // this CTA's outputs, then one fence, before its arrival
-  if (tid == 0) {
-    fence_acq_rel_gpu();
-    const int last = atomicAdd(&a.counters[t], 1) == a.chain_kids[t];
-    if (last) {
-      a.counters[t] = 0;
-      fence_acq_rel_gpu();
-    }
-    flag[1] = last;
-  }
-  __syncthreads();
-  if (!flag[1]) return;
-  const int c0 = a.child_begin[t], cc = a.child_count[t];
+  // The last of a top node and its chains forms the node's two terms of r.  With a general A
+  // (s_t = xi_t + A' sum_c s_c) they are no plain sums: there the last of a top node and all
+  // its children forms its s and r, and climbs on.
   const VT* sp = reinterpret_cast<const VT*>(a.spub);
   VT* rp = reinterpret_cast<VT*>(a.rpub);
-  VT* wt = reinterpret_cast<VT*>(a.wbuf) + (long long)t * n_k;
-  VT *S0 = Z, *R0 = Z + 2 * n_k;  // row 0: [S; 0], row 1: [0; psi], then R
-  for (int q = tid; q < n_x + n_k; q += kSweepThreads) {
-    if (q < n_x) {
-      S0[n_k + q] = 0;
-    } else {
-      const int e = q - n_x;
-      if (e < n_x) continue;
-      S0[e] = 0;
-      S0[n_k + e] = ldcg(wt + e);
+  VT *Z0 = Z, *Z1 = Z + n_k, *R0 = Z + 2 * n_k;
+  const bool climb = a.A != nullptr;
+  for (int t = d0.x; t >= 0; t = climb ? a.parent[t] : -1) {
+    __syncthreads();  // this CTA's outputs, then one fence, before its arrival
+    if (tid == 0) {
+      fence_acq_rel_gpu();
+      const int last = atomicAdd(&a.counters[t], 1) == (climb ? a.top_expect[t] - 1 : a.chain_kids[t]);
+      if (last) {
+        a.counters[t] = 0;
+        fence_acq_rel_gpu();
+      }
+      flag[1] = last;
     }
-  }
-  for (int q = tid; q < n_x + n_v; q += kSweepThreads) {
-    const bool tank = q < n_x;
-    const VT* in = tank ? sp : rp;
-    const int cols = tank ? n_x : n_v, e = tank ? q : q - n_x;
-    ST sum = st_from<ST>(0.0);
-    st_fma_acc(sum, (VT)1, tank ? ldcg(wt + e) : reinterpret_cast<const VT*>(a.beta)[(long long)t * n_v + e]);
-    constexpr int C = 8;
-    for (int i = 0; i < cc; i += C) {  // children in index order, C loads in flight
-      VT v[C];
-#pragma unroll
-      for (int k = 0; k < C; ++k)
-        v[k] = i + k < cc && a.top_expect[c0 + i + k] == 0 ? ldcg(in + (long long)(c0 + i + k) * cols + e) : (VT)0;
-#pragma unroll
-      for (int k = 0; k < C; ++k) st_fma_acc(sum, (VT)1, v[k]);
+    __syncthreads();
+    if (!flag[1]) return;
+    const int c0 = a.child_begin[t], cc = a.child_count[t];
+    VT* wt = reinterpret_cast<VT*>(a.wbuf) + (long long)t * n_k;
+    // row 0: [S; 0] and row 1: [0; psi]; with A row 0: [xi; psi] and row 1 the children's s.
+    // Row 2: beta and the children's r
+    for (int e = n_x + tid; e < n_k; e += kSweepThreads) {
+      Z1[e] = ldcg(wt + e);
+      Z0[e] = climb ? Z1[e] : (VT)0;
     }
-    (tank ? S0 : R0)[e] = st_val(sum);
+    for (int q = tid; q < n_x + n_v; q += kSweepThreads) {
+      const bool tank = q < n_x;
+      const VT* in = tank ? sp : rp;
+      const int cols = tank ? n_x : n_v, e = tank ? q : q - n_x;
+      const VT own_w = tank ? ldcg(wt + e) : reinterpret_cast<const VT*>(a.beta)[(long long)t * n_v + e];
+      ST sum = st_from<ST>(0.0);
+      if (!(climb && tank)) st_fma_acc(sum, (VT)1, own_w);
+      constexpr int C = 8;
+      for (int i = 0; i < cc; i += C) {  // children in index order, C loads in flight
+        VT v[C];
+#pragma unroll
+        for (int k = 0; k < C; ++k)
+          v[k] = i + k < cc && (climb || a.top_expect[c0 + i + k] == 0) ? ldcg(in + (long long)(c0 + i + k) * cols + e)
+                                                                        : (VT)0;
+#pragma unroll
+        for (int k = 0; k < C; ++k) st_fma_acc(sum, (VT)1, v[k]);
+      }
+      if (!tank) {
+        R0[e] = st_val(sum);
+      } else {
+        Z0[e] = climb ? own_w : st_val(sum);
+        Z1[e] = climb ? st_val(sum) : (VT)0;
+      }
+    }
+    __syncthreads();  // also: w has been read
+    if (climb) {
+      add_Ax<NW>(As, n_x, true, Z1, Z0);
+      __syncthreads();
+      if (tid < n_x) reinterpret_cast<VT*>(a.spub)[(long long)t * n_x + tid] = Z0[tid];
+    }
+    sparse_rows<NW, VT>(
+        et, cptr, cid, n_v, Z, n_k, 0, climb ? 1 : 2, [&](int r, int j) -> VT { return climb || r == 1 ? R0[j] : (VT)0; },
+        [&](int r, int j, VT v) { (climb || r == 1 ? rp + (long long)t * n_v : wt)[j] = v; });
   }
-  __syncthreads();  // also: w has been read
-  sparse_rows<NW, VT>(
-      et, cptr, cid, n_v, Z, n_k, 0, 2, [&](int r, int j) -> VT { return r == 1 ? R0[j] : (VT)0; },
-      [&](int r, int j, VT v) { (r == 1 ? rp + (long long)t * n_v : wt)[j] = v; });
 }
 
 // ---------------------------------------------------------------- delta = Lambda r
@@ -641,7 +686,9 @@ __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 
   __shared__ uint64_t bar[LW];
   __shared__ int2 list[kTopList];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int n_x = a.n_x, n_k = a.n_k, n_v = a.n_v, n_c = a.n - a.n_top;
+  const int n_x = a.n_x, n_k = a.n_k, n_v = a.n_v, n_c = a.A ? a.n : a.n - a.n_top;  // with A the tree pass has formed r of the top nodes
+  const int n_top = a.A ? 0 : a.n_top;
+  auto node = [&](int i) { return a.A ? i : a.chain_node[i]; };
   const int G = (n_v + BS - 1) / BS, steps = G / 2 + 1;
   const long long per = lam_entries(n_v);
   const VT* lam = reinterpret_cast<const VT*>(a.lam);
@@ -660,7 +707,7 @@ __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 
     mbar_init(&bar[warp], 1);
     fence_barrier_init();
     fence_proxy_async();
-    if (one ? warp == 0 : chains) fetch(one ? 0 : a.chain_node[q]);
+    if (one ? warp == 0 : chains) fetch(one ? 0 : node(q));
   }
   const bool mine = one ? warp == 0 : chains;  // a copy of this warp's is under way
   // the top warps: the first top node's sources into shared memory, its matrix towards the L2
@@ -669,7 +716,7 @@ __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 
   VT* lsum = reinterpret_cast<VT*>(part + kWarps * 32);  // the warps' parts of delta
   const int2* src = reinterpret_cast<const int2*>(a.top_src);
   int s0 = 0, s1 = 0, m_top = 0;
-  if (warp >= LW && (int)blockIdx.x < a.n_top) {
+  if (warp >= LW && (int)blockIdx.x < n_top) {
     m_top = a.top_nodes[blockIdx.x];
     s0 = a.top_src_off[blockIdx.x];
     s1 = a.top_src_off[blockIdx.x + 1];
@@ -689,19 +736,19 @@ __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 
     // ids are read two nodes ahead and r one node ahead of their use
     constexpr int RL = BS;  // 32 RL >= n_v
     const bool any = warp < cw && q < n_c;
-    int m = any ? a.chain_node[q] : 0, m1 = any && q + dq < n_c ? a.chain_node[q + dq] : -1;
+    int m = any ? node(q) : 0, m1 = any && q + dq < n_c ? node(q + dq) : -1;
     VT rn[RL], sc = 1;
-    auto read_r = [&](long long node) {
+    auto read_r = [&](long long at) {
 #pragma unroll
       for (int k = 0; k < RL; ++k) {
         const int j = lane + 32 * k;
-        rn[k] = j < n_v ? reinterpret_cast<const VT*>(a.rpub)[node * n_v + j] : (VT)0;
+        rn[k] = j < n_v ? reinterpret_cast<const VT*>(a.rpub)[at * n_v + j] : (VT)0;
       }
-      if (a.pscale) sc = reinterpret_cast<const VT*>(a.pscale)[node];
+      if (a.pscale) sc = reinterpret_cast<const VT*>(a.pscale)[at];
     };
     if (any) read_r(m);
     for (; q < n_c && warp < cw; q += dq) {
-      const int m2 = q + 2 * dq < n_c ? a.chain_node[q + 2 * dq] : -1;
+      const int m2 = q + 2 * dq < n_c ? node(q + 2 * dq) : -1;
       const VT scale = sc;
 #pragma unroll
       for (int k = 0; k < RL; ++k) rs[warp][lane + 32 * k] = rn[k];
@@ -742,7 +789,7 @@ __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 
   VT* rt = rs[LW];
   const VT* rp = reinterpret_cast<const VT*>(a.rpub);
   const VT* wb = reinterpret_cast<const VT*>(a.wbuf);
-  for (int t = blockIdx.x; t < a.n_top; t += gridDim.x) {
+  for (int t = blockIdx.x; t < n_top; t += gridDim.x) {
     const bool first = t == (int)blockIdx.x;
     if (!first) {
       m_top = a.top_nodes[t];
