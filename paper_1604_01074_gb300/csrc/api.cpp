@@ -303,6 +303,7 @@ void set_sweep_args(const smpc_factor_t* f, IterArgs& a) {
   const smpc_tree* t = f->tree;
   a.sp = t->top_src_off.empty() ? nullptr : f->sp;
   a.sp_nnz = f->sp_nnz;
+  a.kd = f->prec == SMPC_BF16 ? f->packs : nullptr;
   a.depth = t->N;
   a.max_len = t->max_chain_len;
   a.lam = f->lam;
@@ -310,6 +311,12 @@ void set_sweep_args(const smpc_factor_t* f, IterArgs& a) {
   a.top_src_off = t->dev.top_src_off;
   a.top_src = t->dev.top_src;
   a.chain_kids = t->dev.chain_kids;
+}
+void set_basis(const smpc_factor_t* f, CostArgs& c) {
+  const bool red = f->schedule == SCHED_SWEEP && f->prec == SMPC_BF16;  // beta enters in the anchors only
+  c.rhat_t = red ? f->rhat_t_red : f->rhat_t;
+  c.Rhat = red ? f->Rhat_red : f->Rhat;
+  c.L = red ? f->L_red : f->L;
 }
 }  // namespace smpc
 
@@ -696,6 +703,7 @@ int plan_iters(const smpc_factor_t* f, const IterArgs& a, const smpc_solve_opts&
     plan->args32 = plan->args;
     plan->args32.packs = f->packs32;
     plan->args32.pack_stride = f->pack_stride32;
+    plan->args32.lam = f->lam32;
     plan->cfg32 = iter_config(SMPC_FP32, plan->args32, f->num_sms, f->schedule);
     if (plan->cfg32.stages < 1) {
       set_error("network too large for the float32 pipeline");
@@ -771,6 +779,7 @@ int launch_planned(IterPlan& plan, int nu, int mode, void* stream) {
     } else {
       mode |= MODE_DELTA;
     }
+    if (nu >= 1 && (nu - 1 >= plan.polish_from || (nu - 1) % plan.anchor_every == 0)) mode |= MODE_AFTER_ANCHOR;
   }
   Profile* pf = plan.profile;
   const bool prof = pf && !anchor && (mode & MODE_BWD) && (mode & MODE_PROX) && nu >= 1 && pf->count < pf->capacity;
@@ -1026,18 +1035,44 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
     if ((rc = f->alloc(&f->ha, hb)) || (rc = f->alloc(&f->wa, hb))) return fail(rc);
     if (cudaMemset(f->ha, 0, hb) != cudaSuccess || cudaMemset(f->wa, 0, hb) != cudaSuccess) return fail(SMPC_ECUDA);
   }
-  // ---- the two-launch form of schedule 4 (with a general A: of schedule 2): only a factor that may choose its schedule
-  const size_t lam_bytes = (size_t)np * lam_pack_entries(n_v) * f->vs;
-  if (o.schedule == 0 && f->prec != SMPC_BF16 && !tree->top_src_off.empty()) {
-    for (double v : K) f->sp_nnz += v != 0.0;
+  // ---- the two-launch form of schedule 4 (with a general A: of schedule 2): only a factor
+  // that may choose its schedule.  A bfloat16 factor's anchors run it in float32 in the reduced
+  // basis, its delta launches on the packs' own [Bbar; L] and Lambda; with one pack for all
+  // nodes those round vectors to bfloat16 for the tensor cores, in an order that the two-launch
+  // form does not keep.
+  const size_t lam_bytes = (size_t)np * lam_pack_entries(n_v) * f->ms, lam32_bytes = (size_t)np * lam_pack_entries(n_v) * 4;
+  const bool b16 = f->prec == SMPC_BF16;
+  if (o.schedule == 0 && !tree->top_src_off.empty() && !(b16 && (f->shared_packs || general_A))) {
+    HostFactor red;
+    const HostFactor* hs = &f->hf;
+    if (b16) {
+      if ((rc = host_factor(*net, cost->W_u, red, true)) != SMPC_OK) return fail(rc);
+      hs = &red;
+    }
+    std::vector<double> Ks((size_t)n_k * n_v);
+    std::copy(hs->Bbar.begin(), hs->Bbar.end(), Ks.begin());
+    std::copy(hs->L.begin(), hs->L.end(), Ks.begin() + (size_t)n_x * n_v);
+    for (double v : Ks) f->sp_nnz += v != 0.0;
     if (f->sp_nnz <= kSparseMax) {
-      const std::vector<unsigned char> image = sparse_image(f->prec, n_k, n_v, K.data());
+      const std::vector<unsigned char> image = sparse_image(f->prec, n_k, n_v, Ks.data());
       if ((rc = f->alloc(&f->sp, image.size()))) return fail(rc);
       if (cudaMemcpy(f->sp, image.data(), image.size(), cudaMemcpyHostToDevice) != cudaSuccess) return fail(SMPC_ECUDA);
-      // without room for it the other schedules run as before
-      if (f->alloc(&f->lam, lam_bytes) == SMPC_OK &&
-          (rc = launch_lam_pack(f->prec, np, n_v, f->Lam64, pprob, f->lam, nullptr)))
-        return fail(rc);
+      // without room for the matrices the other schedules run as before
+      if (f->alloc(&f->lam, lam_bytes) == SMPC_OK) {
+        if ((rc = launch_lam_pack(f->prec, np, n_v, f->Lam64, pprob, f->lam, nullptr))) return fail(rc);
+        if (b16 && f->alloc(&f->lam32, lam32_bytes) == SMPC_OK) {
+          double* Lam = nullptr;
+          if ((rc = up64(&Lam, red.Lam.data(), red.Lam.size())) || (rc = up64(&f->Rhat_red, red.Rhat.data(), red.Rhat.size())) ||
+              (rc = up64(&f->L_red, red.L.data(), red.L.size())) ||
+              (rc = up_csr(&f->rhat_t_red, n_v, n_u, [&](int i, int j) { return red.Rhat[(size_t)j * n_v + i]; })) ||
+              (rc = launch_lam_pack(SMPC_FP32, np, n_v, Lam, pprob, f->lam32, nullptr)))
+            return fail(rc);
+        }
+        if (b16 && !f->lam32) {
+          f->release(f->lam, lam_bytes);
+          f->lam = nullptr;
+        }
+      }
     }
   }
   // ---- vectors
@@ -1192,7 +1227,8 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   if ((rc = tune_tc(f, o.tc_width))) return fail(rc);
   if (f->lam && f->schedule != SCHED_SWEEP) {  // not chosen: its matrices go
     f->release(f->lam, lam_bytes);
-    f->lam = nullptr;
+    f->release(f->lam32, lam32_bytes);
+    f->lam = f->lam32 = nullptr;
   }
   *out = f;
   return SMPC_OK;
@@ -1307,9 +1343,7 @@ int solve_begin(smpc_factor_t* f, const smpc_step_data* data, const smpc_solve_o
   c.prob = f->tree->dev.prob;
   c.pbar = f->tree->dev.pbar;
   c.pue = f->pue;
-  c.rhat_t = f->rhat_t;
-  c.Rhat = f->Rhat;
-  c.L = f->L;
+  set_basis(f, c);
   c.alpha1 = f->alpha1;
   c.W_alpha = f->W_alpha;
   c.dhat = f->d_dhat;

@@ -3241,11 +3241,13 @@ LaunchCfg config_t(const IterArgs& a, int num_sms, int S_max, int schedule, int 
   const bool fits_threads = a.n_k <= kThreads && a.n_v <= kThreads;  // one thread per entry
   if (schedule == SCHED_SWEEP) {  // sparse [Bbar; L] and packed Lambda of the vector type
     c.stages = 0;
-    if constexpr (std::is_same<VT, MT>::value) {
-      c.smem = sweep_smem_bytes<VT>(a.sp_nnz, a.depth, a.n_x, a.n_u, a.n_v, a.A != nullptr);
+    // float64, float32 and bfloat16 factors (kd: the bfloat16 [Bbar; L], also for their float32 anchors)
+    const bool b16 = a.kd != nullptr;
+    if (std::is_same<VT, MT>::value || b16) {
+      c.smem = sweep_smem_bytes<VT>(a.sp_nnz, a.depth, a.n_x, a.n_u, a.n_v, a.A != nullptr, b16);
       c.grid = a.n_chains + a.n_top;
       const int tasks = a.max_len * (1 + (a.n_u + 63) / 64);  // of a chain's prox, one warp each
-      c.sweep_warps = a.n_x > 64 ? 16
+      c.sweep_warps = a.n_x > 64 || b16 ? 16
                       : a.n_chains > 2 * num_sms || tasks <= 8 ? 8
                       : a.n_chains <= num_sms && tasks >= 48 && sizeof(VT) == 4 ? 32 : 16;
       // Lambda: matrix slots for four chain warps where two CTAs fit an SM, else as many as fit
@@ -3255,9 +3257,9 @@ LaunchCfg config_t(const IterArgs& a, int num_sms, int S_max, int schedule, int 
       // float64: the pipe, not the copies, sets the time, and eight warps reading in place keep
       // it busier than the four that slots of 42 KB leave
       c.lam_slots = a.lam_stride == 0 ? 1 : sizeof(VT) == 8 ? 0 : 4;
-      while (c.lam_slots > 1 && lambda_smem_bytes<VT>(a.n_v, c.lam_slots) > room) --c.lam_slots;
-      if (lambda_smem_bytes<VT>(a.n_v, c.lam_slots) > room) c.lam_slots = 0;
-      c.smem_lam = lambda_smem_bytes<VT>(a.n_v, c.lam_slots);
+      while (c.lam_slots > 1 && lambda_smem_bytes<VT, MT>(a.n_v, c.lam_slots) > room) --c.lam_slots;
+      if (lambda_smem_bytes<VT, MT>(a.n_v, c.lam_slots) > room) c.lam_slots = 0;
+      c.smem_lam = lambda_smem_bytes<VT, MT>(a.n_v, c.lam_slots);
       c.lam_warps = a.lam_stride == 0 || sizeof(VT) == 8 ? 8 : 4;  // chain warps a CTA
       const int cw = c.lam_slots == 0 || a.lam_stride == 0 ? c.lam_warps : c.lam_slots;
       c.grid_lam = std::min(std::max((n_c + cw - 1) / cw, a.A ? 1 : a.n_top), ctas * num_sms);
@@ -3365,10 +3367,16 @@ void launch_dep(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaSt
 template <typename VT>
 auto sweep_kernel(const IterArgs& a, int warps) {
   if constexpr (sizeof(VT) == 4) {
-    if (warps == 32) return a.n_x <= 32 ? tree_sweep<VT, 1, 32> : tree_sweep<VT, 2, 32>;
+    if (a.kd)
+      return a.n_x <= 32   ? tree_sweep<VT, 1, 16, true>
+             : a.n_x <= 64 ? tree_sweep<VT, 2, 16, true>
+                           : tree_sweep<VT, 8, 16, true>;
+    if (warps == 32) return a.n_x <= 32 ? tree_sweep<VT, 1, 32, false> : tree_sweep<VT, 2, 32, false>;
   }
-  if (warps == 8) return a.n_x <= 32 ? tree_sweep<VT, 1, 8> : tree_sweep<VT, 2, 8>;
-  return a.n_x <= 32 ? tree_sweep<VT, 1, 16> : a.n_x <= 64 ? tree_sweep<VT, 2, 16> : tree_sweep<VT, 8, 16>;
+  if (warps == 8) return a.n_x <= 32 ? tree_sweep<VT, 1, 8, false> : tree_sweep<VT, 2, 8, false>;
+  return a.n_x <= 32   ? tree_sweep<VT, 1, 16, false>
+         : a.n_x <= 64 ? tree_sweep<VT, 2, 16, false>
+                       : tree_sweep<VT, 8, 16, false>;
 }
 
 template <typename VT, typename MT>
@@ -3393,19 +3401,21 @@ int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream
     if constexpr (std::is_same<MT, __nv_bfloat16>::value) {
       allow(node_mv_tc<VT>);
       allow(node_gt_tc<VT>);
-    } else {
-      IterArgs t{};
-      for (int n_x : {32, 64, 65})
-        for (int warps : {8, 16, 32}) {
-          t.n_x = n_x;
-          if (n_x <= 64 || warps == 16) allow(sweep_kernel<VT>(t, warps));
-        }
-      if constexpr (sizeof(VT) == 4) {
-        allow(lambda_apply<VT, 4, 4>);
-        allow(lambda_apply<VT, 8, 4>);
+    }
+    IterArgs t{};
+    for (int n_x : {32, 64, 65})
+      for (int warps : {8, 16, 32}) {
+        t.n_x = n_x;
+        t.kd = nullptr;
+        if (n_x <= 64 || warps == 16) allow(sweep_kernel<VT>(t, warps));
+        t.kd = &t;  // any address: the bfloat16 factors' kernels
+        if (sizeof(VT) == 4) allow(sweep_kernel<VT>(t, warps));
       }
-      allow(lambda_apply<VT, 4, 8>);
-      allow(lambda_apply<VT, 8, 8>);
+    allow(lambda_apply<VT, MT, 4, 8>);
+    allow(lambda_apply<VT, MT, 8, 8>);
+    if constexpr (sizeof(VT) == 4) {
+      allow(lambda_apply<VT, MT, 4, 4>);
+      allow(lambda_apply<VT, MT, 8, 4>);
     }
     cudaGetLastError();  // a refused attribute surfaces at the launch, not here
     return true;
@@ -3422,22 +3432,20 @@ int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream
     mark();
     return check_launch("apg_iter");
   }
-  if constexpr (std::is_same<VT, MT>::value) {
-    if (c.schedule == SCHED_SWEEP) {
-      // nu = 0 waits for everything before it, so that later launches may read the solve's
-      // affine data before their programmatic wait
-      launch_dep(sweep_kernel<VT>(a, c.sweep_warps), c.grid, 32 * c.sweep_warps, c.smem, s, dep && nu > 0, a, nu, mode);
+  if (c.schedule == SCHED_SWEEP) {
+    // nu = 0 waits for everything before it, so that later launches may read the solve's
+    // affine data before their programmatic wait
+    launch_dep(sweep_kernel<VT>(a, c.sweep_warps), c.grid, 32 * c.sweep_warps, c.smem, s, dep && nu > 0, a, nu, mode);
+    mark();
+    if (mode & MODE_BWD) {
+      const bool wide = lam_bs(a.n_v) == 8;
+      auto kern = wide ? lambda_apply<VT, MT, 8, 8> : lambda_apply<VT, MT, 4, 8>;
+      if constexpr (sizeof(VT) == 4)
+        if (c.lam_warps == 4) kern = wide ? lambda_apply<VT, MT, 8, 4> : lambda_apply<VT, MT, 4, 4>;
+      launch_dep(kern, c.grid_lam, (c.lam_warps + kWarps) * 32, c.smem_lam, s, dep, a, c.lam_slots, nu, mode);
       mark();
-      if (mode & MODE_BWD) {
-        const bool wide = lam_bs(a.n_v) == 8;
-        auto kern = wide ? lambda_apply<VT, 8, 8> : lambda_apply<VT, 4, 8>;
-        if constexpr (sizeof(VT) == 4)
-          if (c.lam_warps == 4) kern = wide ? lambda_apply<VT, 8, 4> : lambda_apply<VT, 4, 4>;
-        launch_dep(kern, c.grid_lam, (c.lam_warps + kWarps) * 32, c.smem_lam, s, dep, a, c.lam_slots, nu, mode);
-        mark();
-      }
-      return check_launch("tree sweep");
     }
+    return check_launch("tree sweep");
   }
   if ((mode & MODE_PROX) && nu >= 1) {
     launch_dep(fwd_scan<VT, MT>, c.grid_fwd, c.block, c.smem_fwd, s, dep, a, nu, mode);
@@ -3563,6 +3571,8 @@ int launch_lam_pack(int prec, int n, int n_v, const double* Lam, const double* p
   const int grid = n < 4096 ? n : 4096;
   if (prec == SMPC_FP64)
     lam_pack_kernel<double><<<grid, 256, 0, s>>>(n, n_v, Lam, prob, (double*)out);
+  else if (prec == SMPC_BF16)
+    lam_pack_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(n, n_v, Lam, prob, (__nv_bfloat16*)out);
   else
     lam_pack_kernel<float><<<grid, 256, 0, s>>>(n, n_v, Lam, prob, (float*)out);
   return check_launch("lam_pack_kernel");

@@ -157,6 +157,7 @@ struct IterArgs {
   // as symmetric blocks (or one unscaled Lambda, lam_stride 0, with pscale), the largest tree
   // depth and chain length, and per top node its sources {node, weight}: the top nodes below and itself.
   const void* sp;
+  const void* kd;                // bfloat16 factors: the packs' [Bbar; L] (one node's), else NULL
   int sp_nnz, depth, max_len;
   const void* lam;
   long long lam_stride;
@@ -175,6 +176,7 @@ enum KernelMode : int {
   MODE_GT = 64,       // backward sweep up to r only: s, g = [Bbar; L]'[s; psi], r for every node
   MODE_WREADY = 128,  // w^nu was written by an earlier launch of the iteration
   MODE_NOCLIMB = 256,  // chain pass of a shard: chains publish their heads' s and r, no top-node climb
+  MODE_AFTER_ANCHOR = 1024,  // anchored solve: the launch before this one was an anchor
   MODE_WONLY = 512     // prox launch writes w^nu of an iteration without a prox (as with MODE_BWD) while
                        // the backward sweep is launched separately
 };
@@ -328,6 +330,8 @@ int plan_iters(const smpc_factor_t* f, const IterArgs& a, const smpc_solve_opts&
 int launch_planned(IterPlan& plan, int nu, int mode, void* stream);
 // The SCHED_SWEEP fields of a.
 void set_sweep_args(const smpc_factor_t* f, IterArgs& a);
+// The basis of beta: c.L, c.Rhat, c.rhat_t.
+void set_basis(const smpc_factor_t* f, CostArgs& c);
 // Copies the final dual of the factor's last solve (vector type) to dst; synchronous.
 int copy_final_y(smpc_factor_t* f, void* dst);
 }  // namespace smpc
@@ -381,6 +385,11 @@ struct smpc_factor_t {
   int num_sms = 0;
   int schedule = smpc::SCHED_CHAIN;  // iteration schedule in use
   void *sp = nullptr, *lam = nullptr;  // SCHED_SWEEP: sparse [Bbar; L], packed Lambda
+  // ... of a bfloat16 factor: the anchors' float32 Lambda and cost-update matrices, in the
+  // reduced basis (lam: bfloat16, in the basis of the packs)
+  void* lam32 = nullptr;
+  double *Rhat_red = nullptr, *L_red = nullptr;
+  smpc::CsrRows rhat_t_red;
   int sp_nnz = 0;
   float tuned_ms[6] = {0, 0, 0, 0, 0, 0};  // per schedule: ms per iteration measured when the factor chose
   int tc_width = 0;                   // bfloat16 shared packs: nodes per tensor-core GEMM (0: none)

@@ -83,12 +83,38 @@ __device__ __forceinline__ void st_state(double* p, double v) { *p = v; }
 __device__ __forceinline__ void st_fma_acc(DS& acc, float w, float v) { acc = st_axpy(acc, w, v); }
 __device__ __forceinline__ void st_fma_acc(double& acc, double w, double v) { acc = fma(w, v, acc); }
 
+// sums in the vector type or in the state type
+template <typename ST, typename VT>
+__device__ __forceinline__ ST to_sum(VT v) {
+  if constexpr (std::is_same<ST, DS>::value)
+    return DS{v, 0.f};
+  else
+    return v;
+}
+__device__ __forceinline__ void add_sum(DS& s, float v) {
+  const DS t = two_sum(s.hi, v);
+  s = fast_two_sum(t.hi, __fadd_rn(t.lo, s.lo));
+}
+__device__ __forceinline__ void add_sum(float& s, float v) { s += v; }
+__device__ __forceinline__ void add_sum(double& s, double v) { s += v; }
+__device__ __forceinline__ float sum_val(DS s) { return st_val(s); }
+__device__ __forceinline__ float sum_val(float s) { return s; }
+__device__ __forceinline__ double sum_val(double s) { return s; }
+
+// Rows of the tree pass's vectors; in bfloat16 factors multiples of four entries, zero-padded,
+// for the dense products below, whose [Bbar; L] has dense_kw words (two entries) a row: an odd
+// number, so that 32 rows' words lie in 32 banks.
+__host__ __device__ inline int sweep_pad(int n, bool b16) { return b16 ? (n + 3) / 4 * 4 : n; }
+__host__ __device__ inline int dense_kw(int n_v) { return sweep_pad(n_v, true) / 2 | 1; }
 template <typename VT>
-__host__ __device__ inline size_t sweep_smem_bytes(int nnz, int depth, int n_x, int n_u, int n_v, bool general_A) {
-  const int n_k = n_x + n_u;
+__host__ __device__ inline size_t sweep_smem_bytes(int nnz, int depth, int n_x, int n_u, int n_v, bool general_A,
+                                                   bool b16) {
+  const int n_k = n_x + n_u, xk = sweep_pad(n_k, b16), xv = sweep_pad(n_v, b16);
   size_t b = sp_bytes<VT>(nnz, n_k, n_v);
-  b += (size_t)(3 * n_x + 2 * n_u + (depth + 3) * (n_v + n_k)) * sizeof(VT);  // depth + 3 >= 4 rows: the last arrival's too
+  b += round_up((size_t)(3 * n_x + 2 * n_u) * sizeof(VT), 16);
+  b += (size_t)(depth + 3) * (xv + xk) * sizeof(VT);  // depth + 3 >= 4 rows: the last arrival's too
   if (general_A) b += (size_t)n_x * n_x * sizeof(VT);
+  if (b16) b += (size_t)xk * dense_kw(n_v) * sizeof(uint32_t);
   return round_up(b + (size_t)depth * sizeof(int), 16);
 }
 
@@ -147,8 +173,11 @@ template <typename VT>
 struct SweepOut {
   MaxAbs<VT> r, h, t;  // residual maxima: |x - t|, |x|, |t| of the prox
 };
-template <typename VT, int NT>
-__device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, const VT* bnd, int it, VT c, VT cn,
+// Anchored solves (bfloat16 packs, B16): a delta launch takes w - w_a, exactly in the state
+// type; an anchor stores w_a = w; the launch after an anchor stores x and u, from which those
+// up to the next anchor continue with the linear part.
+template <typename VT, int NT, bool B16>
+__device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, const VT* bnd, int it, VT c, VT cn, int mode,
                                             SweepOut<VT>& o) {
   using ST = typename St<VT>::T;
   const int lane = threadIdx.x & 31, n_x = a.n_x, nd = 2 * n_x + a.n_u;
@@ -168,6 +197,13 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
       wz[k] = ld_state(y2 + n_x + e);
     }
   }
+  VT wa[NT];
+  if (B16)
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+      const int e = lane + 32 * k;
+      wa[k] = (mode & MODE_DELTA) && e < n_x ? reinterpret_cast<const VT*>(a.wa)[(long long)m * a.n_k + e] : (VT)0;
+    }
   const VT ls = reinterpret_cast<const VT*>(a.step_s)[m], lz = reinterpret_cast<const VT*>(a.step_z)[m];
   const VT is = reinterpret_cast<const VT*>(a.inv_s)[m], iz = reinterpret_cast<const VT*>(a.inv_z)[m];
   const VT mus = reinterpret_cast<const VT*>(a.mu_s)[m], muz = (VT)a.gamma_d;
@@ -216,7 +252,13 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
       st_state(y2 + e, ysn);
       st_state(y2 + n_x + e, yzn);
       xo[e] = x;
-      z[e] = st_extrap_val(ysn, v1[k], cn) + st_extrap_val(yzn, w1[k], cn);
+      if (B16 && (mode & MODE_DELTA)) {
+        z[e] = st_val(st_sub(st_add(st_extrap(ysn, v1[k], cn), st_extrap(yzn, w1[k], cn)), st_from<ST>((double)wa[k])));
+      } else {
+        z[e] = st_extrap_val(ysn, v1[k], cn) + st_extrap_val(yzn, w1[k], cn);
+        if (B16 && (mode & MODE_ANCHOR)) reinterpret_cast<VT*>(a.wa)[(long long)m * a.n_k + e] = z[e];
+      }
+      if (B16 && (mode & MODE_AFTER_ANCHOR)) reinterpret_cast<VT*>(a.ha)[(long long)m * a.n_k + e] = x;
       if (a.xbar) {  // ergodic average (theta_0 = 1: the previous contents are not read then)
         VT* b = reinterpret_cast<VT*>(a.xbar) + (long long)m * n_x + e;
         const VT th = (VT)a.theta[it];
@@ -230,9 +272,9 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
     }
   }
 }
-template <typename VT>
+template <typename VT, bool B16>
 __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, VT* z, const VT* bnd, int it, VT c, VT cn,
-                                             SweepOut<VT>& o) {
+                                             int mode, SweepOut<VT>& o) {
   using ST = typename St<VT>::T;
   constexpr int NU = 2;
   const int lane = threadIdx.x & 31, n_x = a.n_x, n_u = a.n_u, nd = 2 * n_x + n_u;
@@ -242,7 +284,8 @@ __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, V
   const long long mu = (long long)m * n_u;
   const ST zero = st_from<ST>(0.0);
   ST p1[NU], p2[NU];
-  VT lp[NU], ip[NU];
+  VT lp[NU], ip[NU], wa[NU];
+  const long long mk = (long long)m * a.n_k + n_x;
 #pragma unroll
   for (int k = 0; k < NU; ++k) {
     const int i = i0 + lane + 32 * k;
@@ -253,6 +296,7 @@ __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, V
       p2[k] = ld_state(y2 + i);
       lp[k] = reinterpret_cast<const VT*>(a.step_p)[mu + i];
       ip[k] = reinterpret_cast<const VT*>(a.inv_p)[mu + i];
+      if (B16) wa[k] = (mode & MODE_DELTA) ? reinterpret_cast<const VT*>(a.wa)[mk + i] : (VT)0;
     }
   }
 #pragma unroll
@@ -265,7 +309,13 @@ __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, V
       const VT ep = sw_diff(ypn, wp) * ip[k];
       st_state(y2 + i, ypn);
       reinterpret_cast<VT*>(a.uout)[mu + i] = u;
-      z[n_x + i] = st_extrap_val(ypn, p1[k], cn);
+      if (B16 && (mode & MODE_DELTA)) {
+        z[n_x + i] = st_val(st_sub(st_extrap(ypn, p1[k], cn), st_from<ST>((double)wa[k])));
+      } else {
+        z[n_x + i] = st_extrap_val(ypn, p1[k], cn);
+        if (B16 && (mode & MODE_ANCHOR)) reinterpret_cast<VT*>(a.wa)[mk + i] = z[n_x + i];
+      }
+      if (B16 && (mode & MODE_AFTER_ANCHOR)) reinterpret_cast<VT*>(a.ha)[mk + i] = u;
       if (a.ubar) {
         VT* b = reinterpret_cast<VT*>(a.ubar) + mu + i;
         const VT th = (VT)a.theta[it];
@@ -279,10 +329,13 @@ __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, V
 }
 
 // In-place running sums of column `col` over rows r0, r0 + dr, ... (n of them); put(r, v) sees
-// each sum.  Eight rows are read ahead of their sums.
-template <typename VT, typename F>
-__device__ __forceinline__ void run_sums(VT* X, int xs, int col, int r0, int dr, int n, VT v, F&& put) {
+// each sum.  Eight rows are read ahead of their sums.  The backward sums (s and r, ST the state
+// type) run in two float32: their terms nearly cancel, and with them the error of x is a third
+// of that with plain sums (1.0e-6 against 2.8e-6 after 60 iterations of 21 111 nodes).
+template <typename ST, typename VT, typename F>
+__device__ __forceinline__ void run_sums(VT* X, int xs, int col, int r0, int dr, int n, VT first, F&& put) {
   constexpr int B = 8;
+  ST v = to_sum<ST>(first);
   for (int q0 = 0; q0 < n; q0 += B) {
     VT t[B];
 #pragma unroll
@@ -290,9 +343,101 @@ __device__ __forceinline__ void run_sums(VT* X, int xs, int col, int r0, int dr,
 #pragma unroll
     for (int b = 0; b < B; ++b)
       if (q0 + b < n) {
-        v += t[b];
-        put(r0 + (q0 + b) * dr, v);
+        add_sum(v, t[b]);
+        put(r0 + (q0 + b) * dr, (VT)sum_val(v));
       }
+  }
+}
+
+// Entries in pairs: two float32 in one register pair and one fused multiply-add instruction
+// (f32x2), or one float64.
+__device__ __forceinline__ unsigned long long f2(float x, float y) {
+  return (unsigned long long)__float_as_uint(x) | ((unsigned long long)__float_as_uint(y) << 32);
+}
+struct PairF {
+  using T = unsigned long long;
+  static constexpr int N = 2;
+  __device__ static T fma(T a, T b, T c) {
+    T d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+  }
+  __device__ static T dup(float x) { return f2(x, x); }
+  __device__ static T zero() { return 0; }
+  __device__ static float sum(T a) { return __uint_as_float((unsigned)a) + __uint_as_float((unsigned)(a >> 32)); }
+  __device__ static float at(T a, int k) { return __uint_as_float((unsigned)(k ? a >> 32 : a)); }
+  __device__ static void ld(const float* p, T (&o)[2]) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+    o[0] = t.x;
+    o[1] = t.y;
+  }
+};
+
+// Two bfloat16 entries as a float32 pair
+__device__ __forceinline__ unsigned long long bf2(uint32_t u) {
+  return (unsigned long long)(u << 16) | ((unsigned long long)(u & 0xffff0000u) << 32);
+}
+// The dense [Bbar; L] of a bfloat16 factor (K: kw words a row) applied to float32 rows, four
+// rows at a time.  Forward: put(r, e, (K V_r)_e), a lane per row e of K; the four rows' entries
+// are broadcast reads, and pairs of products go through f32x2.  Backward: put(r, j, (K' Z_r)_j),
+// two columns a lane.  They double the pass's instructions (about 550 and 800 a node at 177 x
+// 97 entries); streaming each node's own copy of K through the chains instead took 460 us of a
+// 21 111-node iteration.
+template <int NW, typename F>
+__device__ __forceinline__ void dense_fwd(const uint32_t* K, int kw, int n_k, const float* V, int xv, int r0, int r1,
+                                          F&& put) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ec = (n_k + 31) / 32, ng = (r1 - r0 + 3) / 4;
+  for (int task = warp; task < ec * ng; task += NW) {
+    const int g = task / ec, e = (task - g * ec) * 32 + lane, rb = r0 + 4 * g;
+    const uint32_t* row = K + min(e, n_k - 1) * kw;
+    unsigned long long acc[4] = {0, 0, 0, 0};
+#pragma unroll 2
+    for (int j = 0; j < xv; j += 4) {
+      const unsigned long long k0 = bf2(row[j / 2]), k1 = bf2(row[j / 2 + 1]);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(V + (rb + b) * xv + j);
+        acc[b] = PairF::fma(k0, v.x, acc[b]);
+        acc[b] = PairF::fma(k1, v.y, acc[b]);
+      }
+    }
+    if (e < n_k)
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (rb + b < r1) put(rb + b, e, PairF::sum(acc[b]));
+  }
+}
+template <int NW, typename F>
+__device__ __forceinline__ void dense_bwd(const uint32_t* K, int kw, int n_v, const float* Z, int xk, int r0, int r1,
+                                          F&& put) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int jc = (n_v + 63) / 64, ng = (r1 - r0 + 3) / 4;
+  for (int task = warp; task < jc * ng; task += NW) {
+    const int g = task / jc, w = (task - g * jc) * 32 + lane, rb = r0 + 4 * g;
+    const uint32_t* col = K + min(w, kw - 1);
+    float acc[4][2] = {};
+#pragma unroll 2
+    for (int e = 0; e < xk; e += 4) {
+      uint32_t u[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) u[i] = col[(e + i) * kw];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const float4 y = *reinterpret_cast<const float4*>(Z + (rb + b) * xk + e);
+        const float yv[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          acc[b][0] += __uint_as_float(u[i] << 16) * yv[i];
+          acc[b][1] += __uint_as_float(u[i] & 0xffff0000u) * yv[i];
+        }
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (rb + b < r1 && 2 * w + h < n_v) put(rb + b, 2 * w + h, acc[b][h]);
   }
 }
 
@@ -315,7 +460,7 @@ __device__ __forceinline__ void add_Ax(const VT* A, int n, bool trans, const VT*
 // memory or shared memory with few warps busy, so trees with several chains an SM run four
 // small CTAs there, side by side in different phases; trees with at most a chain an SM have
 // nothing to overlap and spread each chain over as many warps as an SM takes.
-template <typename VT, int NT, int NW>
+template <typename VT, int NT, int NW, bool B16>
 __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 : 16) / NW)
     tree_sweep(const __grid_constant__ IterArgs a, int nu, int mode) {
   using ST = typename St<VT>::T;
@@ -327,6 +472,10 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_x = a.n_x, n_u = a.n_u, n_k = a.n_k, n_v = a.n_v, nnz = a.sp_nnz;
   const bool prox = (mode & MODE_PROX) != 0 && nu >= 1;
+  // bfloat16 factors: the forward part continues a delta launch, the backward part is one
+  // (both in the orthonormal basis of the packs); else they are the anchors' float32 ones
+  const bool fd = B16 && !(mode & MODE_AFTER_ANCHOR), bd = B16 && (mode & MODE_DELTA) != 0;
+  const int xv = sweep_pad(n_v, B16), xk = sweep_pad(n_k, B16);
   // ---- read while the previous launch drains: constants of the factor and the tree, and the
   // solve's affine data, complete before its first launch (nu = 0), which starts without
   // programmatic overlap
@@ -336,10 +485,25 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
   const int* rptr = reinterpret_cast<const int*>(et + nnz);
   const int *rid = rptr + n_k + 1, *cptr = rid + n_k, *cid = cptr + n_v + 1;
   VT* bnd = reinterpret_cast<VT*>(smem_raw + blob);
-  VT* V = bnd + 3 * n_x + 2 * n_u;  // delta, then v, then beta, g and r: a row of n_v per node
-  VT* Z = V + (a.depth + 3) * n_v;  // e and u_hat, then x and u, then w and s: a row of n_k per node
-  VT* As = Z + (a.depth + 3) * n_k;  // a general state matrix
-  int* sid = reinterpret_cast<int*>(As + (a.A ? n_x * n_x : 0));
+  VT* V = reinterpret_cast<VT*>(smem_raw + blob + round_up((3 * n_x + 2 * n_u) * (int)sizeof(VT), 16));  // delta, then v, then beta, g and r: a row of n_v per node
+  VT* Z = V + (a.depth + 3) * xv;  // e and u_hat, then x and u, then w and s: a row of n_k per node
+  VT* As = Z + (a.depth + 3) * xk;  // a general state matrix
+  uint32_t* Kd = reinterpret_cast<uint32_t*>(As + (a.A ? n_x * n_x : 0));  // B16: the dense [Bbar; L]
+  const int kw = dense_kw(n_v);
+  int* sid = reinterpret_cast<int*>(Kd + (B16 ? xk * kw : 0));
+  if (B16) {
+    const int ld = row_stride<__nv_bfloat16>(n_v);  // even
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(a.kd);
+    if ((fd && prox) || bd)
+      for (int q = tid; q < xk * kw; q += kSweepThreads) {
+        const int e = q / kw, w = q - e * kw;
+        Kd[q] = e < n_k && 2 * w < ld ? src[e * (ld / 2) + w] : 0u;  // the pack's padding is zero
+      }
+    for (int r = tid; r < a.depth + 3; r += kSweepThreads) {  // padding columns
+      for (int j = n_v; j < xv; ++j) V[r * xv + j] = 0;
+      for (int e = n_k; e < xk; ++e) Z[r * xk + e] = 0;
+    }
+  }
   if (a.A)
     for (int q = tid; q < n_x * n_x; q += kSweepThreads) As[q] = reinterpret_cast<const VT*>(a.A)[q];
   // chains first (the long tasks), then the top nodes
@@ -359,21 +523,25 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
   }
   const VT c = (VT)a.cvec[prox ? nu - 1 : nu], cn = prox ? (VT)a.cvec[nu] : (VT)0;
   __syncthreads();
-  if (prox) {
+  if (prox && !fd) {
     const VT* E = reinterpret_cast<const VT*>(a.e);
     const VT* UH = reinterpret_cast<const VT*>(a.uhat);
     for (int r = warp; r < L; r += NW) {
       const long long m = sid[r];
-      for (int e = lane; e < n_x; e += 32) cp_async_elem(Z + r * n_k + e, E + m * n_x + e);
+      for (int e = lane; e < n_x; e += 32) cp_async_elem(Z + r * xk + e, E + m * n_x + e);
       if (r >= own)
-        for (int i = lane; i < n_u; i += 32) cp_async_elem(Z + r * n_k + n_x + i, UH + m * n_u + i);
+        for (int i = lane; i < n_u; i += 32) cp_async_elem(Z + r * xk + n_x + i, UH + m * n_u + i);
     }
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (prox) {
     const VT* delta = reinterpret_cast<const VT*>(a.h);
     for (int r = warp; r < L; r += NW)
-      for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * n_v + j, delta + (long long)sid[r] * n_v + j);
+      for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * xv + j, delta + (long long)sid[r] * n_v + j);
+    if (fd)  // the anchor's u (its x is added after the linear path sums)
+      for (int r = own + warp; r < L; r += NW)
+        for (int e = n_x + lane; e < n_k; e += 32)
+          cp_async_elem(Z + r * xk + e, reinterpret_cast<const VT*>(a.ha) + (long long)sid[r] * n_k + e);
   }
   const bool stop = early_exit(a, nu, mode, flag, true) || !tree_active(a, tree, nu);
   cp_async_wait_all();
@@ -383,38 +551,53 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
   if (prox) {
     __syncthreads();
     if (tid < n_v)  // v along the path
-      run_sums(V, n_v, tid, 0, 1, L, (VT)0, [&](int r, VT v) { V[r * n_v + tid] = v; });
+      run_sums<VT>(V, xv, tid, 0, 1, L, (VT)0, [&](int r, VT v) { V[r * xv + tid] = v; });
     __syncthreads();
     // x increments (Bbar v + e) and u; of path nodes only the tanks are used
-    sparse_rows<NW, VT>(
-        ek, rptr, rid, n_k, V, n_v, 0, L, [&](int r, int e) -> VT { return Z[r * n_k + e]; },
-        [&](int r, int e, VT v) { Z[r * n_k + e] = v; });
+    if constexpr (B16) {
+      if (fd)
+        dense_fwd<NW>(Kd, kw, n_k, V, xv, 0, L, [&](int r, int e, VT v) {
+          if (e < n_x)
+            Z[r * xk + e] = v;
+          else if (r >= own)
+            Z[r * xk + e] += v;
+        });
+    }
+    if (!fd) sparse_rows<NW, VT>(
+        ek, rptr, rid, n_k, V, xv, 0, L, [&](int r, int e) -> VT { return Z[r * xk + e]; },
+        [&](int r, int e, VT v) { Z[r * xk + e] = v; });
     __syncthreads();
     if (a.A) {  // x_n = A x_parent + Bbar v_n + e_n (App. B), a barrier a node
-      if (tid < n_x) Z[L * n_k + tid] = reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid];
+      if (tid < n_x) Z[L * xk + tid] = reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid];
       for (int r = 0; r < L; ++r) {
         __syncthreads();
-        add_Ax<NW>(As, n_x, false, Z + (r > 0 ? r - 1 : L) * n_k, Z + r * n_k);
+        add_Ax<NW>(As, n_x, false, Z + (r > 0 ? r - 1 : L) * xk, Z + r * xk);
       }
     } else if (tid < n_x)  // x_n = x_parent + Bbar v_n + e_n
-      run_sums(Z, n_k, tid, 0, 1, L, reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid],
-               [&](int r, VT v) { Z[r * n_k + tid] = v; });
+      run_sums<VT>(Z, xk, tid, 0, 1, L, fd ? (VT)0 : reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid],
+               [&](int r, VT v) { Z[r * xk + tid] = v; });
     __syncthreads();
+    if (fd) {
+      const VT* XA = reinterpret_cast<const VT*>(a.ha);
+      for (int r = own + warp; r < L; r += NW)
+        for (int e = lane; e < n_x; e += 32) Z[r * xk + e] += XA[(long long)sid[r] * n_k + e];
+      __syncthreads();
+    }
   }
-  if (len > 0 && (mode & MODE_BWD)) {  // beta, used after the prox
+  if (len > 0 && (mode & MODE_BWD) && !bd) {  // beta, used after the prox
     const VT* beta = reinterpret_cast<const VT*>(a.beta);
     for (int r = own + warp; r < L; r += NW)
-      for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * n_v + j, beta + (long long)sid[r] * n_v + j);
+      for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * xv + j, beta + (long long)sid[r] * n_v + j);
   }
   if (prox) {
     const int rows = L - own, ni = (n_u + 63) / 64;
     for (int task = warp; task < rows * (1 + ni); task += NW) {
       if (task < rows) {
         const int r = own + task;
-        sweep_tanks<VT, NT>(a, sid[r], Z + r * n_k, bnd, nu - 1, c, cn, o);
+        sweep_tanks<VT, NT, B16>(a, sid[r], Z + r * xk, bnd, nu - 1, c, cn, mode, o);
       } else {
         const int q = (task - rows) / ni, r = own + q;
-        sweep_inputs<VT>(a, sid[r], 64 * (task - rows - q * ni), Z + r * n_k, bnd, nu - 1, c, cn, o);
+        sweep_inputs<VT, B16>(a, sid[r], 64 * (task - rows - q * ni), Z + r * xk, bnd, nu - 1, c, cn, mode, o);
       }
     }
     if (o.r.bad() || o.h.bad()) a.flags[1] = SMPC_EDIVERGED;
@@ -425,10 +608,11 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
       const ST* yb = reinterpret_cast<const ST*>((nu & 1) ? a.ybuf0 : a.ybuf1) + (long long)sid[r] * nd;
       for (int e = lane; e < n_k; e += 32) {
         if (e < n_x)
-          Z[r * n_k + e] = st_val(st_add(st_extrap(ld_state(ya + e), ld_state(yb + e), c),
+          Z[r * xk + e] = st_val(st_add(st_extrap(ld_state(ya + e), ld_state(yb + e), c),
                                          st_extrap(ld_state(ya + n_x + e), ld_state(yb + n_x + e), c)));
         else
-          Z[r * n_k + e] = st_val(st_extrap(ld_state(ya + n_x + e), ld_state(yb + n_x + e), c));
+          Z[r * xk + e] = st_val(st_extrap(ld_state(ya + n_x + e), ld_state(yb + n_x + e), c));
+        if (B16) reinterpret_cast<VT*>(a.wa)[(long long)sid[r] * n_k + e] = Z[r * xk + e];  // the first launch anchors
       }
     }
   }
@@ -452,27 +636,30 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
   if (!(mode & MODE_BWD)) return;
   if (len == 0) {  // a top node: its w
     VT* w = reinterpret_cast<VT*>(a.wbuf) + (long long)sid[own] * n_k;
-    for (int e = tid; e < n_k; e += kSweepThreads) w[e] = Z[own * n_k + e];
+    for (int e = tid; e < n_k; e += kSweepThreads) w[e] = Z[own * xk + e];
   } else {
     if (a.A) {  // s_n = xi_n + A' s_child
       for (int r = L - 2; r >= own; --r) {
-        add_Ax<NW>(As, n_x, true, Z + (r + 1) * n_k, Z + r * n_k);
+        add_Ax<NW>(As, n_x, true, Z + (r + 1) * xk, Z + r * xk);
         __syncthreads();
       }
-      if (tid < n_x) reinterpret_cast<VT*>(a.spub)[(long long)sid[own] * n_x + tid] = Z[own * n_k + tid];
+      if (tid < n_x) reinterpret_cast<VT*>(a.spub)[(long long)sid[own] * n_x + tid] = Z[own * xk + tid];
     } else if (tid < n_x) {  // s along the chain, bottom-up
       VT s = 0;
-      run_sums(Z, n_k, tid, L - 1, -1, len, (VT)0, [&](int r, VT v) { Z[r * n_k + tid] = s = v; });
+      run_sums<ST>(Z, xk, tid, L - 1, -1, len, (VT)0, [&](int r, VT v) { Z[r * xk + tid] = s = v; });
       reinterpret_cast<VT*>(a.spub)[(long long)sid[own] * n_x + tid] = s;
     }
     __syncthreads();
-    sparse_rows<NW, VT>(
-        et, cptr, cid, n_v, Z, n_k, own, L, [&](int r, int j) -> VT { return V[r * n_v + j]; },
-        [&](int r, int j, VT v) { V[r * n_v + j] = v; });
+    if constexpr (B16) {
+      if (bd) dense_bwd<NW>(Kd, kw, n_v, Z, xk, own, L, [&](int r, int j, VT v) { V[r * xv + j] = v; });
+    }
+    if (!bd) sparse_rows<NW, VT>(
+        et, cptr, cid, n_v, Z, xk, own, L, [&](int r, int j) -> VT { return V[r * xv + j]; },
+        [&](int r, int j, VT v) { V[r * xv + j] = v; });
     __syncthreads();
     if (tid < n_v) {  // r along the chain
       VT* R = reinterpret_cast<VT*>(a.rpub);
-      run_sums(V, n_v, tid, L - 1, -1, len, (VT)0, [&](int r, VT v) { R[(long long)sid[r] * n_v + tid] = v; });
+      run_sums<ST>(V, xv, tid, L - 1, -1, len, (VT)0, [&](int r, VT v) { R[(long long)sid[r] * n_v + tid] = v; });
     }
   }
   // The last of a top node and its chains forms the node's two terms of r.  With a general A
@@ -480,7 +667,7 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
   // its children forms its s and r, and climbs on.
   const VT* sp = reinterpret_cast<const VT*>(a.spub);
   VT* rp = reinterpret_cast<VT*>(a.rpub);
-  VT *Z0 = Z, *Z1 = Z + n_k, *R0 = Z + 2 * n_k;
+  VT *Z0 = Z, *Z1 = Z + xk, *R0 = Z + 2 * xk;
   const bool climb = a.A != nullptr;
   for (int t = d0.x; t >= 0; t = climb ? a.parent[t] : -1) {
     __syncthreads();  // this CTA's outputs, then one fence, before its arrival
@@ -509,7 +696,7 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
       const int cols = tank ? n_x : n_v, e = tank ? q : q - n_x;
       const VT own_w = tank ? ldcg(wt + e) : reinterpret_cast<const VT*>(a.beta)[(long long)t * n_v + e];
       ST sum = st_from<ST>(0.0);
-      if (!(climb && tank)) st_fma_acc(sum, (VT)1, own_w);
+      if (!(climb && tank) && (tank || !bd)) st_fma_acc(sum, (VT)1, own_w);
       constexpr int C = 8;
       for (int i = 0; i < cc; i += C) {  // children in index order, C loads in flight
         VT v[C];
@@ -533,8 +720,17 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
       __syncthreads();
       if (tid < n_x) reinterpret_cast<VT*>(a.spub)[(long long)t * n_x + tid] = Z0[tid];
     }
-    sparse_rows<NW, VT>(
-        et, cptr, cid, n_v, Z, n_k, 0, climb ? 1 : 2, [&](int r, int j) -> VT { return climb || r == 1 ? R0[j] : (VT)0; },
+    if constexpr (B16) {
+      if (bd)
+        dense_bwd<NW>(Kd, kw, n_v, Z, xk, 0, 2, [&](int r, int j, VT v) {
+          if (r == 1)
+            rp[(long long)t * n_v + j] = v + R0[j];
+          else
+            wt[j] = v;
+        });
+    }
+    if (!bd) sparse_rows<NW, VT>(
+        et, cptr, cid, n_v, Z, xk, 0, climb ? 1 : 2, [&](int r, int j) -> VT { return climb || r == 1 ? R0[j] : (VT)0; },
         [&](int r, int j, VT v) { (climb || r == 1 ? rp + (long long)t * n_v : wt)[j] = v; });
   }
 }
@@ -574,29 +770,6 @@ __global__ void lam_pack_kernel(int n, int n_v, const double* Lam, const double*
 
 // Steps [k0, k1) of one matrix (in shared or global memory) on a warp: acc += the part of
 // Lambda r in row block `lane`.  rs: r, zero-padded to G BS entries, 16-byte aligned.
-// Entries in pairs: two float32 in one register pair and one fused multiply-add instruction
-// (f32x2), or one float64.
-__device__ __forceinline__ unsigned long long f2(float x, float y) {
-  return (unsigned long long)__float_as_uint(x) | ((unsigned long long)__float_as_uint(y) << 32);
-}
-struct PairF {
-  using T = unsigned long long;
-  static constexpr int N = 2;
-  __device__ static T fma(T a, T b, T c) {
-    T d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-  }
-  __device__ static T dup(float x) { return f2(x, x); }
-  __device__ static T zero() { return 0; }
-  __device__ static float sum(T a) { return __uint_as_float((unsigned)a) + __uint_as_float((unsigned)(a >> 32)); }
-  __device__ static float at(T a, int k) { return __uint_as_float((unsigned)(k ? a >> 32 : a)); }
-  __device__ static void ld(const float* p, T (&o)[2]) {
-    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
-    o[0] = t.x;
-    o[1] = t.y;
-  }
-};
 struct PairD {
   using T = double;
   static constexpr int N = 1;
@@ -611,8 +784,8 @@ struct PairD {
     o[1] = t.y;
   }
 };
-template <typename VT, int BS>
-__device__ __forceinline__ void lam_steps(const VT* lam, int G, const VT* rs, int k0, int k1, VT (&out)[BS]) {
+template <typename VT, int BS, typename MT>
+__device__ __forceinline__ void lam_steps(const MT* lam, int G, const VT* rs, int k0, int k1, VT (&out)[BS]) {
   using P = typename std::conditional<sizeof(VT) == 4, PairF, PairD>::type;
   using T = typename P::T;
   constexpr int CE = 16 / (int)sizeof(VT);  // entries of a chunk: two pairs
@@ -628,16 +801,28 @@ __device__ __forceinline__ void lam_steps(const VT* lam, int G, const VT* rs, in
 #pragma unroll
   for (int q = 0; q < NP; ++q) tr[q] = P::zero();
   const int from = I + 1 < G ? I + 1 : 0;
-  const VT* blk = lam + ((long long)k0 * NC * G + I) * CE;
+  // a 16-byte chunk of the matrix: CE entries, or two times CE in bfloat16
+  constexpr int ME = 16 / (int)sizeof(MT), MC = BS * BS / ME;
+  const MT* blk = lam + ((long long)k0 * MC * G + I) * ME;
   int J = I + k0 < G ? I + k0 : I + k0 - G;
 #pragma unroll 2
   for (int k = k0; k < k1; ++k) {
     T A[NC][2], rj[RC][2];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) P::ld(blk + (long long)c * G * CE, A[c]);
+    for (int c = 0; c < MC; ++c) {
+      if constexpr (sizeof(MT) == 2) {
+        const uint4 u = *reinterpret_cast<const uint4*>(blk + (long long)c * G * ME);
+        A[2 * c][0] = bf2(u.x);
+        A[2 * c][1] = bf2(u.y);
+        A[2 * c + 1][0] = bf2(u.z);
+        A[2 * c + 1][1] = bf2(u.w);
+      } else {
+        P::ld(blk + (long long)c * G * ME, A[c]);
+      }
+    }
 #pragma unroll
     for (int c = 0; c < RC; ++c) P::ld(rs + BS * J + c * CE, rj[c]);
-    blk += (long long)NC * G * CE;
+    blk += (long long)MC * G * ME;
     if (++J == G) J = 0;
     if (k > 0) {  // the diagonal blocks are symmetric themselves
 #pragma unroll
@@ -669,13 +854,13 @@ __device__ __forceinline__ void bar_top() { asm volatile("bar.sync 1, 256;" ::: 
 // constants), the following ones as soon as the slot has been read, and with eight warps on an
 // SM (two CTAs) seven copies are in flight while one is used.  One matrix shared by all nodes
 // is copied once per CTA.  slots = 0: a matrix larger than shared memory is read in place.
-template <typename VT>
+template <typename VT, typename MT>
 __host__ __device__ inline size_t lambda_smem_bytes(int n_v, int slots) {
-  return (size_t)round_up((size_t)slots * lam_entries(n_v) * sizeof(VT), 128) + (size_t)kWarps * 32 * kStateSize +
+  return (size_t)round_up((size_t)slots * lam_entries(n_v) * sizeof(MT), 128) + (size_t)kWarps * 32 * kStateSize +
          (size_t)kWarps * 32 * lam_bs(n_v) * sizeof(VT);
 }
 
-template <typename VT, int BS, int LW>
+template <typename VT, typename MT, int BS, int LW>
 __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 : 1)
     lambda_apply(const __grid_constant__ IterArgs a, int slots, int nu, int mode) {
   using ST = typename St<VT>::T;
@@ -691,17 +876,17 @@ __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 
   auto node = [&](int i) { return a.A ? i : a.chain_node[i]; };
   const int G = (n_v + BS - 1) / BS, steps = G / 2 + 1;
   const long long per = lam_entries(n_v);
-  const VT* lam = reinterpret_cast<const VT*>(a.lam);
+  const MT* lam = reinterpret_cast<const MT*>(a.lam);
   VT* delta = reinterpret_cast<VT*>(a.h);
   const bool one = a.lam_stride == 0;  // one matrix for all nodes
   const int cw = one || slots == 0 ? LW : slots;  // chain warps at work
-  VT* slot = reinterpret_cast<VT*>(smem_raw) + (one ? 0 : (long long)warp * per);
+  MT* slot = reinterpret_cast<MT*>(smem_raw) + (one ? 0 : (long long)warp * per);
   int q = (int)blockIdx.x * cw + warp;
   const int dq = (int)gridDim.x * cw;
   const bool chains = warp < cw && q < n_c;
   auto fetch = [&](int m) {  // lane 0: node m's matrix into this warp's slot
-    mbar_expect_tx(&bar[warp], (uint32_t)(per * sizeof(VT)));
-    bulk_g2s(slot, lam + m * a.lam_stride, (uint32_t)(per * sizeof(VT)), &bar[warp]);
+    mbar_expect_tx(&bar[warp], (uint32_t)(per * sizeof(MT)));
+    bulk_g2s(slot, lam + m * a.lam_stride, (uint32_t)(per * sizeof(MT)), &bar[warp]);
   };
   if (slots > 0 && warp < cw && lane == 0) {
     mbar_init(&bar[warp], 1);
@@ -712,7 +897,7 @@ __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 
   const bool mine = one ? warp == 0 : chains;  // a copy of this warp's is under way
   // the top warps: the first top node's sources into shared memory, its matrix towards the L2
   const int tid = (int)threadIdx.x - LW * 32;
-  ST* part = reinterpret_cast<ST*>(smem_raw + round_up((size_t)slots * per * sizeof(VT), 128));  // ng n_v <= 256 sums
+  ST* part = reinterpret_cast<ST*>(smem_raw + round_up((size_t)slots * per * sizeof(MT), 128));  // ng n_v <= 256 sums
   VT* lsum = reinterpret_cast<VT*>(part + kWarps * 32);  // the warps' parts of delta
   const int2* src = reinterpret_cast<const int2*>(a.top_src);
   int s0 = 0, s1 = 0, m_top = 0;
@@ -722,7 +907,7 @@ __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 
     s1 = a.top_src_off[blockIdx.x + 1];
     if (tid < min(kTopList, s1 - s0)) list[tid] = src[s0 + tid];
     const char* lm = reinterpret_cast<const char*>(lam + m_top * a.lam_stride);
-    for (long long o = 128ll * tid; o < per * (long long)sizeof(VT); o += 128ll * 256)
+    for (long long o = 128ll * tid; o < per * (long long)sizeof(MT); o += 128ll * 256)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(lm + o));
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");

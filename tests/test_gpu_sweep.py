@@ -73,3 +73,28 @@ def test_warm_start_and_early_stop():
     assert out[0][:2] == out[1][:2]
     for p, q in zip(out[0][2], out[1][2]):
         assert np.abs(p - q).max() <= BOUND[0] * (1 + np.abs(p).max())
+
+
+@pytest.mark.parametrize("n_x,n_u,n_e", [(2, 4, 0), (3, 7, 2), (33, 66, 5), (30, 128, 0), (31, 129, 0), (65, 131, 3)])
+@pytest.mark.parametrize("anchor_every,polish", [(16, 0), (3, 4), (1, 0)])
+def test_bf16_per_node(n_x, n_u, n_e, anchor_every, polish):
+    """bfloat16 packs, one per node: the two-launch form applies the same bfloat16 matrices to
+    float32 vectors as schedule 1 and anchors in float32 in another basis, so the iterates
+    agree as float32 ones do (1e-4), far inside the distance to the oracle."""
+    P = synth.custom(54, n_x, n_u, max(n_e, 3), n_e, TREES["fan"] if n_x < 60 else LATE)
+    tree, fac, _ = H.oracle_build(P)
+    steps = oracle.jacobi_steps(fac, tree)
+    out = []
+    for schedule in (1, 0):
+        g = H.Gpu(P, steps=steps, precision=2, schedule=schedule)
+        try:
+            if schedule == 0 and not _uses_sweep(g, P):
+                pytest.skip("another schedule was faster here")
+            info = g.smpc.smpc_solve(g.fac, P["p"], P["q"], P["dhat"], P["alpha2"], eps=P["eps"], max_iters=40, sync=1,
+                                     anchor_every=anchor_every, polish_iters=polish, u=g.u, x=g.x, y=g.y)
+            out.append((info["rho_rel"], g.arrays()))
+        finally:
+            g.close()
+    assert abs(out[0][0] - out[1][0]) <= BOUND[1]
+    for p, q in zip(out[0][1], out[1][1]):
+        assert np.abs(p - q).max() <= BOUND[1] * (1 + np.abs(p).max())
