@@ -3316,6 +3316,14 @@ LaunchCfg config_t(const IterArgs& a, int num_sms, int S_max, int schedule, int 
   c.s_dh = S;
   c.smem_dh = iter_smem_bytes<MT>(S > 0 ? S : 1, a.n_x, a.n_u, a.n_v, true);
   if (c.s_gt < 1 || c.s_dh < 1) c.stages = 0;
+  if (schedule == SCHED_NODE && a.kd && a.pack_stride == 0 && !a.A && sizeof(VT) == 4 && c.stages > 0) {
+    c.smem = hsweep_smem_bytes<VT>(a.depth, a.n_x, a.n_u);
+    if (c.smem + 512 <= (size_t)optin) {
+      c.hsweep = true;
+      c.grid = a.n_chains + a.n_top;
+      c.sweep_warps = a.n_x > 64 || a.n_chains <= 2 * num_sms ? 16 : 8;
+    }
+  }
   // shared pack: kNB nodes per pass when the pack and the staging fit
   c.multi_gt = c.multi_dh = false;
   c.tc = false;
@@ -3368,15 +3376,21 @@ template <typename VT>
 auto sweep_kernel(const IterArgs& a, int warps) {
   if constexpr (sizeof(VT) == 4) {
     if (a.kd)
-      return a.n_x <= 32   ? tree_sweep<VT, 1, 16, true>
-             : a.n_x <= 64 ? tree_sweep<VT, 2, 16, true>
-                           : tree_sweep<VT, 8, 16, true>;
-    if (warps == 32) return a.n_x <= 32 ? tree_sweep<VT, 1, 32, false> : tree_sweep<VT, 2, 32, false>;
+      return a.n_x <= 32   ? tree_sweep<VT, 1, 16, 1>
+             : a.n_x <= 64 ? tree_sweep<VT, 2, 16, 1>
+                           : tree_sweep<VT, 8, 16, 1>;
+    if (warps == 32) return a.n_x <= 32 ? tree_sweep<VT, 1, 32, 0> : tree_sweep<VT, 2, 32, 0>;
   }
-  if (warps == 8) return a.n_x <= 32 ? tree_sweep<VT, 1, 8, false> : tree_sweep<VT, 2, 8, false>;
-  return a.n_x <= 32   ? tree_sweep<VT, 1, 16, false>
-         : a.n_x <= 64 ? tree_sweep<VT, 2, 16, false>
-                       : tree_sweep<VT, 8, 16, false>;
+  if (warps == 8) return a.n_x <= 32 ? tree_sweep<VT, 1, 8, 0> : tree_sweep<VT, 2, 8, 0>;
+  return a.n_x <= 32   ? tree_sweep<VT, 1, 16, 0>
+         : a.n_x <= 64 ? tree_sweep<VT, 2, 16, 0>
+                       : tree_sweep<VT, 8, 16, 0>;
+}
+
+template <typename VT>
+auto hsweep_kernel(const IterArgs& a, int warps) {
+  if (warps == 8) return a.n_x <= 32 ? tree_sweep<VT, 1, 8, 2> : tree_sweep<VT, 2, 8, 2>;
+  return a.n_x <= 32 ? tree_sweep<VT, 1, 16, 2> : a.n_x <= 64 ? tree_sweep<VT, 2, 16, 2> : tree_sweep<VT, 8, 16, 2>;
 }
 
 template <typename VT, typename MT>
@@ -3409,7 +3423,10 @@ int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream
         t.kd = nullptr;
         if (n_x <= 64 || warps == 16) allow(sweep_kernel<VT>(t, warps));
         t.kd = &t;  // any address: the bfloat16 factors' kernels
-        if (sizeof(VT) == 4) allow(sweep_kernel<VT>(t, warps));
+        if constexpr (sizeof(VT) == 4) {
+          allow(sweep_kernel<VT>(t, warps));
+          allow(hsweep_kernel<VT>(t, warps));
+        }
       }
     allow(lambda_apply<VT, MT, 4, 8>);
     allow(lambda_apply<VT, MT, 8, 8>);
@@ -3447,12 +3464,23 @@ int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream
     }
     return check_launch("tree sweep");
   }
-  if ((mode & MODE_PROX) && nu >= 1) {
+  // bfloat16 factors with one pack on schedule 2: forward sweep, prox and s in one launch
+  bool swept = false;
+  if constexpr (sizeof(VT) == 4) {
+    if (c.hsweep) {
+      launch_dep(hsweep_kernel<VT>(a, c.sweep_warps), c.grid, 32 * c.sweep_warps, c.smem, s, dep && nu > 0, a, nu, mode);
+      mark();
+      swept = true;
+    }
+  }
+  if (!swept && (mode & MODE_PROX) && nu >= 1) {
     launch_dep(fwd_scan<VT, MT>, c.grid_fwd, c.block, c.smem_fwd, s, dep, a, nu, mode);
     mark();
   }
-  launch_dep(prox_node<VT, MT>, c.grid_prox, c.block, c.smem_pstage, s, dep, a, nu, mode);
-  mark();
+  if (!swept) {
+    launch_dep(prox_node<VT, MT>, c.grid_prox, c.block, c.smem_pstage, s, dep, a, nu, mode);
+    mark();
+  }
   if ((mode & MODE_BWD) && c.schedule == SCHED_FUSED) {
     // the whole backward sweep (s, [Bbar; L]'[s; psi], r, Lambda r / (2 p) and [Bbar; L] delta)
     // along the chains and up the top nodes: every pack is read once per iteration
@@ -3480,8 +3508,10 @@ int launch_t(const IterArgs& a, const LaunchCfg& c, int nu, int mode, cudaStream
     }
     mark();
   } else if (mode & MODE_BWD) {
-    launch_dep(scan_kernel<VT>, c.grid_scan, c.block, 0, s, dep, a, 0, nu, mode);
-    mark();
+    if (!swept) {
+      launch_dep(scan_kernel<VT>, c.grid_scan, c.block, 0, s, dep, a, 0, nu, mode);
+      mark();
+    }
     bool gt_done = false;
     if constexpr (std::is_same<MT, __nv_bfloat16>::value) {
       if (c.tc && c.tc_gt && (mode & MODE_DELTA)) {

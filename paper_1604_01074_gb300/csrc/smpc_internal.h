@@ -218,6 +218,7 @@ struct LaunchCfg {
   // hybrid schedule: the backward sweep up to r runs as the chain kernel in MODE_GT
   int grid_chain = 1, stages_chain = 0;
   size_t smem_chain = 0;
+  bool hsweep = false;      // bfloat16, one pack, schedule 2: forward sweep, prox and s in one launch (grid, smem)
   int sweep_warps = 16, grid_lam = 1, lam_slots = 0, lam_warps = 8;  // SCHED_SWEEP: the Lambda launch (the tree pass: grid, smem)
   size_t smem_lam = 0;
   // profiling: when set, an event is recorded before the first and after every kernel
@@ -228,6 +229,7 @@ struct LaunchCfg {
 inline int kernels_per_call(const LaunchCfg& c, int mode) {
   if (c.schedule == SCHED_CHAIN) return 1;
   if (c.schedule == SCHED_SWEEP) return 1 + ((mode & MODE_BWD) ? 1 : 0);
+  if (c.hsweep) return 1 + ((mode & MODE_BWD) ? 3 : 0);
   const int bwd = c.schedule == SCHED_HYBRID ? 2 : c.schedule == SCHED_FUSED ? 1 : 4;
   return 1 + ((mode & MODE_PROX) ? 1 : 0) + ((mode & MODE_BWD) ? bwd : 0);
 }

@@ -176,10 +176,20 @@ struct SweepOut {
 // Anchored solves (bfloat16 packs, B16): a delta launch takes w - w_a, exactly in the state
 // type; an anchor stores w_a = w; the launch after an anchor stores x and u, from which those
 // up to the next anchor continue with the linear part.
-template <typename VT, int NT, bool B16>
+// FORM 2 (the tensor-core path) keeps every operation of warp_prox_staged: its vectors are
+// rounded to bfloat16 further on, where a last bit more or less turns into 2^-9.
+template <int FORM, typename ST, typename AT>
+__device__ __forceinline__ ST form_extrap(ST y1, ST y2, AT c) {
+  if constexpr (FORM == 2)
+    return st_extrap(y1, y2, c);
+  else
+    return sw_extrap(y1, y2, c);
+}
+template <typename VT, int NT, int FORM>
 __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, const VT* bnd, int it, VT c, VT cn, int mode,
                                             SweepOut<VT>& o) {
   using ST = typename St<VT>::T;
+  constexpr bool B16 = FORM != 0;
   const int lane = threadIdx.x & 31, n_x = a.n_x, nd = 2 * n_x + a.n_u;
   const VT *xs = bnd, *xhi = xs + n_x, *xlo = xhi + n_x;
   const ST* y1 = reinterpret_cast<const ST*>((it & 1) ? a.ybuf1 : a.ybuf0) + (long long)m * nd;
@@ -217,8 +227,8 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
     qs[k] = qz[k] = zero;
     if (e < n_x) {
       const VT x = z[e];
-      ws[k] = sw_extrap(v1[k], ws[k], c);
-      wz[k] = sw_extrap(w1[k], wz[k], c);
+      ws[k] = form_extrap<FORM>(v1[k], ws[k], c);
+      wz[k] = form_extrap<FORM>(w1[k], wz[k], c);
       const ST q = st_axpy(ws[k], ls, x - xs[e]);
       qs[k] = sw_neg(q) ? q : zero;  // C = {x >= x_s}
       qz[k] = sw_box(st_axpy(wz[k], lz, x - xhi[e]), st_axpy(wz[k], lz, x - xlo[e]));
@@ -237,7 +247,7 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
   for (int d = 8; d > 0; d >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, d);
   const VT mu = lo ? mus : muz;
   VT kap = 1;
-  if (!(sq <= mu * mu)) {
+  if (FORM == 2 || !(sq <= mu * mu)) {
     const VT dist = sqrt(sq);
     kap = dist > mu ? mu / dist : (VT)1;
   }
@@ -272,10 +282,11 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
     }
   }
 }
-template <typename VT, bool B16>
+template <typename VT, int FORM>
 __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, VT* z, const VT* bnd, int it, VT c, VT cn,
                                              int mode, SweepOut<VT>& o) {
   using ST = typename St<VT>::T;
+  constexpr bool B16 = FORM != 0;
   constexpr int NU = 2;
   const int lane = threadIdx.x & 31, n_x = a.n_x, n_u = a.n_u, nd = 2 * n_x + n_u;
   const VT *uhi = bnd + 3 * n_x, *ulo = uhi + n_u;
@@ -304,7 +315,7 @@ __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, V
     const int i = i0 + lane + 32 * k;
     if (i < n_u) {
       const VT u = z[n_x + i];
-      const ST wp = sw_extrap(p1[k], p2[k], c);
+      const ST wp = form_extrap<FORM>(p1[k], p2[k], c);
       const ST ypn = sw_box(st_axpy(wp, lp[k], u - uhi[i]), st_axpy(wp, lp[k], u - ulo[i]));
       const VT ep = sw_diff(ypn, wp) * ip[k];
       st_state(y2 + i, ypn);
@@ -460,17 +471,29 @@ __device__ __forceinline__ void add_Ax(const VT* A, int n, bool trans, const VT*
 // memory or shared memory with few warps busy, so trees with several chains an SM run four
 // small CTAs there, side by side in different phases; trees with at most a chain an SM have
 // nothing to overlap and spread each chain over as many warps as an SM takes.
-template <typename VT, int NT, int NW, bool B16>
+//
+// FORM 0: float64 and float32 factors.  1: bfloat16 factors with a pack per node (see
+// dense_fwd).  2: bfloat16 factors with one pack, whose products stay on the tensor cores:
+// the first half of an iteration of schedule 2 in one launch - path sums of h, prox, s of every
+// node - with the arithmetic of fwd_scan, prox_node and scan_kernel, in place of those three:
+// 38 us instead of 73 on 13 830 nodes and 20 tanks, 72 instead of 109 on 15 876 nodes and 63.
+template <typename VT>
+__host__ __device__ inline size_t hsweep_smem_bytes(int depth, int n_x, int n_u) {
+  const size_t b = round_up((size_t)(3 * n_x + 2 * n_u) * sizeof(VT), 16) + (size_t)3 * (depth + 3) * (n_x + n_u) * sizeof(VT);
+  return round_up(b + (size_t)depth * sizeof(int), 16);
+}
+template <typename VT, int NT, int NW, int FORM>
 __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 : 16) / NW)
     tree_sweep(const __grid_constant__ IterArgs a, int nu, int mode) {
   using ST = typename St<VT>::T;
   constexpr int kSweepThreads = 32 * NW;
+  constexpr bool B16 = FORM == 1, H = FORM == 2;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int flag[2];
   __shared__ VT red[3 * NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n_x = a.n_x, n_u = a.n_u, n_k = a.n_k, n_v = a.n_v, nnz = a.sp_nnz;
+  const int n_x = a.n_x, n_u = a.n_u, n_k = a.n_k, n_v = a.n_v, nnz = H ? 0 : a.sp_nnz;
   const bool prox = (mode & MODE_PROX) != 0 && nu >= 1;
   // bfloat16 factors: the forward part continues a delta launch, the backward part is one
   // (both in the orthonormal basis of the packs); else they are the anchors' float32 ones
@@ -479,18 +502,20 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
   // ---- read while the previous launch drains: constants of the factor and the tree, and the
   // solve's affine data, complete before its first launch (nu = 0), which starts without
   // programmatic overlap
-  const int blob = sp_bytes<VT>(nnz, n_k, n_v);
+  const int blob = H ? 0 : sp_bytes<VT>(nnz, n_k, n_v);
   const SpEnt<VT>* ek = reinterpret_cast<const SpEnt<VT>*>(smem_raw);
   const SpEnt<VT>* et = ek + nnz;
   const int* rptr = reinterpret_cast<const int*>(et + nnz);
   const int *rid = rptr + n_k + 1, *cptr = rid + n_k, *cid = cptr + n_v + 1;
   VT* bnd = reinterpret_cast<VT*>(smem_raw + blob);
   VT* V = reinterpret_cast<VT*>(smem_raw + blob + round_up((3 * n_x + 2 * n_u) * (int)sizeof(VT), 16));  // delta, then v, then beta, g and r: a row of n_v per node
-  VT* Z = V + (a.depth + 3) * xv;  // e and u_hat, then x and u, then w and s: a row of n_k per node
+  VT* Z = H ? V : V + (a.depth + 3) * xv;  // e and u_hat, then x and u, then w and s: a row of n_k per node
+  VT* HA = Z + (a.depth + 3) * xk;   // FORM 2: h_a, then e and u_hat, a row of n_k per node each
+  VT* HE = HA + (a.depth + 3) * xk;
   VT* As = Z + (a.depth + 3) * xk;  // a general state matrix
   uint32_t* Kd = reinterpret_cast<uint32_t*>(As + (a.A ? n_x * n_x : 0));  // B16: the dense [Bbar; L]
   const int kw = dense_kw(n_v);
-  int* sid = reinterpret_cast<int*>(Kd + (B16 ? xk * kw : 0));
+  int* sid = H ? reinterpret_cast<int*>(HE + (a.depth + 3) * xk) : reinterpret_cast<int*>(Kd + (B16 ? xk * kw : 0));
   if (B16) {
     const int ld = row_stride<__nv_bfloat16>(n_v);  // even
     const uint32_t* src = reinterpret_cast<const uint32_t*>(a.kd);
@@ -528,15 +553,22 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
     const VT* UH = reinterpret_cast<const VT*>(a.uhat);
     for (int r = warp; r < L; r += NW) {
       const long long m = sid[r];
-      for (int e = lane; e < n_x; e += 32) cp_async_elem(Z + r * xk + e, E + m * n_x + e);
+      VT* to = (H ? HE : Z) + r * xk;
+      for (int e = lane; e < n_x; e += 32) cp_async_elem(to + e, E + m * n_x + e);
       if (r >= own)
-        for (int i = lane; i < n_u; i += 32) cp_async_elem(Z + r * xk + n_x + i, UH + m * n_u + i);
+        for (int i = lane; i < n_u; i += 32) cp_async_elem(to + n_x + i, UH + m * n_u + i);
     }
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (prox) {
     const VT* delta = reinterpret_cast<const VT*>(a.h);
-    for (int r = warp; r < L; r += NW)
+    if (H)
+      for (int r = warp; r < L; r += NW)
+        for (int e = lane; e < n_k; e += 32) {
+          cp_async_elem(Z + r * xk + e, delta + (long long)sid[r] * n_k + e);
+          cp_async_elem(HA + r * xk + e, reinterpret_cast<const VT*>(a.ha) + (long long)sid[r] * n_k + e);
+        }
+    for (int r = H ? L : warp; r < L; r += NW)
       for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * xv + j, delta + (long long)sid[r] * n_v + j);
     if (fd)  // the anchor's u (its x is added after the linear path sums)
       for (int r = own + warp; r < L; r += NW)
@@ -550,6 +582,22 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
   SweepOut<VT> o;
   if (prox) {
     __syncthreads();
+    if (H) {  // path sums of h + h_a, as in fwd_scan
+      for (int e = tid; e < n_k; e += kSweepThreads) {
+        VT v = 0, x = e < n_x ? reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + e] : (VT)0;
+#pragma unroll 4
+        for (int r = 0; r < L; ++r) {
+          v += Z[r * xk + e] + HA[r * xk + e];
+          const VT ev = e < n_x || r >= own ? HE[r * xk + e] : (VT)0;
+          if (e < n_x)
+            x += v + ev;
+          else
+            x = v + ev;
+          Z[r * xk + e] = x;
+        }
+      }
+      __syncthreads();
+    } else {
     if (tid < n_v)  // v along the path
       run_sums<VT>(V, xv, tid, 0, 1, L, (VT)0, [&](int r, VT v) { V[r * xv + tid] = v; });
     __syncthreads();
@@ -583,21 +631,23 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
         for (int e = lane; e < n_x; e += 32) Z[r * xk + e] += XA[(long long)sid[r] * n_k + e];
       __syncthreads();
     }
+    }
   }
-  if (len > 0 && (mode & MODE_BWD) && !bd) {  // beta, used after the prox
+  if (!H && len > 0 && (mode & MODE_BWD) && !bd) {  // beta, used after the prox
     const VT* beta = reinterpret_cast<const VT*>(a.beta);
     for (int r = own + warp; r < L; r += NW)
       for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * xv + j, beta + (long long)sid[r] * n_v + j);
   }
   if (prox) {
+    const int pmode = H ? mode & ~MODE_AFTER_ANCHOR : mode;  // FORM 2 keeps h_a, not x and u
     const int rows = L - own, ni = (n_u + 63) / 64;
     for (int task = warp; task < rows * (1 + ni); task += NW) {
       if (task < rows) {
         const int r = own + task;
-        sweep_tanks<VT, NT, B16>(a, sid[r], Z + r * xk, bnd, nu - 1, c, cn, mode, o);
+        sweep_tanks<VT, NT, FORM>(a, sid[r], Z + r * xk, bnd, nu - 1, c, cn, pmode, o);
       } else {
         const int q = (task - rows) / ni, r = own + q;
-        sweep_inputs<VT, B16>(a, sid[r], 64 * (task - rows - q * ni), Z + r * xk, bnd, nu - 1, c, cn, mode, o);
+        sweep_inputs<VT, FORM>(a, sid[r], 64 * (task - rows - q * ni), Z + r * xk, bnd, nu - 1, c, cn, pmode, o);
       }
     }
     if (o.r.bad() || o.h.bad()) a.flags[1] = SMPC_EDIVERGED;
@@ -612,7 +662,7 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
                                          st_extrap(ld_state(ya + n_x + e), ld_state(yb + n_x + e), c)));
         else
           Z[r * xk + e] = st_val(st_extrap(ld_state(ya + n_x + e), ld_state(yb + n_x + e), c));
-        if (B16) reinterpret_cast<VT*>(a.wa)[(long long)sid[r] * n_k + e] = Z[r * xk + e];  // the first launch anchors
+        if (FORM != 0) reinterpret_cast<VT*>(a.wa)[(long long)sid[r] * n_k + e] = Z[r * xk + e];  // the first launch anchors
       }
     }
   }
@@ -634,6 +684,42 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
     if (a.res_tree) atomic_max_nonneg(a.res_tree + 3ll * ((long long)(nu - 1) * a.R + tree) + k, (double)v);
   }
   if (!(mode & MODE_BWD)) return;
+  if constexpr (H) {  // w and s of every node (scan_kernel's sums); the top nodes' by last arrival
+    VT* S = reinterpret_cast<VT*>(a.spub);
+    for (int r = own + warp; r < L; r += NW)
+      for (int e = lane; e < n_k; e += 32) reinterpret_cast<VT*>(a.wbuf)[(long long)sid[r] * n_k + e] = Z[r * xk + e];
+    if (len > 0 && tid < n_x)
+      run_sums<VT>(Z, xk, tid, L - 1, -1, len, (VT)0, [&](int r, VT v) { S[(long long)sid[r] * n_x + tid] = v; });
+    for (int t = d0.x; t >= 0; t = a.parent[t]) {
+      __syncthreads();
+      if (tid == 0) {
+        fence_acq_rel_gpu();
+        const int last = atomicAdd(&a.counters[t], 1) == a.top_expect[t] - 1;
+        if (last) {
+          a.counters[t] = 0;
+          fence_acq_rel_gpu();
+        }
+        flag[1] = last;
+      }
+      __syncthreads();
+      if (!flag[1]) return;
+      const int c0 = a.child_begin[t], cc = a.child_count[t];
+      for (int e = tid; e < n_x; e += kSweepThreads) {
+        VT v = ldcg(reinterpret_cast<const VT*>(a.wbuf) + (long long)t * n_k + e);
+        constexpr int C = 8;
+        for (int i = 0; i < cc; i += C) {
+          VT u[C];
+#pragma unroll
+          for (int k = 0; k < C; ++k) u[k] = i + k < cc ? ldcg(S + (long long)(c0 + i + k) * n_x + e) : (VT)0;
+#pragma unroll
+          for (int k = 0; k < C; ++k)
+            if (i + k < cc) v += u[k];
+        }
+        S[(long long)t * n_x + e] = v;
+      }
+    }
+    return;
+  } else {
   if (len == 0) {  // a top node: its w
     VT* w = reinterpret_cast<VT*>(a.wbuf) + (long long)sid[own] * n_k;
     for (int e = tid; e < n_k; e += kSweepThreads) w[e] = Z[own * xk + e];
@@ -732,6 +818,7 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
     if (!bd) sparse_rows<NW, VT>(
         et, cptr, cid, n_v, Z, xk, 0, climb ? 1 : 2, [&](int r, int j) -> VT { return climb || r == 1 ? R0[j] : (VT)0; },
         [&](int r, int j, VT v) { (climb || r == 1 ? rp + (long long)t * n_v : wt)[j] = v; });
+  }
   }
 }
 
