@@ -123,7 +123,7 @@ typedef struct smpc_factor_opts {
    * sweep and prox, then the whole backward sweep as one chain pass (every pack read once
    * per iteration); 0 = time all of them on this GPU when the factor is built and keep the
    * fastest.  Where [Bbar; L] is sparse (at most 4096 entries in the reduced basis,
-   * float64, float32, or SMPC_BF16 with a pack per node) 0 also times a two-launch form of 4 - a tree pass with the sparse
+   * float64, float32, or SMPC_BF16 with a pack per node and at most 18 stages) 0 also times a two-launch form of 4 - a tree pass with the sparse
    * products inside, and Lambda r of every node - which is reported as 4 (with a general A,
    * as 2).  Results agree to
    * rounding. */

@@ -1039,10 +1039,10 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   // that may choose its schedule.  A bfloat16 factor's anchors run it in float32 in the reduced
   // basis, its delta launches on the packs' own [Bbar; L] and Lambda; with one pack for all
   // nodes those round vectors to bfloat16 for the tensor cores, in an order that the two-launch
-  // form does not keep.
+  // form does not keep. Deep trees (kB16Stages) keep schedules 1 to 4 as well.
   const size_t lam_bytes = (size_t)np * lam_pack_entries(n_v) * f->ms, lam32_bytes = (size_t)np * lam_pack_entries(n_v) * 4;
   const bool b16 = f->prec == SMPC_BF16;
-  if (o.schedule == 0 && !tree->top_src_off.empty() && !(b16 && (f->shared_packs || general_A))) {
+  if (o.schedule == 0 && !tree->top_src_off.empty() && !(b16 && (f->shared_packs || general_A || tree->N > kB16Stages))) {
     HostFactor red;
     const HostFactor* hs = &f->hf;
     if (b16) {

@@ -21,7 +21,7 @@
 // Per iteration on GB300, one pack per node (the launches of schedules 2 to 4 before): 2081
 // nodes 27.2 us in float32 (104), 116 us in float64 (381); 21 111 nodes 145 us (577), the tree
 // pass 71 and Lambda 75; one pack for all of 21 111 nodes 107 us (396).  The tree pass is bound
-// by issue slots (some 1900 warp instructions a node, half of them the prox in float32 pairs),
+// by issue slots (some 2400 warp instructions a node, half of them the prox in float32 pairs),
 // Lambda by HBM (439 MB at 5.9 TB/s) and in float64 by the pipe (2 lanes a cycle and SM).
 // Vectors between the launches: h holds delta (n x n_v), rpub r of the chain nodes, spub s of
 // the chain heads; a top node m's row of rpub holds R_m + L' psi_m, the first n_v entries of
@@ -392,8 +392,8 @@ __device__ __forceinline__ unsigned long long bf2(uint32_t u) {
 // rows at a time.  Forward: put(r, e, (K V_r)_e), a lane per row e of K; the four rows' entries
 // are broadcast reads, and pairs of products go through f32x2.  Backward: put(r, j, (K' Z_r)_j),
 // two columns a lane.  They double the pass's instructions (about 550 and 800 a node at 177 x
-// 97 entries); streaming each node's own copy of K through the chains instead took 460 us of a
-// 21 111-node iteration.
+// 97 entries): 174 us on 21 111 nodes, against 457 us for streaming each node's own copy of K
+// through the chains.
 template <int NW, typename F>
 __device__ __forceinline__ void dense_fwd(const uint32_t* K, int kw, int n_k, const float* V, int xv, int r0, int r1,
                                           F&& put) {
