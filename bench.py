@@ -425,6 +425,8 @@ def kernel_roofline(S, P, prec, inp, stream, fp64_peak, iters=200):
     stage_ms = S.smpc.smpc_profile_solve(S.fac, host["p"], host["q"], host["dhat"], host["alpha2"], eps=P["eps"],
                                          iters=iters)
     names = stages_of(S.schedule, stage_ms)
+    if names is SWEEP_STAGES:  # what the two-launch form must move: one half of Lambda, no pack
+        nbytes = sum(stage_bytes(k, S.n, S.n_x, S.n_u, n_v, prec, False) for k in names)
     hbm, src = peaks()
     if S.schedule == 1:
         kern, k_ms, k_bytes = "apg_iter", stage_ms[0], nbytes
