@@ -123,10 +123,13 @@ typedef struct smpc_factor_opts {
    * sweep and prox, then the whole backward sweep as one chain pass (every pack read once
    * per iteration); 0 = time all of them on this GPU when the factor is built and keep the
    * fastest.  Where [Bbar; L] is sparse (at most 4096 entries in the reduced basis,
-   * float64, float32, or SMPC_BF16 with a pack per node and at most 18 stages) 0 also times a two-launch form of 4 - a tree pass with the sparse
-   * products inside, and Lambda r of every node - which is reported as 4 (with a general A,
-   * as 2).  Results agree to
-   * rounding. */
+   * float64, float32, or SMPC_BF16 with a pack per node and at most 18 stages) 0 also times a
+   * two-launch form of 4 - a tree pass with the sparse products inside, and Lambda r of every
+   * node - which is reported as 4 (with a general A, as 2).  Results agree to rounding.
+   * Diagnostics: smpc_factor reads the environment variable SMPC_ITERATION_FORM.  With
+   * "two-launch", 0 takes the two-launch form without timing (SMPC_ENOTSUP where it does not
+   * fit), so that a program or test can rely on it; with "separate" 0 considers 1 to 4 only,
+   * and schedule 2 of SMPC_BF16 with shared packs runs its first three launches one by one. */
   int32_t schedule;
   /* SMPC_BF16 with shared_packs = 1: the Lambda and [Bbar; L] products of the delta
    * iterations (and, on the node-parallel schedule 2, their [Bbar; L]' products) run on the

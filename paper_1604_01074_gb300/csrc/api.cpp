@@ -303,7 +303,7 @@ void set_sweep_args(const smpc_factor_t* f, IterArgs& a) {
   const smpc_tree* t = f->tree;
   a.sp = t->top_src_off.empty() ? nullptr : f->sp;
   a.sp_nnz = f->sp_nnz;
-  a.kd = f->prec == SMPC_BF16 ? f->packs : nullptr;
+  a.kd = f->prec == SMPC_BF16 && f->form != FORM_SEPARATE ? f->packs : nullptr;
   a.depth = t->N;
   a.max_len = t->max_chain_len;
   a.lam = f->lam;
@@ -572,6 +572,14 @@ int choose_schedule(smpc_factor_t* f, int requested) {
       return SMPC_ENOTSUP;
     }
     f->schedule = requested;
+    return SMPC_OK;
+  }
+  if (f->form == FORM_TWO_LAUNCH) {
+    if (!fits[SCHED_SWEEP]) {
+      set_error("the two-launch form does not fit this network, tree or precision");
+      return SMPC_ENOTSUP;
+    }
+    f->schedule = SCHED_SWEEP;
     return SMPC_OK;
   }
   if (n_fit <= 1) {
@@ -959,6 +967,9 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
     const unsigned long long v = std::strtoull(w, &end, 10);
     if (end != w) f->wait_ns = v;
   }
+  // Diagnostics: the iteration form without timing (smpc_factor_opts.schedule)
+  if (const char* w = std::getenv("SMPC_ITERATION_FORM"))
+    f->form = !std::strcmp(w, "two-launch") ? FORM_TWO_LAUNCH : !std::strcmp(w, "separate") ? FORM_SEPARATE : FORM_TIMED;
   const int n = f->n, n_k = f->n_k, nd = f->nd;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&f->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -1042,7 +1053,7 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   // form does not keep. Deep trees (kB16Stages) keep schedules 1 to 4 as well.
   const size_t lam_bytes = (size_t)np * lam_pack_entries(n_v) * f->ms, lam32_bytes = (size_t)np * lam_pack_entries(n_v) * 4;
   const bool b16 = f->prec == SMPC_BF16;
-  if (o.schedule == 0 && !tree->top_src_off.empty() && !(b16 && (f->shared_packs || general_A || tree->N > kB16Stages))) {
+  if (o.schedule == 0 && f->form != FORM_SEPARATE && !tree->top_src_off.empty() && !(b16 && (f->shared_packs || general_A || tree->N > kB16Stages))) {
     HostFactor red;
     const HostFactor* hs = &f->hf;
     if (b16) {

@@ -192,6 +192,9 @@ constexpr int kSchedules = 4;
 // tree pass and one Lambda launch per iteration (sweep.cuh).  Reported as schedule 4, with a
 // general A as schedule 2, the one that carries it.
 constexpr int SCHED_SWEEP = 5;
+// Which launches a factor's iterations may use (SMPC_ITERATION_FORM, read by smpc_factor):
+// chosen by timing, SCHED_SWEEP without timing, or those of schedules 1 to 4 one by one.
+enum IterForm : int { FORM_TIMED = 0, FORM_TWO_LAUNCH, FORM_SEPARATE };
 // Entries of [Bbar; L] up to which it counts as sparse: its image is read into shared memory
 // by every CTA of the tree pass (64 KB at this size in float32).
 constexpr int kSparseMax = 4096;
@@ -392,6 +395,7 @@ struct smpc_factor_t {
   int last_launches = 0;
   int num_sms = 0;
   int schedule = smpc::SCHED_CHAIN;  // iteration schedule in use
+  int form = smpc::FORM_TIMED;
   void *sp = nullptr, *lam = nullptr;  // SCHED_SWEEP: sparse [Bbar; L], packed Lambda
   // ... of a bfloat16 factor: the anchors' float32 Lambda and cost-update matrices, in the
   // reduced basis (lam: bfloat16, in the basis of the packs)
