@@ -536,6 +536,93 @@ int power_iteration(smpc_factor_t* f, int iters, double* out) {
   return SMPC_OK;
 }
 
+int upload64(smpc_factor_t* f, double** dst, const double* src, size_t cnt) {
+  TRY(f->alloc(dst, cnt * sizeof(double)));
+  if (cnt) CK(cudaMemcpy(*dst, src, cnt * sizeof(double), cudaMemcpyHostToDevice));
+  return SMPC_OK;
+}
+
+// The nonzero entries of a rows x cols matrix at(i, j), row by row.
+template <typename F>
+int upload_csr(smpc_factor_t* f, CsrRows* out, int rows, int cols, F&& at) {
+  std::vector<int> ptr(1, 0), col;
+  std::vector<double> val;
+  for (int i = 0; i < rows; ++i) {
+    for (int j = 0; j < cols; ++j)
+      if (at(i, j) != 0.0) {
+        col.push_back(j);
+        val.push_back(at(i, j));
+      }
+    ptr.push_back((int)col.size());
+  }
+  int *dp = nullptr, *dc = nullptr;
+  double* dv = nullptr;
+  TRY(f->alloc(&dp, ptr.size() * sizeof(int)));
+  TRY(f->alloc(&dc, col.size() * sizeof(int)));
+  TRY(upload64(f, &dv, val.data(), val.size()));
+  CK(cudaMemcpy(dp, ptr.data(), ptr.size() * sizeof(int), cudaMemcpyHostToDevice));
+  if (!col.empty()) CK(cudaMemcpy(dc, col.data(), col.size() * sizeof(int), cudaMemcpyHostToDevice));
+  out->ptr = dp;
+  out->col = dc;
+  out->val = dv;
+  return SMPC_OK;
+}
+
+// The matrices of the two-launch form of schedule 4 (with a general A: of schedule 2), for a
+// factor that may choose its schedule; f->lam stays NULL where the form does not apply.  A
+// bfloat16 factor's anchors run it in float32 in the reduced basis, its delta launches on the
+// packs' own [Bbar; L] and Lambda; with one pack for all nodes those round vectors to bfloat16
+// for the tensor cores, in an order that the two-launch form does not keep.  Deep trees
+// (kB16Stages) keep schedules 1 to 4 as well.
+int build_two_launch(smpc_factor_t* f, const smpc_network& net, const double* W_u) {
+  const smpc_tree* tree = f->tree;
+  const int n_x = f->n_x, n_u = f->n_u, n_v = f->n_v, n_k = f->n_k;
+  const bool b16 = f->prec == SMPC_BF16;
+  if (f->form == FORM_SEPARATE || tree->top_src_off.empty() ||
+      (b16 && (f->shared_packs || f->A || tree->N > kB16Stages)))
+    return SMPC_OK;
+  HostFactor red;
+  const HostFactor* hs = &f->hf;
+  if (b16) {
+    TRY(host_factor(net, W_u, red, true));
+    hs = &red;
+  }
+  std::vector<double> Ks((size_t)n_k * n_v);
+  std::copy(hs->Bbar.begin(), hs->Bbar.end(), Ks.begin());
+  std::copy(hs->L.begin(), hs->L.end(), Ks.begin() + (size_t)n_x * n_v);
+  f->sp_nnz = 0;
+  for (double v : Ks) f->sp_nnz += v != 0.0;
+  if (f->sp_nnz > kSparseMax) return SMPC_OK;
+  const int np = f->shared_packs ? 1 : f->n;
+  const double* prob = f->shared_packs ? nullptr : tree->dev.prob;
+  const size_t entries = (size_t)np * lam_pack_entries(n_v);
+  const std::vector<unsigned char> image = sparse_image(f->prec, n_k, n_v, Ks.data());
+  TRY(f->alloc(&f->sp, image.size()));
+  CK(cudaMemcpy(f->sp, image.data(), image.size(), cudaMemcpyHostToDevice));
+  TRY(f->alloc(&f->lam, entries * f->ms));
+  TRY(launch_lam_pack(f->prec, np, n_v, f->Lam64, prob, f->lam, nullptr));
+  if (b16) {
+    double* Lam = nullptr;
+    TRY(f->alloc(&f->lam32, entries * sizeof(float)));
+    TRY(upload64(f, &Lam, red.Lam.data(), red.Lam.size()));
+    TRY(upload64(f, &f->Rhat_red, red.Rhat.data(), red.Rhat.size()));
+    TRY(upload64(f, &f->L_red, red.L.data(), red.L.size()));
+    TRY(upload_csr(f, &f->rhat_t_red, n_v, n_u, [&](int i, int j) { return red.Rhat[(size_t)j * n_v + i]; }));
+    TRY(launch_lam_pack(SMPC_FP32, np, n_v, Lam, prob, f->lam32, nullptr));
+  }
+  CK(cudaDeviceSynchronize());
+  return SMPC_OK;
+}
+
+// Gives back what build_two_launch allocated: everything behind the first `mark` allocations.
+void drop_two_launch(smpc_factor_t* f, size_t mark, size_t bytes) {
+  for (; f->allocs.size() > mark; f->allocs.pop_back()) cudaFree(f->allocs.back());
+  f->device_bytes = bytes;
+  f->sp = f->lam = f->lam32 = nullptr;
+  f->Rhat_red = f->L_red = nullptr;
+  f->rhat_t_red = CsrRows();
+}
+
 }  // namespace
 
 namespace smpc {
@@ -982,46 +1069,18 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
     for (int j = 0; j < n_v; ++j) K[(size_t)i * n_v + j] = f->hf.Bbar[(size_t)i * n_v + j];
   for (int i = 0; i < n_u; ++i)
     for (int j = 0; j < n_v; ++j) K[(size_t)(n_x + i) * n_v + j] = f->hf.L[(size_t)i * n_v + j];
-  auto up64 = [&](double** dst, const double* src, size_t cnt) -> int {
-    TRY(f->alloc(dst, cnt * sizeof(double)));
-    if (cnt) CK(cudaMemcpy(*dst, src, cnt * sizeof(double), cudaMemcpyHostToDevice));
-    return SMPC_OK;
-  };
-  if ((rc = up64(&f->K64, K.data(), K.size())) || (rc = up64(&f->Lam64, f->hf.Lam.data(), f->hf.Lam.size())) ||
-      (rc = up64(&f->Rhat, f->hf.Rhat.data(), f->hf.Rhat.size())) || (rc = up64(&f->L, f->hf.L.data(), f->hf.L.size())) ||
-      (rc = up64(&f->alpha1, cost->alpha1, n_u)))
+  if ((rc = upload64(f, &f->K64, K.data(), K.size())) || (rc = upload64(f, &f->Lam64, f->hf.Lam.data(), f->hf.Lam.size())) ||
+      (rc = upload64(f, &f->Rhat, f->hf.Rhat.data(), f->hf.Rhat.size())) || (rc = upload64(f, &f->L, f->hf.L.data(), f->hf.L.size())) ||
+      (rc = upload64(f, &f->alpha1, cost->alpha1, n_u)))
     return fail(rc);
-  auto up_csr = [&](CsrRows* out, int rows, int cols, auto&& at) -> int {
-    std::vector<int> ptr(1, 0), col;
-    std::vector<double> val;
-    for (int i = 0; i < rows; ++i) {
-      for (int j = 0; j < cols; ++j)
-        if (at(i, j) != 0.0) {
-          col.push_back(j);
-          val.push_back(at(i, j));
-        }
-      ptr.push_back((int)col.size());
-    }
-    int *dp = nullptr, *dc = nullptr;
-    double* dv = nullptr;
-    TRY(f->alloc(&dp, ptr.size() * sizeof(int)));
-    TRY(f->alloc(&dc, col.size() * sizeof(int)));
-    TRY(up64(&dv, val.data(), val.size()));
-    CK(cudaMemcpy(dp, ptr.data(), ptr.size() * sizeof(int), cudaMemcpyHostToDevice));
-    if (!col.empty()) CK(cudaMemcpy(dc, col.data(), col.size() * sizeof(int), cudaMemcpyHostToDevice));
-    out->ptr = dp;
-    out->col = dc;
-    out->val = dv;
-    return SMPC_OK;
-  };
   size_t rhat_nnz = 0;
   for (double v : f->hf.Rhat) rhat_nnz += v != 0.0;
-  if ((rc = up_csr(&f->pue, n_u + n_x, n_d, [&](int i, int j) {
+  if ((rc = upload_csr(f, &f->pue, n_u + n_x, n_d, [&](int i, int j) {
          return i < n_u ? f->hf.Pu[(size_t)i * n_d + j] : f->hf.Pe[(size_t)(i - n_u) * n_d + j];
        })) ||
       // a dense Rhat (the orthonormal basis, coupled input weights) is read by coalesced columns
       (4 * rhat_nnz <= f->hf.Rhat.size() &&
-       (rc = up_csr(&f->rhat_t, n_v, n_u, [&](int i, int j) { return f->hf.Rhat[(size_t)j * n_v + i]; }))))
+       (rc = upload_csr(f, &f->rhat_t, n_v, n_u, [&](int i, int j) { return f->hf.Rhat[(size_t)j * n_v + i]; }))))
     return fail(rc);
   // ---- packs: one per node, or one shared pack (Lambda unscaled) and the node scales
   f->shared_packs = o.shared_packs != 0;
@@ -1045,46 +1104,6 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
     const size_t hb = sizeof(float) * (size_t)n * n_k;
     if ((rc = f->alloc(&f->ha, hb)) || (rc = f->alloc(&f->wa, hb))) return fail(rc);
     if (cudaMemset(f->ha, 0, hb) != cudaSuccess || cudaMemset(f->wa, 0, hb) != cudaSuccess) return fail(SMPC_ECUDA);
-  }
-  // ---- the two-launch form of schedule 4 (with a general A: of schedule 2): only a factor
-  // that may choose its schedule.  A bfloat16 factor's anchors run it in float32 in the reduced
-  // basis, its delta launches on the packs' own [Bbar; L] and Lambda; with one pack for all
-  // nodes those round vectors to bfloat16 for the tensor cores, in an order that the two-launch
-  // form does not keep. Deep trees (kB16Stages) keep schedules 1 to 4 as well.
-  const size_t lam_bytes = (size_t)np * lam_pack_entries(n_v) * f->ms, lam32_bytes = (size_t)np * lam_pack_entries(n_v) * 4;
-  const bool b16 = f->prec == SMPC_BF16;
-  if (o.schedule == 0 && f->form != FORM_SEPARATE && !tree->top_src_off.empty() && !(b16 && (f->shared_packs || general_A || tree->N > kB16Stages))) {
-    HostFactor red;
-    const HostFactor* hs = &f->hf;
-    if (b16) {
-      if ((rc = host_factor(*net, cost->W_u, red, true)) != SMPC_OK) return fail(rc);
-      hs = &red;
-    }
-    std::vector<double> Ks((size_t)n_k * n_v);
-    std::copy(hs->Bbar.begin(), hs->Bbar.end(), Ks.begin());
-    std::copy(hs->L.begin(), hs->L.end(), Ks.begin() + (size_t)n_x * n_v);
-    for (double v : Ks) f->sp_nnz += v != 0.0;
-    if (f->sp_nnz <= kSparseMax) {
-      const std::vector<unsigned char> image = sparse_image(f->prec, n_k, n_v, Ks.data());
-      if ((rc = f->alloc(&f->sp, image.size()))) return fail(rc);
-      if (cudaMemcpy(f->sp, image.data(), image.size(), cudaMemcpyHostToDevice) != cudaSuccess) return fail(SMPC_ECUDA);
-      // without room for the matrices the other schedules run as before
-      if (f->alloc(&f->lam, lam_bytes) == SMPC_OK) {
-        if ((rc = launch_lam_pack(f->prec, np, n_v, f->Lam64, pprob, f->lam, nullptr))) return fail(rc);
-        if (b16 && f->alloc(&f->lam32, lam32_bytes) == SMPC_OK) {
-          double* Lam = nullptr;
-          if ((rc = up64(&Lam, red.Lam.data(), red.Lam.size())) || (rc = up64(&f->Rhat_red, red.Rhat.data(), red.Rhat.size())) ||
-              (rc = up64(&f->L_red, red.L.data(), red.L.size())) ||
-              (rc = up_csr(&f->rhat_t_red, n_v, n_u, [&](int i, int j) { return red.Rhat[(size_t)j * n_v + i]; })) ||
-              (rc = launch_lam_pack(SMPC_FP32, np, n_v, Lam, pprob, f->lam32, nullptr)))
-            return fail(rc);
-        }
-        if (b16 && !f->lam32) {
-          f->release(f->lam, lam_bytes);
-          f->lam = nullptr;
-        }
-      }
-    }
   }
   // ---- vectors
   const size_t vs = f->vs;
@@ -1234,13 +1253,14 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
     set_error("factor: %s", cudaGetErrorString(cudaGetLastError()));
     return fail(SMPC_ECUDA);
   }
+  // last of the allocations: where it finds no room the other schedules run as without it
+  const size_t mark = f->allocs.size(), mark_bytes = f->device_bytes;
+  if (o.schedule == 0) rc = build_two_launch(f, *net, cost->W_u);
+  if (rc != SMPC_OK && rc != SMPC_ENOMEM) return fail(rc);
+  if (rc == SMPC_ENOMEM) drop_two_launch(f, mark, mark_bytes);
   if ((rc = choose_schedule(f, o.schedule))) return fail(rc);
   if ((rc = tune_tc(f, o.tc_width))) return fail(rc);
-  if (f->lam && f->schedule != SCHED_SWEEP) {  // not chosen: its matrices go
-    f->release(f->lam, lam_bytes);
-    f->release(f->lam32, lam32_bytes);
-    f->lam = f->lam32 = nullptr;
-  }
+  if (f->schedule != SCHED_SWEEP) drop_two_launch(f, mark, mark_bytes);
   *out = f;
   return SMPC_OK;
 }

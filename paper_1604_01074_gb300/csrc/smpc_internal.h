@@ -426,15 +426,6 @@ struct smpc_factor_t {
     graphs.clear();
   }
 
-  void release(void* p, size_t bytes) {
-    for (size_t i = 0; i < allocs.size(); ++i)
-      if (allocs[i] == p) {
-        cudaFree(p);
-        allocs.erase(allocs.begin() + (long)i);
-        device_bytes -= bytes;
-        return;
-      }
-  }
   template <typename T>
   int alloc(T** p, size_t bytes) {
     *p = nullptr;
