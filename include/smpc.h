@@ -122,7 +122,7 @@ typedef struct smpc_factor_opts {
    * pass up to r, and the node-parallel Lambda / [Bbar; L] launch; 4 = node-parallel forward
    * sweep and prox, then the whole backward sweep as one chain pass (every pack read once
    * per iteration); 0 = time all of them on this GPU when the factor is built and keep the
-   * fastest.  Where [Bbar; L] is sparse (at most 4096 entries in the reduced basis,
+   * fastest.  Where [Bbar; L] is sparse (at most 4096 entries in a well conditioned reduced basis,
    * float64, float32, or SMPC_BF16 with a pack per node and at most 18 stages) 0 also times a
    * two-launch form of 4 - a tree pass with the sparse products inside, and Lambda r of every
    * node - which is reported as 4 (with a general A, as 2).  Results agree to rounding.
@@ -224,9 +224,9 @@ int smpc_tree_info_get(const smpc_tree* tree, smpc_tree_info* info);
 void smpc_tree_destroy(smpc_tree* tree);
 
 /* Offline factor step (App. A and App. B; Alg. 2 lines 1-2), in float64 on the
- * host: L = basis of null(E) (orthonormal; in float64 and float32 factors the reduced one
- * [-E1^{-1} E2; I] where its entries stay within 4, since it keeps a network's incidence
- * structure; u, x and y do not depend on the basis), B_bar = B L, R_hat = W_u L,
+ * host: L = orthonormal basis of null(E) (the two-launch form: the reduced basis
+ * [-E1^{-1} E2; I], which keeps a network's incidence structure, where cond(L'L) <= 40; u, x
+ * and y do not depend on the basis), B_bar = B L, R_hat = W_u L,
  * R_bar = L' R_hat, Cholesky of R_bar, Lambda = -R_bar^{-1}; then per-node packs
  * [B_bar; L] (n_x + n_u) x n_v and Lambda / (2 p_n) (n_v x n_v, Alg. 1's
  * node-indexed factor matrices) in the requested precision on the device, the

@@ -312,8 +312,8 @@ void set_sweep_args(const smpc_factor_t* f, IterArgs& a) {
   a.top_src = t->dev.top_src;
   a.chain_kids = t->dev.chain_kids;
 }
-void set_basis(const smpc_factor_t* f, CostArgs& c) {
-  const bool red = f->schedule == SCHED_SWEEP && f->prec == SMPC_BF16;  // beta enters in the anchors only
+void set_basis(const smpc_factor_t* f, bool shard, CostArgs& c) {
+  const bool red = f->schedule == SCHED_SWEEP && !shard;  // bfloat16 factors: beta enters in the anchors only
   c.rhat_t = red ? f->rhat_t_red : f->rhat_t;
   c.Rhat = red ? f->Rhat_red : f->Rhat;
   c.L = red ? f->L_red : f->L;
@@ -568,28 +568,34 @@ int upload_csr(smpc_factor_t* f, CsrRows* out, int rows, int cols, F&& at) {
   return SMPC_OK;
 }
 
+// Rhat' by its nonzero entries; a dense Rhat (the orthonormal basis, coupled input weights) is
+// read by coalesced columns instead.
+int upload_rhat_t(smpc_factor_t* f, CsrRows* out, const HostFactor& h) {
+  size_t nnz = 0;
+  for (double v : h.Rhat) nnz += v != 0.0;
+  if (4 * nnz > h.Rhat.size()) return SMPC_OK;
+  return upload_csr(f, out, h.n_v, h.n_u, [&](int i, int j) { return h.Rhat[(size_t)j * h.n_v + i]; });
+}
+
 // The matrices of the two-launch form of schedule 4 (with a general A: of schedule 2), for a
-// factor that may choose its schedule; f->lam stays NULL where the form does not apply.  A
-// bfloat16 factor's anchors run it in float32 in the reduced basis, its delta launches on the
-// packs' own [Bbar; L] and Lambda; with one pack for all nodes those round vectors to bfloat16
-// for the tensor cores, in an order that the two-launch form does not keep.  Deep trees
+// factor that may choose its schedule; f->lam stays NULL where the form does not apply.  They
+// are those of the reduced basis, in which a network's [Bbar; L] is sparse; the packs keep the
+// orthonormal one.  A bfloat16 factor runs its anchors in them in float32, its delta launches on
+// the packs' own [Bbar; L] and Lambda; with one pack for all nodes those round vectors to
+// bfloat16 for the tensor cores, in an order that the two-launch form does not keep.  Deep trees
 // (kB16Stages) keep schedules 1 to 4 as well.
 int build_two_launch(smpc_factor_t* f, const smpc_network& net, const double* W_u) {
   const smpc_tree* tree = f->tree;
-  const int n_x = f->n_x, n_u = f->n_u, n_v = f->n_v, n_k = f->n_k;
+  const int n_x = f->n_x, n_v = f->n_v, n_k = f->n_k;
   const bool b16 = f->prec == SMPC_BF16;
   if (f->form == FORM_SEPARATE || tree->top_src_off.empty() ||
       (b16 && (f->shared_packs || f->A || tree->N > kB16Stages)))
     return SMPC_OK;
   HostFactor red;
-  const HostFactor* hs = &f->hf;
-  if (b16) {
-    TRY(host_factor(net, W_u, red, true));
-    hs = &red;
-  }
+  if (host_factor(net, W_u, red, true) != SMPC_OK) return SMPC_OK;
   std::vector<double> Ks((size_t)n_k * n_v);
-  std::copy(hs->Bbar.begin(), hs->Bbar.end(), Ks.begin());
-  std::copy(hs->L.begin(), hs->L.end(), Ks.begin() + (size_t)n_x * n_v);
+  std::copy(red.Bbar.begin(), red.Bbar.end(), Ks.begin());
+  std::copy(red.L.begin(), red.L.end(), Ks.begin() + (size_t)n_x * n_v);
   f->sp_nnz = 0;
   for (double v : Ks) f->sp_nnz += v != 0.0;
   if (f->sp_nnz > kSparseMax) return SMPC_OK;
@@ -599,18 +605,20 @@ int build_two_launch(smpc_factor_t* f, const smpc_network& net, const double* W_
   const std::vector<unsigned char> image = sparse_image(f->prec, n_k, n_v, Ks.data());
   TRY(f->alloc(&f->sp, image.size()));
   CK(cudaMemcpy(f->sp, image.data(), image.size(), cudaMemcpyHostToDevice));
-  TRY(f->alloc(&f->lam, entries * f->ms));
-  TRY(launch_lam_pack(f->prec, np, n_v, f->Lam64, prob, f->lam, nullptr));
+  double* Lam = nullptr;
+  TRY(upload64(f, &Lam, red.Lam.data(), red.Lam.size()));
+  TRY(upload64(f, &f->Rhat_red, red.Rhat.data(), red.Rhat.size()));
+  TRY(upload64(f, &f->L_red, red.L.data(), red.L.size()));
+  TRY(upload_rhat_t(f, &f->rhat_t_red, red));
+  void* lam = nullptr;
+  TRY(f->alloc(&lam, entries * f->ms));
+  TRY(launch_lam_pack(f->prec, np, n_v, b16 ? f->Lam64 : Lam, prob, lam, nullptr));
   if (b16) {
-    double* Lam = nullptr;
     TRY(f->alloc(&f->lam32, entries * sizeof(float)));
-    TRY(upload64(f, &Lam, red.Lam.data(), red.Lam.size()));
-    TRY(upload64(f, &f->Rhat_red, red.Rhat.data(), red.Rhat.size()));
-    TRY(upload64(f, &f->L_red, red.L.data(), red.L.size()));
-    TRY(upload_csr(f, &f->rhat_t_red, n_v, n_u, [&](int i, int j) { return red.Rhat[(size_t)j * n_v + i]; }));
     TRY(launch_lam_pack(SMPC_FP32, np, n_v, Lam, prob, f->lam32, nullptr));
   }
   CK(cudaDeviceSynchronize());
+  f->lam = lam;
   return SMPC_OK;
 }
 
@@ -1033,9 +1041,7 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   f->n_u = n_u;
   f->n_d = n_d;
   f->n_e = n_e;
-  // A bfloat16 factor keeps the orthonormal basis: its entries are rounded to 8 bits, and the
-  // orthonormal one has no large entries to round.
-  int rc = host_factor(*net, cost->W_u, f->hf, f->prec != SMPC_BF16);
+  int rc = host_factor(*net, cost->W_u, f->hf, false);
   if (rc != SMPC_OK) return fail(rc);
   const int n_v = f->hf.n_v;
   f->n_v = n_v;
@@ -1073,14 +1079,10 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
       (rc = upload64(f, &f->Rhat, f->hf.Rhat.data(), f->hf.Rhat.size())) || (rc = upload64(f, &f->L, f->hf.L.data(), f->hf.L.size())) ||
       (rc = upload64(f, &f->alpha1, cost->alpha1, n_u)))
     return fail(rc);
-  size_t rhat_nnz = 0;
-  for (double v : f->hf.Rhat) rhat_nnz += v != 0.0;
   if ((rc = upload_csr(f, &f->pue, n_u + n_x, n_d, [&](int i, int j) {
          return i < n_u ? f->hf.Pu[(size_t)i * n_d + j] : f->hf.Pe[(size_t)(i - n_u) * n_d + j];
        })) ||
-      // a dense Rhat (the orthonormal basis, coupled input weights) is read by coalesced columns
-      (4 * rhat_nnz <= f->hf.Rhat.size() &&
-       (rc = upload_csr(f, &f->rhat_t, n_v, n_u, [&](int i, int j) { return f->hf.Rhat[(size_t)j * n_v + i]; }))))
+      (rc = upload_rhat_t(f, &f->rhat_t, f->hf)))
     return fail(rc);
   // ---- packs: one per node, or one shared pack (Lambda unscaled) and the node scales
   f->shared_packs = o.shared_packs != 0;
@@ -1315,7 +1317,7 @@ namespace smpc {
 // loop): checks, the launch plan, the step-data upload, the cost update of App. A, the
 // initial duals and the per-solve flags, all enqueued on s.
 int solve_begin(smpc_factor_t* f, const smpc_step_data* data, const smpc_solve_opts* opts, cudaStream_t s,
-                IterPlan* plan_out, IterArgs* args_out) {
+                IterPlan* plan_out, IterArgs* args_out, bool shard) {
   if (!f || !data || !opts) {
     set_error("NULL argument");
     return SMPC_EINVAL;
@@ -1374,7 +1376,7 @@ int solve_begin(smpc_factor_t* f, const smpc_step_data* data, const smpc_solve_o
   c.prob = f->tree->dev.prob;
   c.pbar = f->tree->dev.pbar;
   c.pue = f->pue;
-  set_basis(f, c);
+  set_basis(f, shard, c);
   c.alpha1 = f->alpha1;
   c.W_alpha = f->W_alpha;
   c.dhat = f->d_dhat;

@@ -95,12 +95,45 @@ void householder_q(std::vector<double> M, int rows, int cols, std::vector<double
   }
 }
 
+// Largest condition number of L'L at which the reduced basis is taken (reduced_null_basis).
+// Errors of the two-launch form against 64 bits, relative to those of schedules 1 to 4 in the
+// orthonormal basis (float32, u and x, 40 iterations, means of three seeds on 48 network shapes
+// of 10 to 90 inputs): 0.5 to 1.25 up to 40; from there on networks whose junctions share many
+// inputs lose (dense E 1.3 at 44, entries all near 1: 3.6 at 77, 5.6 at 230, 9.4 at 520).  The
+// networks of 4 to 63 tanks with a junction per six inputs or so have 2 to 15, those with forty
+// inputs to each junction 24 to 37.
+constexpr double kMaxCond = 40;
+
+// Largest eigenvalue of F F' (F n_e x n_f, row-major) by power iteration.
+double spectral_square(const std::vector<double>& F, int n_e, int n_f) {
+  std::vector<double> x(n_e), y(n_f);
+  for (int i = 0; i < n_e; ++i) x[i] = 1.0 + 0.37 * ((i * 7919) % 101) / 101.0;
+  double top = 0;
+  for (int it = 0; it < 100; ++it) {
+    double nrm = 0;
+    for (int i = 0; i < n_e; ++i) nrm += x[i] * x[i];
+    nrm = std::sqrt(nrm);
+    if (!(nrm > 0)) return top;
+    for (int i = 0; i < n_e; ++i) x[i] /= nrm;
+    top = 0;
+    for (int j = 0; j < n_f; ++j) {
+      y[j] = 0;
+      for (int i = 0; i < n_e; ++i) y[j] += F[(size_t)i * n_f + j] * x[i];
+      top += y[j] * y[j];
+    }
+    for (int i = 0; i < n_e; ++i) {
+      x[i] = 0;
+      for (int j = 0; j < n_f; ++j) x[i] += F[(size_t)i * n_f + j] * y[j];
+    }
+  }
+  return top;
+}
+
 // A basis of null(E) in reduced form: with E column-permuted to [E1 E2], E1 square, the rows
-// of the basis are those of -E1^{-1} E2 for E1's columns and unit rows for the others.  For an
-// incidence matrix it is sparse (a junction's balance solved for one of its actuators), and so
-// is B L.  Gauss-Jordan elimination with complete pivoting, ties towards the column with the
-// fewest entries.  False (L untouched) when an entry of -E1^{-1} E2 exceeds 4: the basis could
-// then be worse conditioned than the orthonormal one by more than rounding forgives.
+// of the basis are those of F = -E1^{-1} E2 for E1's columns and unit rows for the others.  For
+// an incidence matrix it is sparse (a junction's balance solved for one of its actuators), and
+// so is B L.  Gauss-Jordan elimination with complete pivoting, ties towards the column with the
+// fewest entries.  False (L untouched) when cond(L'L) = 1 + ||F||^2 exceeds kMaxCond.
 bool reduced_null_basis(const double* E, int n_e, int n_u, std::vector<double>& L) {
   std::vector<double> M(E, E + (size_t)n_e * n_u);
   std::vector<int> piv(n_e, -1), used(n_u, 0), count(n_u, 0);
@@ -134,17 +167,20 @@ bool reduced_null_basis(const double* E, int n_e, int n_u, std::vector<double>& 
     }
   }
   const int n_v = n_u - n_e;
-  std::vector<double> B((size_t)n_u * n_v, 0.0);
+  std::vector<double> B((size_t)n_u * n_v, 0.0), F((size_t)n_e * n_v, 0.0);
   for (int j = 0, k = 0; j < n_u; ++j) {
     if (used[j]) continue;
     B[(size_t)j * n_v + k] = 1.0;
     for (int i = 0; i < n_e; ++i) {
       const double v = M[(size_t)i * n_u + j];
-      if (!(std::fabs(v) <= 4.0)) return false;
-      if (std::fabs(v) > 1e-15) B[(size_t)piv[i] * n_v + k] = -v;  // cancellations leave some 1e-16
+      if (std::fabs(v) > 1e-15) {  // cancellations leave some 1e-16
+        B[(size_t)piv[i] * n_v + k] = -v;
+        F[(size_t)i * n_v + k] = -v;
+      }
     }
     ++k;
   }
+  if (!(1.0 + spectral_square(F, n_e, n_v) <= kMaxCond)) return false;
   L = B;
   return true;
 }
@@ -181,7 +217,7 @@ int host_factor(const smpc_network& net, const double* W_u, HostFactor& f, bool 
     f.L.assign((size_t)n_u * f.n_v, 0.0);
     for (int i = 0; i < n_u; ++i)
       for (int j = 0; j < f.n_v; ++j) f.L[i * f.n_v + j] = Q[i * n_u + n_e + j];
-    if (reduced_basis) reduced_null_basis(net.E, n_e, n_u, f.L);
+    if (reduced_basis && !reduced_null_basis(net.E, n_e, n_u, f.L)) return SMPC_ENOTSUP;
     // Pu = -E' (E E')^{-1} Ed  (minimum-norm particular solution of E u + Ed d = 0)
     std::vector<double> EEt((size_t)n_e * n_e);
     for (int i = 0; i < n_e; ++i)

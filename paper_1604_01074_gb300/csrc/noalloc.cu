@@ -286,7 +286,7 @@ extern "C" int smpc_solve_static(smpc_factor_t* f, const smpc_step_data* data, c
   c.prob = f->tree->dev.prob;
   c.pbar = f->tree->dev.pbar;
   c.pue = f->pue;
-  set_basis(f, c);
+  set_basis(f, false, c);
   c.alpha1 = f->alpha1;
   c.W_alpha = f->W_alpha;
   c.dhat = f->d_dhat;

@@ -198,7 +198,7 @@ int smpc_shard_begin(smpc_shard* sh, const smpc_step_data* data, const smpc_solv
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   IterPlan plan;
   IterArgs a;
-  SHTRY(solve_begin(f, data, opts, s, &plan, &a));
+  SHTRY(solve_begin(f, data, opts, s, &plan, &a, true));
   const smpc_tree* t = f->tree;
   sh->iters = opts->max_iters;
   sh->s = s;

@@ -32,7 +32,8 @@ struct HostFactor {
   std::vector<double> diagL;  // n_u, diag(L Rbar^{-1} L')
 };
 // Returns SMPC_OK or SMPC_EINVAL (rank-deficient E, W_u not positive definite).
-// reduced_basis: L in reduced form where that basis is well conditioned (factor_host.cpp).
+// reduced_basis: L in reduced form (factor_host.cpp), SMPC_ENOTSUP where that is not well
+// conditioned; else orthonormal.
 int host_factor(const smpc_network& net, const double* W_u, HostFactor& out, bool reduced_basis);
 
 // ---------------------------------------------------------------------------
@@ -331,9 +332,10 @@ namespace smpc {
 // The parts of smpc_solve around its iteration chunks (api.cpp), shared with the batch
 // solve (batch.cpp): solve_begin checks the call, plans the launches and enqueues the
 // step-data upload, the cost update, the initial duals and the per-solve flags;
-// solve_end enqueues the tail launch, the final dual and the outputs.
+// solve_end enqueues the tail launch, the final dual and the outputs.  shard: the iterations
+// will run on the factor's packs, whatever its own schedule.
 int solve_begin(smpc_factor_t* f, const smpc_step_data* data, const smpc_solve_opts* opts, cudaStream_t s,
-                IterPlan* plan, IterArgs* args);
+                IterPlan* plan, IterArgs* args, bool shard = false);
 int solve_end(smpc_factor_t* f, IterPlan& plan, const IterArgs& a, int launched, smpc_result* res, cudaStream_t s);
 // Validates polish_iters and the kernel configuration; SMPC_ENOTSUP when the network
 // does not fit the shared-memory pipeline.
@@ -341,8 +343,9 @@ int plan_iters(const smpc_factor_t* f, const IterArgs& a, const smpc_solve_opts&
 int launch_planned(IterPlan& plan, int nu, int mode, void* stream);
 // The SCHED_SWEEP fields of a.
 void set_sweep_args(const smpc_factor_t* f, IterArgs& a);
-// The basis of beta: c.L, c.Rhat, c.rhat_t.
-void set_basis(const smpc_factor_t* f, CostArgs& c);
+// The basis of beta (c.L, c.Rhat, c.rhat_t): the reduced one for the two-launch form, the
+// orthonormal one of the packs for the other schedules and for shards.
+void set_basis(const smpc_factor_t* f, bool shard, CostArgs& c);
 // Copies the final dual of the factor's last solve (vector type) to dst; synchronous.
 int copy_final_y(smpc_factor_t* f, void* dst);
 }  // namespace smpc
@@ -397,9 +400,10 @@ struct smpc_factor_t {
   int schedule = smpc::SCHED_CHAIN;  // iteration schedule in use
   int form = smpc::FORM_TIMED;
   void *sp = nullptr, *lam = nullptr;  // SCHED_SWEEP: sparse [Bbar; L], packed Lambda
-  // ... of a bfloat16 factor: the anchors' float32 Lambda and cost-update matrices, in the
-  // reduced basis (lam: bfloat16, in the basis of the packs)
+  // ... of a bfloat16 factor: the anchors' float32 Lambda, in the reduced basis (lam: bfloat16,
+  // in the orthonormal basis of the packs)
   void* lam32 = nullptr;
+  // ... the cost update's matrices in the reduced basis
   double *Rhat_red = nullptr, *L_red = nullptr;
   smpc::CsrRows rhat_t_red;
   int sp_nnz = 0;
