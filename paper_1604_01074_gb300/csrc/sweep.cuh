@@ -138,24 +138,7 @@ struct MaxAbs<double> {
   __device__ double value() const { return __longlong_as_double((long long)b); }
 };
 
-// Extrapolation and signs of the tree pass: in float64 the extrapolation is one fused
-// multiply-add on the difference, and signs are read from the bits.  In float32 the difference
-// and the product stay unnormalised pairs (their low parts are still below an ulp of the high
-// ones), which saves six of st_extrap's 28 operations; only the sum is renormalised.
-__device__ __forceinline__ DS sw_extrap(DS y1, DS y2, float c) {
-  const DS d = two_sum(y1.hi, -y2.hi);
-  const float dl = __fadd_rn(d.lo, __fsub_rn(y1.lo, y2.lo));
-  const float p = __fmul_rn(d.hi, c);
-  const float pe = __fmaf_rn(dl, c, __fmaf_rn(d.hi, c, -p));
-  const DS t = two_sum(y1.hi, p);
-  return fast_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(y1.lo, pe)));
-}
-// a - b rounded to the vector type
-__device__ __forceinline__ float sw_diff(DS a, DS b) {
-  return __fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo));
-}
-__device__ __forceinline__ double sw_diff(double a, double b) { return a - b; }
-__device__ __forceinline__ double sw_extrap(double y1, double y2, double c) { return fma(c, y1 - y2, y1); }
+// Signs of the tree pass: in float64 read from the bits, off the float64 pipe.
 __device__ __forceinline__ bool sw_neg(DS x) { return x.hi < 0.f; }
 __device__ __forceinline__ bool sw_neg(double x) { return __double_as_longlong(x) < 0; }
 __device__ __forceinline__ bool sw_pos(DS x) { return x.hi > 0.f; }
@@ -176,15 +159,9 @@ struct SweepOut {
 // Anchored solves (bfloat16 packs, B16): a delta launch takes w - w_a, exactly in the state
 // type; an anchor stores w_a = w; the launch after an anchor stores x and u, from which those
 // up to the next anchor continue with the linear part.
-// FORM 2 (the tensor-core path) keeps every operation of warp_prox_staged: its vectors are
-// rounded to bfloat16 further on, where a last bit more or less turns into 2^-9.
-template <int FORM, typename ST, typename AT>
-__device__ __forceinline__ ST form_extrap(ST y1, ST y2, AT c) {
-  if constexpr (FORM == 2)
-    return st_extrap(y1, y2, c);
-  else
-    return sw_extrap(y1, y2, c);
-}
+// All forms keep every operation of warp_prox_staged on the duals (the unnormalised float32
+// extrapolation tried here had 1.4 times its mean error): in FORM 2 (the tensor-core path) the
+// vectors are rounded to bfloat16 further on, where a last bit more or less turns into 2^-9.
 template <typename VT, int NT, int FORM>
 __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, const VT* bnd, int it, VT c, VT cn, int mode,
                                             SweepOut<VT>& o) {
@@ -227,8 +204,8 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
     qs[k] = qz[k] = zero;
     if (e < n_x) {
       const VT x = z[e];
-      ws[k] = form_extrap<FORM>(v1[k], ws[k], c);
-      wz[k] = form_extrap<FORM>(w1[k], wz[k], c);
+      ws[k] = st_extrap(v1[k], ws[k], c);
+      wz[k] = st_extrap(w1[k], wz[k], c);
       const ST q = st_axpy(ws[k], ls, x - xs[e]);
       qs[k] = sw_neg(q) ? q : zero;  // C = {x >= x_s}
       qz[k] = sw_box(st_axpy(wz[k], lz, x - xhi[e]), st_axpy(wz[k], lz, x - xlo[e]));
@@ -258,7 +235,7 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
     if (e < n_x) {
       const VT x = z[e];
       const ST ysn = st_scale(qs[k], ks), yzn = st_scale(qz[k], kz);
-      const VT es = sw_diff(ysn, ws[k]) * is, ez = sw_diff(yzn, wz[k]) * iz;
+      const VT es = st_val(st_sub(ysn, ws[k])) * is, ez = st_val(st_sub(yzn, wz[k])) * iz;
       st_state(y2 + e, ysn);
       st_state(y2 + n_x + e, yzn);
       xo[e] = x;
@@ -315,9 +292,9 @@ __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, V
     const int i = i0 + lane + 32 * k;
     if (i < n_u) {
       const VT u = z[n_x + i];
-      const ST wp = form_extrap<FORM>(p1[k], p2[k], c);
+      const ST wp = st_extrap(p1[k], p2[k], c);
       const ST ypn = sw_box(st_axpy(wp, lp[k], u - uhi[i]), st_axpy(wp, lp[k], u - ulo[i]));
-      const VT ep = sw_diff(ypn, wp) * ip[k];
+      const VT ep = st_val(st_sub(ypn, wp)) * ip[k];
       st_state(y2 + i, ypn);
       reinterpret_cast<VT*>(a.uout)[mu + i] = u;
       if (B16 && (mode & MODE_DELTA)) {
