@@ -306,6 +306,7 @@ void set_sweep_args(const smpc_factor_t* f, IterArgs& a) {
   a.kd = f->prec == SMPC_BF16 && f->form != FORM_SEPARATE ? f->packs : nullptr;
   a.depth = t->N;
   a.max_len = t->max_chain_len;
+  a.ha_lo = f->ha_lo;
   a.lam = f->lam;
   a.lam_stride = f->shared_packs ? 0 : lam_pack_entries(f->n_v);
   a.top_src_off = t->dev.top_src_off;
@@ -614,6 +615,7 @@ int build_two_launch(smpc_factor_t* f, const smpc_network& net, const double* W_
   TRY(f->alloc(&lam, entries * f->ms));
   TRY(launch_lam_pack(f->prec, np, n_v, b16 ? f->Lam64 : Lam, prob, lam, nullptr));
   if (b16) {
+    TRY(f->alloc(&f->ha_lo, sizeof(float) * (size_t)f->n * n_k));
     TRY(f->alloc(&f->lam32, entries * sizeof(float)));
     TRY(launch_lam_pack(SMPC_FP32, np, n_v, Lam, prob, f->lam32, nullptr));
   }
@@ -626,7 +628,7 @@ int build_two_launch(smpc_factor_t* f, const smpc_network& net, const double* W_
 void drop_two_launch(smpc_factor_t* f, size_t mark, size_t bytes) {
   for (; f->allocs.size() > mark; f->allocs.pop_back()) cudaFree(f->allocs.back());
   f->device_bytes = bytes;
-  f->sp = f->lam = f->lam32 = nullptr;
+  f->sp = f->lam = f->lam32 = f->ha_lo = nullptr;
   f->Rhat_red = f->L_red = nullptr;
   f->rhat_t_red = CsrRows();
 }

@@ -158,6 +158,7 @@ struct IterArgs {
   // as symmetric blocks (or one unscaled Lambda, lam_stride 0, with pscale), the largest tree
   // depth and chain length, and per top node its sources {node, weight}: the top nodes below and itself.
   const void* sp;
+  void* ha_lo;                   // bfloat16 factors: low parts of the anchor's x and u (in ha), n x n_k
   const void* kd;                // bfloat16 factors: the packs' [Bbar; L] (one node's), else NULL
   int sp_nnz, depth, max_len;
   const void* lam;
@@ -199,11 +200,15 @@ enum IterForm : int { FORM_TIMED = 0, FORM_TWO_LAUNCH, FORM_SEPARATE };
 // Entries of [Bbar; L] up to which it counts as sparse: its image is read into shared memory
 // by every CTA of the tree pass (64 KB at this size in float32).
 constexpr int kSparseMax = 4096;
-// Stages up to which a bfloat16 factor with a pack per node takes SCHED_SWEEP.  The delta
-// iterations enlarge rounding differences, the more so the deeper the tree: after 60 iterations
-// the largest difference of an entry of x to schedule 4 (relative to the root mean square) was
-// 4.6e-5 at 12 stages, 1.3e-4 at 18, and 3e-4 to 1.5e-3 at 24, on 1831 to 21 111 nodes, far
-// below the distance to float64 (1e-2) but beyond float32 agreement at 24.
+// Stages up to which a bfloat16 factor with a pack per node takes SCHED_SWEEP.  Its errors are
+// not the reason: the distance to float64 is the same as schedules 1 to 4's at 6 to 24 stages
+// (ratio 1.00), and so are the rounding errors (the distance to the same iteration in 64 bits).
+// But the delta iterations enlarge rounding differences, the more so the deeper the tree, also
+// those between schedules 1 and 4, and results of one factor should not move with the schedule by
+// more than float32 ones do (1e-4 of 1 + the largest entry).  Largest difference of an entry of x
+// to schedule 4 after 60 iterations, five seeds each of four trees of 4 to 400 scenarios on 20 to
+// 63 tanks: 5e-6 at 12 stages, 1.4e-5 at 15, 5.2e-5 at 18, 4.7e-5 at 19, 1.3e-4 at 20, 1.0e-4 at
+// 21, 1.4e-4 at 22, 1.5e-4 at 24.
 constexpr int kB16Stages = 18;
 
 struct LaunchCfg {
@@ -403,6 +408,7 @@ struct smpc_factor_t {
   // ... of a bfloat16 factor: the anchors' float32 Lambda, in the reduced basis (lam: bfloat16,
   // in the orthonormal basis of the packs)
   void* lam32 = nullptr;
+  void* ha_lo = nullptr;  // IterArgs::ha_lo
   // ... the cost update's matrices in the reduced basis
   double *Rhat_red = nullptr, *L_red = nullptr;
   smpc::CsrRows rhat_t_red;

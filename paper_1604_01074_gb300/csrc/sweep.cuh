@@ -157,8 +157,7 @@ struct SweepOut {
   MaxAbs<VT> r, h, t;  // residual maxima: |x - t|, |x|, |t| of the prox
 };
 // Anchored solves (bfloat16 packs, B16): a delta launch takes w - w_a, exactly in the state
-// type; an anchor stores w_a = w; the launch after an anchor stores x and u, from which those
-// up to the next anchor continue with the linear part.
+// type; an anchor stores w_a = w.
 // All forms keep every operation of warp_prox_staged on the duals (the unnormalised float32
 // extrapolation tried here had 1.4 times its mean error): in FORM 2 (the tensor-core path) the
 // vectors are rounded to bfloat16 further on, where a last bit more or less turns into 2^-9.
@@ -245,7 +244,6 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
         z[e] = st_extrap_val(ysn, v1[k], cn) + st_extrap_val(yzn, w1[k], cn);
         if (B16 && (mode & MODE_ANCHOR)) reinterpret_cast<VT*>(a.wa)[(long long)m * a.n_k + e] = z[e];
       }
-      if (B16 && (mode & MODE_AFTER_ANCHOR)) reinterpret_cast<VT*>(a.ha)[(long long)m * a.n_k + e] = x;
       if (a.xbar) {  // ergodic average (theta_0 = 1: the previous contents are not read then)
         VT* b = reinterpret_cast<VT*>(a.xbar) + (long long)m * n_x + e;
         const VT th = (VT)a.theta[it];
@@ -303,7 +301,6 @@ __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, V
         z[n_x + i] = st_extrap_val(ypn, p1[k], cn);
         if (B16 && (mode & MODE_ANCHOR)) reinterpret_cast<VT*>(a.wa)[mk + i] = z[n_x + i];
       }
-      if (B16 && (mode & MODE_AFTER_ANCHOR)) reinterpret_cast<VT*>(a.ha)[mk + i] = u;
       if (a.ubar) {
         VT* b = reinterpret_cast<VT*>(a.ubar) + mu + i;
         const VT th = (VT)a.theta[it];
@@ -536,6 +533,13 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
         for (int i = lane; i < n_u; i += 32) cp_async_elem(to + n_x + i, UH + m * n_u + i);
     }
   }
+  if (prox && fd)  // the anchor's x and u, read behind the path sums: towards the L2
+    for (int r = own + warp; r < L; r += NW)
+      for (int e = 32 * lane; e < n_k; e += 32 * 32) {
+        const long long at = (long long)sid[r] * n_k + e;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const VT*>(a.ha) + at));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const VT*>(a.ha_lo) + at));
+      }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (prox) {
     const VT* delta = reinterpret_cast<const VT*>(a.h);
@@ -547,10 +551,6 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
         }
     for (int r = H ? L : warp; r < L; r += NW)
       for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * xv + j, delta + (long long)sid[r] * n_v + j);
-    if (fd)  // the anchor's u (its x is added after the linear path sums)
-      for (int r = own + warp; r < L; r += NW)
-        for (int e = n_x + lane; e < n_k; e += 32)
-          cp_async_elem(Z + r * xk + e, reinterpret_cast<const VT*>(a.ha) + (long long)sid[r] * n_k + e);
   }
   const bool stop = early_exit(a, nu, mode, flag, true) || !tree_active(a, tree, nu);
   cp_async_wait_all();
@@ -574,40 +574,58 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
         }
       }
       __syncthreads();
-    } else {
-    if (tid < n_v)  // v along the path
-      run_sums<VT>(V, xv, tid, 0, 1, L, (VT)0, [&](int r, VT v) { V[r * xv + tid] = v; });
-    __syncthreads();
-    // x increments (Bbar v + e) and u; of path nodes only the tanks are used
-    if constexpr (B16) {
-      if (fd)
-        dense_fwd<NW>(Kd, kw, n_k, V, xv, 0, L, [&](int r, int e, VT v) {
-          if (e < n_x)
-            Z[r * xk + e] = v;
-          else if (r >= own)
-            Z[r * xk + e] += v;
-        });
-    }
-    if (!fd) sparse_rows<NW, VT>(
-        ek, rptr, rid, n_k, V, xv, 0, L, [&](int r, int e) -> VT { return Z[r * xk + e]; },
-        [&](int r, int e, VT v) { Z[r * xk + e] = v; });
-    __syncthreads();
-    if (a.A) {  // x_n = A x_parent + Bbar v_n + e_n (App. B), a barrier a node
-      if (tid < n_x) Z[L * xk + tid] = reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid];
-      for (int r = 0; r < L; ++r) {
-        __syncthreads();
-        add_Ax<NW>(As, n_x, false, Z + (r > 0 ? r - 1 : L) * xk, Z + r * xk);
+    } else if (B16 && !fd) {
+      // The base of the delta launches up to the next anchor, in two float32 throughout (ha,
+      // ha_lo): rounded to one, the same error would enter the duals in each of them.
+      if (tid < n_k) {
+        const int e = rid[tid], q0 = rptr[tid], q1 = rptr[tid + 1];
+        ST inc = st_from<ST>(0.0), x = to_sum<ST>(e < n_x ? reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + e] : (VT)0);
+        for (int r = 0; r < L; ++r) {
+          for (int q = q0; q < q1; ++q) st_fma_acc(inc, ek[q].v, V[r * xv + (int)ek[q].c]);
+          if (e >= n_x) x = to_sum<ST>((VT)0);  // u_n = L v_n + u_hat_n, x_n = x_parent + Bbar v_n + e_n
+          if (e < n_x || r >= own) add_sum(x, Z[r * xk + e]);
+          x = st_add(x, inc);
+          Z[r * xk + e] = st_val(x);
+          if (r >= own) {
+            reinterpret_cast<VT*>(a.ha)[(long long)sid[r] * n_k + e] = st_val(x);
+            reinterpret_cast<VT*>(a.ha_lo)[(long long)sid[r] * n_k + e] = st_val(st_sub(x, to_sum<ST>(st_val(x))));
+          }
+        }
       }
-    } else if (tid < n_x)  // x_n = x_parent + Bbar v_n + e_n
-      run_sums<VT>(Z, xk, tid, 0, 1, L, fd ? (VT)0 : reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid],
-               [&](int r, VT v) { Z[r * xk + tid] = v; });
-    __syncthreads();
-    if (fd) {
-      const VT* XA = reinterpret_cast<const VT*>(a.ha);
-      for (int r = own + warp; r < L; r += NW)
-        for (int e = lane; e < n_x; e += 32) Z[r * xk + e] += XA[(long long)sid[r] * n_k + e];
       __syncthreads();
-    }
+    } else {
+      if (tid < n_v)  // v along the path
+        run_sums<VT>(V, xv, tid, 0, 1, L, (VT)0, [&](int r, VT v) { V[r * xv + tid] = v; });
+      __syncthreads();
+      // x increments (Bbar v + e) and u; of path nodes only the tanks are used
+      if constexpr (B16)
+        dense_fwd<NW>(Kd, kw, n_k, V, xv, 0, L, [&](int r, int e, VT v) { Z[r * xk + e] = v; });
+      else
+        sparse_rows<NW, VT>(
+            ek, rptr, rid, n_k, V, xv, 0, L, [&](int r, int e) -> VT { return Z[r * xk + e]; },
+            [&](int r, int e, VT v) { Z[r * xk + e] = v; });
+      __syncthreads();
+      if (a.A) {  // x_n = A x_parent + Bbar v_n + e_n (App. B), a barrier a node
+        if (tid < n_x) Z[L * xk + tid] = reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid];
+        for (int r = 0; r < L; ++r) {
+          __syncthreads();
+          add_Ax<NW>(As, n_x, false, Z + (r > 0 ? r - 1 : L) * xk, Z + r * xk);
+        }
+      } else if (tid < n_x)  // x_n = x_parent + Bbar v_n + e_n
+        run_sums<VT>(Z, xk, tid, 0, 1, L, B16 ? (VT)0 : reinterpret_cast<const VT*>(a.p0)[(long long)tree * n_x + tid],
+                     [&](int r, VT v) { Z[r * xk + tid] = v; });
+      __syncthreads();
+      if (B16) {  // the linear part on the anchor's x and u
+        for (int r = own + warp; r < L; r += NW)
+          for (int e = lane; e < n_k; e += 32) {
+            const long long at = (long long)sid[r] * n_k + e;
+            ST x = to_sum<ST>(reinterpret_cast<const VT*>(a.ha)[at]);
+            add_sum(x, reinterpret_cast<const VT*>(a.ha_lo)[at]);
+            add_sum(x, Z[r * xk + e]);
+            Z[r * xk + e] = sum_val(x);
+          }
+        __syncthreads();
+      }
     }
   }
   if (!H && len > 0 && (mode & MODE_BWD) && !bd) {  // beta, used after the prox
@@ -616,15 +634,14 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
       for (int j = lane; j < n_v; j += 32) cp_async_elem(V + r * xv + j, beta + (long long)sid[r] * n_v + j);
   }
   if (prox) {
-    const int pmode = H ? mode & ~MODE_AFTER_ANCHOR : mode;  // FORM 2 keeps h_a, not x and u
     const int rows = L - own, ni = (n_u + 63) / 64;
     for (int task = warp; task < rows * (1 + ni); task += NW) {
       if (task < rows) {
         const int r = own + task;
-        sweep_tanks<VT, NT, FORM>(a, sid[r], Z + r * xk, bnd, nu - 1, c, cn, pmode, o);
+        sweep_tanks<VT, NT, FORM>(a, sid[r], Z + r * xk, bnd, nu - 1, c, cn, mode, o);
       } else {
         const int q = (task - rows) / ni, r = own + q;
-        sweep_inputs<VT, FORM>(a, sid[r], 64 * (task - rows - q * ni), Z + r * xk, bnd, nu - 1, c, cn, pmode, o);
+        sweep_inputs<VT, FORM>(a, sid[r], 64 * (task - rows - q * ni), Z + r * xk, bnd, nu - 1, c, cn, mode, o);
       }
     }
     if (o.r.bad() || o.h.bad()) a.flags[1] = SMPC_EDIVERGED;
