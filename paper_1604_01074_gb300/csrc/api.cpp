@@ -1054,8 +1054,8 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   f->W_alpha = cost->W_alpha;
   f->gamma_d = cost->gamma_d;
   // Diagnostics: SMPC_PIPELINE_WAIT_NS (nanoseconds; 0 = one non-blocking test) replaces
-  // the 2 s bound of node_mv's pack-pipeline waits for this factor's solves, so that a test
-  // can make a wait give up (SMPC_ETIMEOUT) without a fault; the waits that let copies in
+  // the 2 s bound of the matrix waits of node_mv and lambda_apply for this factor's solves, so
+  // that a test can make a wait give up (SMPC_ETIMEOUT) without a fault; the waits that let copies in
   // flight land keep the 2 s bound.
   if (const char* w = std::getenv("SMPC_PIPELINE_WAIT_NS")) {
     char* end = nullptr;

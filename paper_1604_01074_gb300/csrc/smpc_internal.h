@@ -142,7 +142,7 @@ struct IterArgs {
   double tol;
   double* pw;                    // power iteration: [k] ||y_k||^2, [K + k] <y_k, y_{k+1}>
   int pw_len;
-  unsigned long long wait_ns;    // bound of the per-node pack pipeline waits of node_mv
+  unsigned long long wait_ns;    // bound of the matrix waits of node_mv and lambda_apply
   // Forests (R > 1 trees): each tree stops at its own first iterate whose relative residual
   // meets tol.  res_tree: per iteration and tree, (rho, ||Hz||, ||t||) as float64 bits, or
   // NULL (one residual for the whole forest); tree_done: per tree, the iterations it ran

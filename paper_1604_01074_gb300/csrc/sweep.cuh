@@ -1020,7 +1020,7 @@ __global__ void __launch_bounds__((LW + 8) * 32, BS == 4 && sizeof(VT) == 4 ? 2 
       for (int k = 0; k < RL; ++k) rs[warp][lane + 32 * k] = rn[k];
       if (m1 >= 0) read_r(m1);
       if (slots > 0) {
-        const bool ok = mbar_wait(one ? &bar[0] : &bar[warp], one ? 0 : phase);
+        const bool ok = mbar_wait(one ? &bar[0] : &bar[warp], one ? 0 : phase, a.wait_ns);
         if (!__all_sync(0xffffffffu, ok)) {
           if (lane == 0) a.flags[1] = SMPC_ETIMEOUT;
           mbar_wait(one ? &bar[0] : &bar[warp], one ? 0 : phase);  // bounded: let the copy land
