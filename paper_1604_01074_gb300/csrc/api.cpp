@@ -1285,7 +1285,7 @@ int smpc_factor_schedule(const smpc_factor_t* f, double* ms_per_iter) {
     ms_per_iter[3] = f->tuned_ms[SCHED_FUSED];
     const float sw = f->tuned_ms[SCHED_SWEEP];  // the two-launch form, where that was timed and is faster
     double& as = ms_per_iter[(f->A ? SCHED_NODE : SCHED_FUSED) - 1];
-    if (sw > 0 && sw < as) as = sw;
+    if (sw > 0 && (as == 0 || sw < as)) as = sw;  // 0: that schedule itself does not fit
   }
   return f->schedule == SCHED_SWEEP ? (int)(f->A ? SCHED_NODE : SCHED_FUSED) : f->schedule;
 }
