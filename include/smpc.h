@@ -232,7 +232,9 @@ void smpc_tree_destroy(smpc_tree* tree);
  * node-indexed factor matrices) in the requested precision on the device, the
  * Jacobi scaling (Sec. IV-D) and the step lambda = 1/L_{H_D} (power iteration
  * on the device, unless given).  An SMPC_BF16 factor also keeps float32 packs for
- * the anchor and polish iterations of smpc_solve_opts.  The tree must outlive the factor.
+ * the anchor and polish iterations of smpc_solve_opts.  A factor in the two-launch form (see
+ * smpc_factor_opts.schedule) keeps one half of every symmetric Lambda / (2 p_n) and one sparse
+ * [B_bar; L] in place of the packs once it is built.  The tree must outlive the factor.
  * Errors: SMPC_EINVAL (sizes, NaN, E rank deficient, W_u not SPD),
  *         SMPC_ENOTSUP (A != I with a schedule other than 0 or 2), SMPC_ENOMEM, SMPC_ECUDA. */
 int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost* cost,
@@ -332,6 +334,7 @@ void smpc_batch_destroy(smpc_batch* batch);
  * outputs hold its own chains' and the top nodes' entries (others are not updated).  Stops
  * are the same on every GPU since every GPU reads the same residuals.  float64 and float32
  * factors of a single tree whose root is a top node; all calls on the stream of begin.
+ * smpc_shard_create allocates the packs of a factor that keeps none (the two-launch form).
  * Errors: SMPC_EINVAL, SMPC_ENOTSUP (bfloat16, a chain starting at a root), SMPC_ENOMEM,
  * SMPC_ECUDA, and the solve's own errors from smpc_shard_finish. */
 int smpc_shard_create(smpc_factor_t* fac, int32_t chain_begin, int32_t chain_end, smpc_shard** out);

@@ -303,7 +303,7 @@ void set_sweep_args(const smpc_factor_t* f, IterArgs& a) {
   const smpc_tree* t = f->tree;
   a.sp = t->top_src_off.empty() ? nullptr : f->sp;
   a.sp_nnz = f->sp_nnz;
-  a.kd = f->prec == SMPC_BF16 && f->form != FORM_SEPARATE ? f->packs : nullptr;
+  a.kd = f->prec == SMPC_BF16 && f->form != FORM_SEPARATE ? (f->kd ? f->kd : f->packs) : nullptr;
   a.depth = t->N;
   a.max_len = t->max_chain_len;
   a.ha_lo = f->ha_lo;
@@ -615,6 +615,9 @@ int build_two_launch(smpc_factor_t* f, const smpc_network& net, const double* W_
   TRY(f->alloc(&lam, entries * f->ms));
   TRY(launch_lam_pack(f->prec, np, n_v, b16 ? f->Lam64 : Lam, prob, lam, nullptr));
   if (b16) {
+    const long long pe = pack_entries(SMPC_BF16, n_k, n_v);  // one node's pack: its [Bbar; L]
+    TRY(f->alloc(&f->kd, (size_t)pe * f->ms));
+    TRY(launch_pack(SMPC_BF16, 1, n_k, n_v, f->K64, f->Lam64, nullptr, f->kd, pe, nullptr));
     TRY(f->alloc(&f->ha_lo, sizeof(float) * (size_t)f->n * n_k));
     TRY(f->alloc(&f->lam32, entries * sizeof(float)));
     TRY(launch_lam_pack(SMPC_FP32, np, n_v, Lam, prob, f->lam32, nullptr));
@@ -628,7 +631,7 @@ int build_two_launch(smpc_factor_t* f, const smpc_network& net, const double* W_
 void drop_two_launch(smpc_factor_t* f, size_t mark, size_t bytes) {
   for (; f->allocs.size() > mark; f->allocs.pop_back()) cudaFree(f->allocs.back());
   f->device_bytes = bytes;
-  f->sp = f->lam = f->lam32 = f->ha_lo = nullptr;
+  f->sp = f->kd = f->lam = f->lam32 = f->ha_lo = nullptr;
   f->Rhat_red = f->L_red = nullptr;
   f->rhat_t_red = CsrRows();
 }
@@ -802,7 +805,7 @@ int plan_iters(const smpc_factor_t* f, const IterArgs& a, const smpc_solve_opts&
   plan->polish_from = 0x7fffffff;
   plan->anchor_every = 0;
   plan->profile = f->profile;
-  if (f->packs32) {  // SMPC_BF16: anchored solve, float32 packs for anchors and polish
+  if (f->prec == SMPC_BF16) {  // anchored solve, float32 packs for anchors and polish
     plan->args.ha = f->ha;
     plan->args.wa = f->wa;
     plan->args32 = plan->args;
@@ -818,6 +821,14 @@ int plan_iters(const smpc_factor_t* f, const IterArgs& a, const smpc_solve_opts&
     if (opts.polish_iters > 0) plan->polish_from = iters - opts.polish_iters;
   }
   return SMPC_OK;
+}
+
+int build_packs(smpc_factor_t* f) {
+  const int np = f->shared_packs ? 1 : f->n;
+  const double* prob = f->shared_packs ? nullptr : f->tree->dev.prob;
+  const long long pe = pack_entries(f->prec, f->n_k, f->n_v);
+  TRY(f->alloc(&f->packs, (size_t)np * pe * f->ms));
+  return launch_pack(f->prec, np, f->n_k, f->n_v, f->K64, f->Lam64, prob, f->packs, pe, nullptr);
 }
 
 int copy_final_y(smpc_factor_t* f, void* dst) {
@@ -1092,8 +1103,7 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   const double* pprob = f->shared_packs ? nullptr : tree->dev.prob;
   const long long pe = pack_entries(f->prec, n_k, n_v);
   f->pack_stride = f->shared_packs ? 0 : pe;
-  if ((rc = f->alloc(&f->packs, (size_t)np * pe * f->ms))) return fail(rc);
-  if ((rc = launch_pack(f->prec, np, n_k, n_v, f->K64, f->Lam64, pprob, f->packs, pe, nullptr))) return fail(rc);
+  if ((rc = build_packs(f))) return fail(rc);
   if (f->shared_packs) {
     std::vector<double> sc(n);
     for (int m = 0; m < n; ++m) sc[m] = 1.0 / (2.0 * tree->prob[m]);
@@ -1264,7 +1274,13 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   if (rc == SMPC_ENOMEM) drop_two_launch(f, mark, mark_bytes);
   if ((rc = choose_schedule(f, o.schedule))) return fail(rc);
   if ((rc = tune_tc(f, o.tc_width))) return fail(rc);
-  if (f->schedule != SCHED_SWEEP) drop_two_launch(f, mark, mark_bytes);
+  if (f->schedule != SCHED_SWEEP) {
+    drop_two_launch(f, mark, mark_bytes);
+  } else {  // its solves read no pack; a shard builds them again
+    const size_t nodes = f->shared_packs ? 1 : (size_t)n;
+    f->release(&f->packs, nodes * pe * f->ms);
+    f->release(&f->packs32, nodes * pack_entries(SMPC_FP32, n_k, n_v) * sizeof(float));
+  }
   *out = f;
   return SMPC_OK;
 }

@@ -105,6 +105,10 @@ int smpc_shard_create(smpc_factor_t* f, int32_t chain_begin, int32_t chain_end, 
       set_error("chain %d starts at a root: a tree split into shards needs top nodes above every chain", c);
       return SMPC_ENOTSUP;
     }
+  if (!f->packs) {  // a factor in the two-launch form keeps none for its own solves
+    SHTRY(build_packs(f));
+    SHCK(cudaDeviceSynchronize());
+  }
   auto* sh = new (std::nothrow) smpc_shard();
   if (!sh) {
     set_error("out of host memory");

@@ -2,6 +2,7 @@
 // the device code (kernels.cu).  Not part of the public ABI.
 #pragma once
 
+#include <algorithm>
 #include <array>
 #include <cstddef>
 #include <cstdint>
@@ -351,6 +352,8 @@ void set_sweep_args(const smpc_factor_t* f, IterArgs& a);
 // The basis of beta (c.L, c.Rhat, c.rhat_t): the reduced one for the two-launch form, the
 // orthonormal one of the packs for the other schedules and for shards.
 void set_basis(const smpc_factor_t* f, bool shard, CostArgs& c);
+// The packs of schedules 1 to 4 (f->packs), from the float64 matrices on the device.
+int build_packs(smpc_factor_t* f);
 // Copies the final dual of the factor's last solve (vector type) to dst; synchronous.
 int copy_final_y(smpc_factor_t* f, void* dst);
 }  // namespace smpc
@@ -369,7 +372,7 @@ struct smpc_factor_t {
   std::vector<void*> allocs;
   size_t device_bytes = 0;  // sum of this factor's device allocations
   // device
-  void* packs = nullptr;
+  void* packs = nullptr;      // schedules 1 to 4 and shards (NULL: SCHED_SWEEP without a shard)
   bool shared_packs = false;  // one pack [Bbar; L | Lambda] for every node, scaled by pscale
   void* pscale = nullptr;     // shared packs: per node 1 / (2 p_n), vector type
   void* packs32 = nullptr;    // SMPC_BF16 only: float32 packs (anchor and polish launches)
@@ -408,6 +411,7 @@ struct smpc_factor_t {
   // ... of a bfloat16 factor: the anchors' float32 Lambda, in the reduced basis (lam: bfloat16,
   // in the orthonormal basis of the packs)
   void* lam32 = nullptr;
+  void* kd = nullptr;     // IterArgs::kd
   void* ha_lo = nullptr;  // IterArgs::ha_lo
   // ... the cost update's matrices in the reduced basis
   double *Rhat_red = nullptr, *L_red = nullptr;
@@ -436,6 +440,15 @@ struct smpc_factor_t {
     graphs.clear();
   }
 
+  template <typename T>
+  void release(T** p, size_t bytes) {
+    const auto it = std::find(allocs.begin(), allocs.end(), (void*)*p);
+    if (!*p || it == allocs.end()) return;
+    cudaFree(*p);
+    allocs.erase(it);
+    device_bytes -= bytes;
+    *p = nullptr;
+  }
   template <typename T>
   int alloc(T** p, size_t bytes) {
     *p = nullptr;
