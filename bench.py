@@ -125,11 +125,15 @@ def algorithmic_bytes_per_iteration(n, n_x, n_u, n_v, prec):
 
 STAGES = {1: ["apg_iter"], 2: ["fwd_scan", "prox_node", "scan_s", "node_mv_gt", "scan_r", "node_mv_dh"],
           3: ["fwd_scan", "prox_node", "apg_iter_gt", "node_mv_dh"], 4: ["fwd_scan", "prox_node", "apg_iter_bwd"]}
-SWEEP_STAGES = ["tree_sweep", "lambda_apply"]  # the two-launch form of schedule 4 (sparse [Bbar; L])
+SWEEP_STAGES = ["tree_sweep", "lambda_apply"]  # the two-launch form (sparse [Bbar; L]), reported as 4 (general A: 2)
+MERGED_STAGES = ["merged_sweep", "node_mv_gt", "scan_r", "node_mv_dh"]  # schedule 2, bfloat16 shared packs
 
 
 def stages_of(schedule, stage_ms):
-    return SWEEP_STAGES if len(stage_ms) == 2 else STAGES[schedule]
+    """The launches of an iteration that smpc_profile_solve timed, by their number."""
+    if len(stage_ms) == 2:
+        return SWEEP_STAGES
+    return MERGED_STAGES if schedule == 2 and len(stage_ms) == 4 else STAGES[schedule]
 
 
 def stage_bytes(stage, n, n_x, n_u, n_v, prec, shared):
@@ -386,6 +390,11 @@ class Solver:
     def finish(self):
         return self.smpc.smpc_solve_info(self.fac)
 
+    def schedule_name(self):
+        P = self.P
+        ms = self.smpc.smpc_profile_solve(self.fac, P["p"], P["q"], P["dhat"], P["alpha2"], eps=P["eps"], iters=4)
+        return schedule_name(self.schedule, len(ms))
+
     def close(self):
         self.smpc.smpc_factor_destroy(self.fac)
         self.smpc.smpc_tree_destroy(self.tree)
@@ -412,6 +421,11 @@ def time_per_iteration(S, inp, stream, lo=100, hi=400, reps=3):
 
 
 SCHED_NAMES = {1: "chain", 2: "node-parallel", 3: "hybrid", 4: "fused chain pass"}
+
+
+def schedule_name(schedule, launches):
+    """The schedule's name from its number and the launches of an iteration."""
+    return "two-launch (tree pass, Lambda)" if launches == 2 else SCHED_NAMES[schedule]
 
 
 def kernel_roofline(S, P, prec, inp, stream, fp64_peak, iters=200):
@@ -542,7 +556,7 @@ def run_ours(args, rank, world, local_rank):
         "vs_baseline": None, "dtype": PREC_NAMES[prec], "data": "synthetic",
         "config": {"workload": WORKLOADS[args.config], "solve": "cold start, tol 1e-3 on rho_rel", "tol": args.tol,
                    "max_iters": args.max_iters, "precision": args.precision, "packs": "per node",
-                   "schedule": SCHED_NAMES[S.schedule], "schedule_tuning_ms": S.tuned_ms,
+                   "schedule": S.schedule_name(), "schedule_tuning_ms": S.tuned_ms,
                    "l2": "inputs (packs) larger than L2, and a 256 MB buffer written between timed solves",
                    "parallelism": f"replicas x{world}",
                    "launch": "plain launches" if args.no_graph else
@@ -593,7 +607,7 @@ def run_legs(args, P, prec, dev_in, stream, flush, fp64_peak):
                 steps = So.smpc.smpc_factor_steps(So.fac, n, P["net"]["n_u"])[1]
             if other != prec:
                 leg = kernel_roofline(So, P, other, dev_in[0], stream, fp64_peak)
-                leg["schedule"] = SCHED_NAMES[So.schedule]
+                leg["schedule"] = So.schedule_name()
                 legs[PREC_NAMES[other] + "_per_node"] = leg
                 log("leg", PREC_NAMES[other], {k: leg[k] for k in ("us_per_iteration", "kernel", "frac")})
         finally:
@@ -605,7 +619,7 @@ def run_legs(args, P, prec, dev_in, stream, flush, fp64_peak):
         times, iters, _ = timed_solves(Sh, dev_in, range(min(len(dev_in), args.leg_solves)), stream, args, flush)
         legs[PREC_NAMES[prec] + "_shared_packs"] = {
             "solves_per_s": 1000.0 * len(times) / sum(times), "ms_per_solve": float(np.mean(times)),
-            "iterations_mean": float(np.mean(iters)), "schedule": SCHED_NAMES[Sh.schedule],
+            "iterations_mean": float(np.mean(iters)), "schedule": Sh.schedule_name(),
             "factor_device_bytes": Sh.smpc.smpc_factor_device_bytes(Sh.fac),
             "note": "one pack per factor: the per-node matrices differ only by 1/(2 p_n), applied to Lambda r"}
         log("leg shared", legs[PREC_NAMES[prec] + "_shared_packs"])
@@ -624,7 +638,7 @@ def run_legs(args, P, prec, dev_in, stream, flush, fp64_peak):
         times, iters, _ = timed_solves(Sb, inb, range(1, args.leg_solves + 1), stream, args, flush)
         leg = {"workload": WORKLOADS["barcelona"], "precision": "fp32", "packs": "per node",
                "solves_per_s": 1000.0 * len(times) / sum(times), "ms_per_solve": float(np.mean(times)),
-               "iterations_mean": float(np.mean(iters)), "schedule": SCHED_NAMES[Sb.schedule]}
+               "iterations_mean": float(np.mean(iters)), "schedule": Sb.schedule_name()}
         leg["roofline"] = kernel_roofline(Sb, Pb, 1, inb[0], stream, fp64_peak)
         legs["barcelona_fp32_per_node"] = leg
         log("leg barcelona", {k: leg[k] for k in ("solves_per_s", "iterations_mean", "schedule")})

@@ -354,10 +354,12 @@ void smpc_shard_destroy(smpc_shard* shard);
  * of every full iteration, and writes the mean device time in ms
  * of each kernel of an iteration to stage_ms[0 .. min(n, max_stages)).  n = 1 for schedule 1
  * (apg_iter), 6 for schedule 2 (forward sweep, prox and dual update, subtree scan of s,
- * [Bbar; L]' mat-vec, subtree scan of r, Lambda and [Bbar; L] mat-vecs) and 4 for schedule 3
- * (forward sweep; prox and dual update; s, [Bbar; L]' mat-vecs and r along the chains; Lambda
- * and [Bbar; L] mat-vecs) and 3 for schedule 4 (forward sweep; prox and dual update; the
- * whole backward sweep along the chains; n = 2 for the two-launch form: tree pass; Lambda r).
+ * [Bbar; L]' mat-vec, subtree scan of r, Lambda and [Bbar; L] mat-vecs; 4 for SMPC_BF16 with
+ * shared packs, whose first three are one launch where the tree's depth fits its shared
+ * memory), 4 for schedule 3 (forward sweep; prox and dual update; s, [Bbar; L]' mat-vecs and r
+ * along the chains; Lambda and [Bbar; L] mat-vecs), 3 for schedule 4 (forward sweep; prox and
+ * dual update; the whole backward sweep along the chains) and 2 for the two-launch form, which
+ * is reported as schedule 4 or, with a general A, 2 (tree pass; Lambda r).
  * SMPC_BF16 anchor iterations are not timed.  Leaves
  * the factor's duals as that solve ends.  Returns n, or minus an smpc_status. */
 int smpc_profile_solve(smpc_factor_t* fac, const smpc_step_data* data, int32_t iters, double* stage_ms,
