@@ -58,14 +58,18 @@ FP64_FMA_TFLOPS = 1.157
 
 
 def recorded_traffic(prec_name):
-    """DRAM bytes per launch from the last ncu capture in profiles/, if the kernel
-    source is unchanged since (else None)."""
+    """DRAM bytes per launch from the last ncu capture in profiles/, if the source of its
+    kernel is unchanged since (else None): sweep.cuh for the two-launch form's kernels
+    (the list two_launch), kernels.cu for the others."""
     import hashlib
     try:
         rec = json.load(open(os.path.join(ROOT, "profiles", "traffic.json")))
-        src = open(os.path.join(ROOT, "paper_1604_01074_gb300", "csrc", "kernels.cu"), "rb").read()
-        if hashlib.sha256(src).hexdigest()[:16] != rec.get("kernel_sha256_16"):
+        sweep = any(k in prec_name for k in SWEEP_STAGES)
+        src = open(os.path.join(ROOT, "paper_1604_01074_gb300", "csrc", "sweep.cuh" if sweep else "kernels.cu"), "rb").read()
+        if hashlib.sha256(src).hexdigest()[:16] != rec.get("sweep_sha256_16" if sweep else "kernel_sha256_16"):
             return None
+        if sweep:
+            return next((r["dram_bytes_per_launch"] for r in rec["two_launch"] if r["key"] == prec_name), None)
         return rec.get(prec_name, {}).get("dram_bytes_per_launch")
     except Exception:  # noqa: BLE001
         return None

@@ -3246,7 +3246,12 @@ LaunchCfg config_t(const IterArgs& a, int num_sms, int S_max, int schedule, int 
     if (std::is_same<VT, MT>::value || b16) {
       c.smem = sweep_smem_bytes<VT>(a.sp_nnz, a.depth, a.n_x, a.n_u, a.n_v, a.A != nullptr, b16);
       c.grid = a.n_chains + a.n_top;
-      const int tasks = a.max_len * (1 + (a.n_u + 63) / 64);  // of a chain's prox, one warp each
+      // Warps a CTA, by chains per SM and by the tasks of a chain's prox (one warp each): few warps
+      // where chains share an SM, many where one chain has it alone.  us an iteration with 8, 16,
+      // 32 warps, float32: 100 chains of 20 nodes 45, 32, 28; 242 of 21: 61, 46, 62; 300: 66, 57,
+      // 71; 400: 73, 73, 90; 1000: 148, 163, 204; chains of 4 nodes 20, 20, 26 and of 3 (9 tasks at
+      // most) 13.2, 13.3, 14.1.  float64 (16 at most): 100 chains 145, 117; 500: 411, 442.
+      const int tasks = a.max_len * (1 + (a.n_u + 63) / 64);
       c.sweep_warps = a.n_x > 64 || b16 ? 16
                       : a.n_chains > 2 * num_sms || tasks <= 8 ? 8
                       : a.n_chains <= num_sms && tasks >= 48 && sizeof(VT) == 4 ? 32 : 16;

@@ -17,12 +17,12 @@
 //                 itself forms the two terms in tree_sweep, so no top node waits for another.
 // A general A: x and s along a chain take one product with A per node (A in shared memory, a
 // block barrier each), and s and r of the top nodes climb in tree_sweep.  1531 nodes of a
-// 50-tank network: 45 us an iteration, against 128 us of the six launches of schedule 2.
-// Per iteration on GB300, one pack per node (the launches of schedules 2 to 4 before): 2081
-// nodes 27.2 us in float32 (104), 116 us in float64 (381); 21 111 nodes 145 us (577), the tree
-// pass 71 and Lambda 75; one pack for all of 21 111 nodes 107 us (396).  The tree pass is bound
-// by issue slots (some 2400 warp instructions a node, half of them the prox in float32 pairs),
-// Lambda by HBM (439 MB at 5.9 TB/s) and in float64 by the pipe (2 lanes a cycle and SM).
+// 50-tank network: 46 us an iteration, against 137 us of the six launches of schedule 2.
+// Per iteration on GB300, one pack per node (the fastest of schedules 1 to 4): 2081 nodes 28 us in
+// float32 (105), 117 us in float64 (388); 21 111 nodes 147 us (580), between events the tree pass
+// 76 and Lambda 85; one pack for all of 21 111 nodes 107 us (401).  The tree pass is bound by issue
+// slots (2 530 warp instructions a node, half of them the prox in float32 pairs), Lambda by HBM
+// (439 MB, 5.9 TB/s without the gap before it) and in float64 by the pipe (2 lanes a cycle and SM).
 // Vectors between the launches: h holds delta (n x n_v), rpub r of the chain nodes, spub s of
 // the chain heads; a top node m's row of rpub holds R_m + L' psi_m, the first n_v entries of
 // its row of wbuf (w, until the last arrival) Bbar' S_m.
@@ -366,8 +366,9 @@ __device__ __forceinline__ unsigned long long bf2(uint32_t u) {
 // rows at a time.  Forward: put(r, e, (K V_r)_e), a lane per row e of K; the four rows' entries
 // are broadcast reads, and pairs of products go through f32x2.  Backward: put(r, j, (K' Z_r)_j),
 // two columns a lane.  They double the pass's instructions (about 550 and 800 a node at 177 x
-// 97 entries): 174 us on 21 111 nodes, against 457 us for streaming each node's own copy of K
-// through the chains.
+// 97 entries), and still take less than streaming each node's own copy of K through the chains:
+// 15 111 nodes of 18 stages 175 us an iteration, the pass 147 of them, against 433 with a chain
+// pass of 366.
 template <int NW, typename F>
 __device__ __forceinline__ void dense_fwd(const uint32_t* K, int kw, int n_k, const float* V, int xv, int r0, int r1,
                                           F&& put) {
@@ -450,7 +451,7 @@ __device__ __forceinline__ void add_Ax(const VT* A, int n, bool trans, const VT*
 // dense_fwd).  2: bfloat16 factors with one pack, whose products stay on the tensor cores:
 // the first half of an iteration of schedule 2 in one launch - path sums of h, prox, s of every
 // node - with the arithmetic of fwd_scan, prox_node and scan_kernel, in place of those three:
-// 38 us instead of 73 on 13 830 nodes and 20 tanks, 72 instead of 109 on 15 876 nodes and 63.
+// 40 us instead of 73 on 13 830 nodes and 20 tanks, 72 instead of 108 on 15 876 nodes and 63.
 template <typename VT>
 __host__ __device__ inline size_t hsweep_smem_bytes(int depth, int n_x, int n_u) {
   const size_t b = round_up((size_t)(3 * n_x + 2 * n_u) * sizeof(VT), 16) + (size_t)3 * (depth + 3) * (n_x + n_u) * sizeof(VT);
@@ -713,7 +714,7 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
       }
     }
     return;
-  } else {
+  }
   if (len == 0) {  // a top node: its w
     VT* w = reinterpret_cast<VT*>(a.wbuf) + (long long)sid[own] * n_k;
     for (int e = tid; e < n_k; e += kSweepThreads) w[e] = Z[own * xk + e];
@@ -812,7 +813,6 @@ __global__ void __launch_bounds__(32 * NW, NT == 8 ? 1 : (sizeof(VT) == 4 ? 32 :
     if (!bd) sparse_rows<NW, VT>(
         et, cptr, cid, n_v, Z, xk, 0, climb ? 1 : 2, [&](int r, int j) -> VT { return climb || r == 1 ? R0[j] : (VT)0; },
         [&](int r, int j, VT v) { (climb || r == 1 ? rp + (long long)t * n_v : wt)[j] = v; });
-  }
   }
 }
 

@@ -1,4 +1,8 @@
-"""bench.py's names for the launches of an iteration, by schedule and number."""
+"""bench.py's names for the launches of an iteration, by schedule and number, and the recorded DRAM
+traffic of the two-launch form's kernels, valid while their own source is unchanged."""
+import hashlib
+import json
+
 import pytest
 
 import bench
@@ -20,3 +24,21 @@ def test_merged_launch_is_followed_by_the_product_of_the_transposed_pack():
 def test_two_launch_form_has_its_own_label():
     assert bench.schedule_name(4, 2) == bench.schedule_name(2, 2) != bench.schedule_name(4, 3)
     assert bench.schedule_name(2, 4) == bench.schedule_name(2, 6)
+
+
+def test_traffic_of_the_two_launch_kernels_follows_their_source(tmp_path, monkeypatch):
+    src = tmp_path / "paper_1604_01074_gb300" / "csrc"
+    src.mkdir(parents=True)
+    (tmp_path / "profiles").mkdir()
+    (src / "kernels.cu").write_bytes(b"// k")
+    (src / "sweep.cuh").write_bytes(b"// s1")
+    sha = hashlib.sha256(b"// s1").hexdigest()[:16]
+    rec = {"kernel_sha256_16": "0", "sweep_sha256_16": sha,
+           "two_launch": [{"key": "fp32_lambda_apply_21111", "dram_bytes_per_launch": 5}]}
+    (tmp_path / "profiles" / "traffic.json").write_text(json.dumps(rec))
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    assert bench.recorded_traffic("fp32_lambda_apply_21111") == 5
+    assert bench.recorded_traffic("fp32_tree_sweep_21111") is None
+    assert bench.recorded_traffic("fp32_apg_iter_bwd_21111") is None
+    (src / "sweep.cuh").write_bytes(b"// s2")
+    assert bench.recorded_traffic("fp32_lambda_apply_21111") is None
