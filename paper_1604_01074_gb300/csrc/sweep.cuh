@@ -138,6 +138,13 @@ struct MaxAbs<double> {
   __device__ double value() const { return __longlong_as_double((long long)b); }
 };
 
+// st_val(st_sub(a, b)): the rounded sum of the difference's two terms is what renormalising them
+// and adding them up again gives.
+__device__ __forceinline__ float sub_val(DS a, DS b) {
+  const DS t = two_sum(a.hi, -b.hi);
+  return __fadd_rn(t.hi, __fadd_rn(t.lo, __fsub_rn(a.lo, b.lo)));
+}
+__device__ __forceinline__ double sub_val(double a, double b) { return a - b; }
 // Signs of the tree pass: in float64 read from the bits, off the float64 pipe.
 __device__ __forceinline__ bool sw_neg(DS x) { return x.hi < 0.f; }
 __device__ __forceinline__ bool sw_neg(double x) { return __double_as_longlong(x) < 0; }
@@ -234,7 +241,7 @@ __device__ __forceinline__ void sweep_tanks(const IterArgs& a, int m, VT* z, con
     if (e < n_x) {
       const VT x = z[e];
       const ST ysn = st_scale(qs[k], ks), yzn = st_scale(qz[k], kz);
-      const VT es = st_val(st_sub(ysn, ws[k])) * is, ez = st_val(st_sub(yzn, wz[k])) * iz;
+      const VT es = sub_val(ysn, ws[k]) * is, ez = sub_val(yzn, wz[k]) * iz;
       st_state(y2 + e, ysn);
       st_state(y2 + n_x + e, yzn);
       xo[e] = x;
@@ -292,7 +299,7 @@ __device__ __forceinline__ void sweep_inputs(const IterArgs& a, int m, int i0, V
       const VT u = z[n_x + i];
       const ST wp = st_extrap(p1[k], p2[k], c);
       const ST ypn = sw_box(st_axpy(wp, lp[k], u - uhi[i]), st_axpy(wp, lp[k], u - ulo[i]));
-      const VT ep = st_val(st_sub(ypn, wp)) * ip[k];
+      const VT ep = sub_val(ypn, wp) * ip[k];
       st_state(y2 + i, ypn);
       reinterpret_cast<VT*>(a.uout)[mu + i] = u;
       if (B16 && (mode & MODE_DELTA)) {
