@@ -225,8 +225,8 @@ void smpc_tree_destroy(smpc_tree* tree);
 
 /* Offline factor step (App. A and App. B; Alg. 2 lines 1-2), in float64 on the
  * host: L = orthonormal basis of null(E) (the two-launch form: the reduced basis
- * [-E1^{-1} E2; I], which keeps a network's incidence structure, where cond(L'L) <= 40; u, x
- * and y do not depend on the basis), B_bar = B L, R_hat = W_u L,
+ * [-E1^{-1} E2; I], which keeps a network's incidence structure, where cond(L'L) <= 40 or no
+ * other schedule fits; u, x and y do not depend on the basis), B_bar = B L, R_hat = W_u L,
  * R_bar = L' R_hat, Cholesky of R_bar, Lambda = -R_bar^{-1}; then per-node packs
  * [B_bar; L] (n_x + n_u) x n_v and Lambda / (2 p_n) (n_v x n_v, Alg. 1's
  * node-indexed factor matrices) in the requested precision on the device, the

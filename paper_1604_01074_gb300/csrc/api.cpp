@@ -593,7 +593,12 @@ int build_two_launch(smpc_factor_t* f, const smpc_network& net, const double* W_
       (b16 && (f->shared_packs || f->A || tree->N > kB16Stages)))
     return SMPC_OK;
   HostFactor red;
-  if (host_factor(net, W_u, red, true) != SMPC_OK) return SMPC_OK;
+  // a network whose packs none of schedules 1 to 4 can hold (float64, more than about 100 free
+  // inputs) has no better conditioned choice
+  const IterArgs a = make_args(f);
+  bool others = false;
+  for (int s = 1; s <= kSchedules; ++s) others = others || iter_config(f->prec, a, f->num_sms, s).stages > 0;
+  if (host_factor(net, W_u, red, others ? BASIS_REDUCED : BASIS_REDUCED_ANY) != SMPC_OK) return SMPC_OK;
   std::vector<double> Ks((size_t)n_k * n_v);
   std::copy(red.Bbar.begin(), red.Bbar.end(), Ks.begin());
   std::copy(red.L.begin(), red.L.end(), Ks.begin() + (size_t)n_x * n_v);
@@ -1054,7 +1059,7 @@ int smpc_factor(const smpc_tree* tree, const smpc_network* net, const smpc_cost*
   f->n_u = n_u;
   f->n_d = n_d;
   f->n_e = n_e;
-  int rc = host_factor(*net, cost->W_u, f->hf, false);
+  int rc = host_factor(*net, cost->W_u, f->hf, BASIS_ORTHONORMAL);
   if (rc != SMPC_OK) return fail(rc);
   const int n_v = f->hf.n_v;
   f->n_v = n_v;

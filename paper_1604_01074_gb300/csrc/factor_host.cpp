@@ -133,8 +133,9 @@ double spectral_square(const std::vector<double>& F, int n_e, int n_f) {
 // of the basis are those of F = -E1^{-1} E2 for E1's columns and unit rows for the others.  For
 // an incidence matrix it is sparse (a junction's balance solved for one of its actuators), and
 // so is B L.  Gauss-Jordan elimination with complete pivoting, ties towards the column with the
-// fewest entries.  False (L untouched) when cond(L'L) = 1 + ||F||^2 exceeds kMaxCond.
-bool reduced_null_basis(const double* E, int n_e, int n_u, std::vector<double>& L) {
+// fewest entries.  False (L untouched) when cond(L'L) = 1 + ||F||^2 exceeds kMaxCond or, with any, an
+// entry of F exceeds 4.
+bool reduced_null_basis(const double* E, int n_e, int n_u, bool any, std::vector<double>& L) {
   std::vector<double> M(E, E + (size_t)n_e * n_u);
   std::vector<int> piv(n_e, -1), used(n_u, 0), count(n_u, 0);
   for (int i = 0; i < n_e; ++i)
@@ -173,6 +174,7 @@ bool reduced_null_basis(const double* E, int n_e, int n_u, std::vector<double>& 
     B[(size_t)j * n_v + k] = 1.0;
     for (int i = 0; i < n_e; ++i) {
       const double v = M[(size_t)i * n_u + j];
+      if (any && !(std::fabs(v) <= 4.0)) return false;
       if (std::fabs(v) > 1e-15) {  // cancellations leave some 1e-16
         B[(size_t)piv[i] * n_v + k] = -v;
         F[(size_t)i * n_v + k] = -v;
@@ -180,14 +182,14 @@ bool reduced_null_basis(const double* E, int n_e, int n_u, std::vector<double>& 
     }
     ++k;
   }
-  if (!(1.0 + spectral_square(F, n_e, n_v) <= kMaxCond)) return false;
+  if (!any && !(1.0 + spectral_square(F, n_e, n_v) <= kMaxCond)) return false;
   L = B;
   return true;
 }
 
 }  // namespace
 
-int host_factor(const smpc_network& net, const double* W_u, HostFactor& f, bool reduced_basis) {
+int host_factor(const smpc_network& net, const double* W_u, HostFactor& f, Basis basis) {
   const int n_x = net.n_x, n_u = net.n_u, n_d = net.n_d, n_e = net.n_e;
   f.n_x = n_x;
   f.n_u = n_u;
@@ -217,7 +219,8 @@ int host_factor(const smpc_network& net, const double* W_u, HostFactor& f, bool 
     f.L.assign((size_t)n_u * f.n_v, 0.0);
     for (int i = 0; i < n_u; ++i)
       for (int j = 0; j < f.n_v; ++j) f.L[i * f.n_v + j] = Q[i * n_u + n_e + j];
-    if (reduced_basis && !reduced_null_basis(net.E, n_e, n_u, f.L)) return SMPC_ENOTSUP;
+    if (basis != BASIS_ORTHONORMAL && !reduced_null_basis(net.E, n_e, n_u, basis == BASIS_REDUCED_ANY, f.L))
+      return SMPC_ENOTSUP;
     // Pu = -E' (E E')^{-1} Ed  (minimum-norm particular solution of E u + Ed d = 0)
     std::vector<double> EEt((size_t)n_e * n_e);
     for (int i = 0; i < n_e; ++i)

@@ -33,9 +33,10 @@ struct HostFactor {
   std::vector<double> diagL;  // n_u, diag(L Rbar^{-1} L')
 };
 // Returns SMPC_OK or SMPC_EINVAL (rank-deficient E, W_u not positive definite).
-// reduced_basis: L in reduced form (factor_host.cpp), SMPC_ENOTSUP where that is not well
-// conditioned; else orthonormal.
-int host_factor(const smpc_network& net, const double* W_u, HostFactor& out, bool reduced_basis);
+// basis: L orthonormal, or in reduced form (factor_host.cpp), SMPC_ENOTSUP where that is not well
+// conditioned or, with BASIS_REDUCED_ANY, has entries above 4.
+enum Basis { BASIS_ORTHONORMAL, BASIS_REDUCED, BASIS_REDUCED_ANY };
+int host_factor(const smpc_network& net, const double* W_u, HostFactor& out, Basis basis);
 
 // ---------------------------------------------------------------------------
 // Tree structure after validation (host copy + device mirrors).

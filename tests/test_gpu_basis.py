@@ -75,6 +75,22 @@ def test_two_launch_form_needs_a_well_conditioned_basis(precision):
     _refused(P, H.full_size_steps(P), precision)
 
 
+@pytest.mark.parametrize("shared", [0, 1])
+def test_network_that_only_the_two_launch_form_can_run(shared):
+    """float64 packs beyond shared memory: no better conditioned choice than the reduced basis."""
+    P = synth.custom(62, 40, 150, 6, 6, synth.make_tree([3, 2], 5))
+    E = np.hstack([np.eye(6), np.random.default_rng(0).uniform(0.9, 1.0, (6, 144))])
+    P["net"] = {**P["net"], "E": E}
+    steps = H.full_size_steps(P)
+    g = H.Gpu(P, steps=steps, shared_packs=shared)
+    try:
+        g.solve(30)
+        got = g.arrays()
+    finally:
+        g.close()
+    assert errors(got, H.oracle_run(P, steps, 30)) <= BOUND[0]
+
+
 @pytest.mark.parametrize("precision", [0, 1])
 def test_shard_of_a_two_launch_factor(precision):
     """A shard runs the factor's packs, in their basis, although the factor's own solves run in

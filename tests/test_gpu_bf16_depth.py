@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 
 
 def _null_basis(E):
-    """The orthonormal null-space basis of Householder's QR of E' (signs as in LAPACK-free code)."""
+    """The orthonormal null-space basis of E, by Householder reflections of E'."""
     M, n_e = E.T.copy(), E.shape[0]
     Q = np.eye(len(M))
     for k in range(n_e):
